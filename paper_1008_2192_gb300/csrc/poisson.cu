@@ -17,7 +17,8 @@
 // (Cody-Waite reduction -mu = n ln2 + r, the Taylor polynomial of e^r to
 // degree 13 by Horner's rule, scaling by 2^n), with the rounded operations
 // spelled out so that no multiply-add is fused; the comparisons q >= e^-mu are
-// therefore those of any implementation that takes the same steps. mu <= 0 or
+// therefore those of any implementation that takes the same steps (a product
+// in float decides all but the closest of them, see poisson_kernel). mu <= 0 or
 // NaN gives 0, mu above 700 is taken as 700, and at most 4096 factors are
 // drawn, which bounds every thread's loop.
 
@@ -37,6 +38,7 @@ namespace {
 constexpr uint64_t kGamma = 0x9e3779b97f4a7c15ULL;
 constexpr double kMuMax = 700.0;
 constexpr int kQMax = 4096;
+constexpr int kPThreads = 128;
 constexpr int kFramesPerLaunch = 256;  // the frame table travels in the launch parameters
 
 struct PFrame {
@@ -82,7 +84,70 @@ __device__ __forceinline__ double exp_neg(double mu, const PLaunch& P) {
   return ldexp(p, int(n));
 }
 
-__global__ void __launch_bounds__(256) poisson_kernel(const __grid_constant__ PLaunch P) {
+// The deviate of pixel p by the defining steps in double: every product and
+// comparison as stated in the header.
+__device__ __noinline__ int deviate_exact(float mean, uint64_t key, const PLaunch& P) {
+  // q and e^-mu are non-negative doubles, which order as their bit patterns
+  const long long L = __double_as_longlong(exp_neg(fmin(double(mean), kMuMax), P));
+  uint64_t ctr = key + kGamma;  // key + (j + 1) * gamma for draw j
+  double q = uniform53(mix13(ctr));
+  int k = 0;
+  while (__double_as_longlong(q) >= L && k < kQMax) {
+    ++k;
+    ctr += kGamma;
+    q = __dmul_rn(q, uniform53(mix13(ctr)));
+  }
+  return k;
+}
+
+// hi * 2^-32 in float, rounded once: the top 23 bits and the low 9 as
+// significands of 2^23 + x, so that no conversion instruction is needed (they
+// run on the FP64 pipe here: 2 lanes per clock and SM).
+__device__ __forceinline__ float unit_float(uint32_t hi) {
+  const float a = __fsub_rn(__uint_as_float(__funnelshift_r(hi, 0x96u, 9)), 0x1p23f);  // hi >> 9, exact
+  const float b = __fmaf_rn(__uint_as_float((hi & 511u) | 0x4b000000u), 0x1p-32f, -0x1p-9f);  // exact
+  return __fmaf_rn(a, 0x1p-23f, b);
+}
+
+// The state after mix13's second product: its top 32 bits are those of the
+// output but for the lowest, since the last XOR (by z >> 31) moves the high word
+// by one at most.
+__device__ __forceinline__ uint64_t mix_head(uint64_t s) {
+  const uint64_t z = (s ^ (s >> 30)) * 0xbf58476d1ce4e5b9ULL;
+  return (z ^ (z >> 27)) * 0x94d049bb133111ebULL;
+}
+
+// The uniform of a draw in float, with a relative error below 3 * 2^-24 against
+// the 53-bit one: 2^-24 of the rounding and 2/hi of the bits left out, where
+// the 32 bits taken (hi) are at least 2^24. kSmall: the top word is less (one
+// draw in 256); then the 32 bits eight places further down, with the same
+// bound, or for a still smaller value the whole output.
+template <bool kSmall>
+__device__ __forceinline__ float uniform_approx(uint64_t z) {
+  const uint32_t hi = uint32_t(z >> 32);
+  if (!kSmall || hi >= (1u << 24)) return unit_float(hi);
+  const uint32_t w = uint32_t(z >> 24);
+  if (w >= (1u << 24)) return unit_float(w) * 0x1p-8f;
+  return __ull2float_rn((z ^ (z >> 31)) >> 11) * 0x1p-53f;
+}
+
+// The defining steps decide only where the running product falls below e^-mu,
+// so the product is first taken in float with a bound on its relative error:
+// 4 * 2^-24 per factor (the uniform above and the rounded product), and 2^-20
+// for e^-mu in float. Only where the product lands within that bound of e^-mu
+// (about 4e-5 of the pixels at mu = 24) is the pixel drawn again in double
+// (deviate_exact); the deviates are the same bits.
+// What bounds it: the ALU pipe (69 % active, issue 76 %), the shifts, XORs and
+// 64-bit products of each draw's mix, and the lanes of a warp that wait for its
+// longest draw (22.5 of 32 active). The form that multiplied in double was bound
+// by the FP64 pipe (2 lanes per clock and SM, 81 % active): 94.2 us on a 750x750
+// image of mean 24.3, against 31.1 us (with an integer-to-float conversion
+// instruction, which runs on the FP64 pipe too, 47.8 us). Two draws per step with
+// one comparison: the products fall monotonically, so the second one alone
+// tells whether to go on.
+// mu > 60, where e^-mu leaves float's range: the product is scaled up by 2^64
+// each time it falls below 2^-64, until the rest of e^-mu lies above 2^-90.
+__global__ void __launch_bounds__(kPThreads) poisson_kernel(const __grid_constant__ PLaunch P) {
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < P.total;
        t += (long long)gridDim.x * blockDim.x) {
     int lo = 0, hi = P.n - 1;  // frame of pixel t
@@ -92,20 +157,55 @@ __global__ void __launch_bounds__(256) poisson_kernel(const __grid_constant__ PL
     }
     const PFrame& f = P.f[lo];
     const long long p = t - f.pix0;
-    double mu = double(__ldg(f.in + p));
+    const float mean = __ldg(f.in + p);
     int k = 0;
-    if (mu > 0.0) {
-      mu = fmin(mu, kMuMax);
-      // q and e^-mu are non-negative doubles, which order as their bit patterns
-      const long long L = __double_as_longlong(exp_neg(mu, P));
+    if (mean > 0.f) {
+      const float mu = fminf(mean, float(kMuMax));
       const uint64_t key = stream_value(f.seed, uint64_t(p));
-      uint64_t ctr = key + kGamma;  // key + (j + 1) * gamma for draw j
-      double q = uniform53(mix13(ctr));
-      while (__double_as_longlong(q) >= L && k < kQMax) {
-        ++k;
-        ctr += kGamma;
-        q = __dmul_rn(q, uniform53(mix13(ctr)));
+      // e^-mu = 2^-e * m, m in [2^-0.5, 2^0.5]: mu * log2(e) in two floats
+      constexpr float kLog2eHi = 1.44269502f, kLog2eLo = 1.92596299e-8f;
+      const float h = __fmul_rn(mu, kLog2eHi);
+      const float l = __fmaf_rn(mu, kLog2eHi, -h) + mu * kLog2eLo;
+      const float n = rintf(h);
+      const float m = exp2f(-((h - n) + l));
+      int e = int(n);
+      const int kmax = int(2.f * mu) + 64;  // factors the error bound below allows for
+      const float delta = float(kmax + 16) * 0x1p-22f;
+      const float mhi = m * (1.f + delta), mlow = m * (1.f - delta);
+      uint64_t ctr = key;
+      float q = 1.f, q1 = 1.f, thr;
+      bool exact = false;
+      for (;;) {
+        const bool last = e <= 90;
+        thr = last ? mhi * __int_as_float((127 - e) << 23) : 0x1p-64f;
+        if (q < thr) {  // two tiny factors in a row after a scaling
+          exact = true;
+          break;
+        }
+        for (;;) {
+          const uint64_t z1 = mix_head(ctr + kGamma);
+          ctr += 2 * kGamma;
+          const uint64_t z2 = mix_head(ctr);
+          float u1 = uniform_approx<false>(z1), u2 = uniform_approx<false>(z2);
+          if (min(uint32_t(z1 >> 32), uint32_t(z2 >> 32)) < (1u << 24)) {
+            u1 = uniform_approx<true>(z1);
+            u2 = uniform_approx<true>(z2);
+          }
+          q1 = q * u1;
+          q = q1 * u2;
+          if (q < thr || k >= kmax) break;
+          k += 2;
+        }
+        if (last || k >= kmax) break;
+        k += 2;
+        q *= 0x1p64f;
+        e -= 64;
       }
+      // the factor that crossed: the first of the pair unless q1 is still above
+      const bool first = q1 < thr;
+      const float qc = first ? q1 : q, low = mlow * __int_as_float((127 - e) << 23);
+      k += first ? 0 : 1;
+      if (exact || k >= kmax || qc >= low) k = deviate_exact(mean, key, P);
     }
     f.out[p] = float(k);
   }
@@ -132,14 +232,9 @@ void fill_constants(PLaunch& P) {
 }
 
 int launch(PLaunch& P, cudaStream_t stream) {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
-                                                cudaSuccess) {
-    cudaGetLastError();
-    return fail(CRB_ECUDA, "crb_poisson: no CUDA device");
-  }
-  const long long blocks = std::min<long long>((P.total + 255) / 256, (long long)sms * 8);
-  poisson_kernel<<<int(std::max<long long>(blocks, 1)), 256, 0, stream>>>(P);
+  // a pixel per thread: blocks that draw long are balanced by the blocks still to start
+  const long long blocks = std::min<long long>((P.total + kPThreads - 1) / kPThreads, 1 << 22);
+  poisson_kernel<<<int(std::max<long long>(blocks, 1)), kPThreads, 0, stream>>>(P);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(CRB_ECUDA, std::string("crb_poisson launch: ") + cudaGetErrorString(e));
   return CRB_OK;

@@ -46,6 +46,15 @@ def test_special_values():
     assert np.array_equal(gpu_poisson(img, 5), oracle.poisson(img, 5))
 
 
+@pytest.mark.parametrize("mean", [1.9e-5, 0.3, 62.73, 107.09, 151.45, 695.0])
+def test_float_product_edges(mean):
+    """Means across the edges of the float product: where its error bound exceeds 1 - e^-mu (1.9e-5), where
+    the product is first scaled (e^-mu = 2^-90.5 at 62.73) and once more (2^-154.5, 2^-218.5), and the cap. Enough
+    draws that some products land within the bound of e^-mu and are taken again in double."""
+    img = (mean * np.linspace(0.98, 1.02, 384 * 250)).astype(np.float32).reshape(250, 384)
+    assert np.array_equal(gpu_poisson(img, 31), oracle.poisson(img, 31))
+
+
 def test_batch_equals_single_and_many_frames():
     """Frames with their own seeds in one call (more than one launch of 256 frames) equal single calls."""
     rng = np.random.default_rng(4)
