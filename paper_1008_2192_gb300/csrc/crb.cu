@@ -18,6 +18,7 @@
 #include "crb.h"
 #include "kernels.cuh"
 #include "pipeline.cuh"
+#include "tile.cuh"
 
 namespace {
 
@@ -71,13 +72,22 @@ const std::vector<DetectShape>& detect_shapes() {
   return v;
 }
 
-// tile_shape 0 takes 64 x 32 tiles, or the single-buffered 64 x 28 tiles when
-// all of those fit in one round of resident blocks and the 64 x 32 tiles do
-// not. A tile's detection is a chain of block-wide phases whose latency, not
-// an issue or memory rate, bounds the launch, so a second round of a few tiles
-// costs nearly a whole tile latency (one 800 x 800 frame: 325 tiles of 64 x 32
-// on 152 SMs x 2 blocks; 377 tiles of 64 x 28 on 152 x 3).
+// Three blocks of this shape per SM need the largest shared-memory carveout.
 constexpr int kOneRoundShape = 5;
+
+// The row kernels (tile.cuh) by tile height.
+struct TileKernels {
+  int th;
+  void (*fn[3])(const crb::Frame*, int, crb::Params, int, int);  // iteration 1, later ones, the last replacement
+  int smem;
+};
+template <int TH>
+constexpr TileKernels make_tile() {
+  return TileKernels{TH, {crb::tile_kernel<TH, 0>, crb::tile_kernel<TH, 1>, crb::tile_kernel<TH, 2>},
+                     crb::TileLayout<TH>::bytes};
+}
+const TileKernels kTileKernels[] = {make_tile<30>(), make_tile<22>()};
+constexpr int kNumTileKernels = 2;
 
 constexpr int kRW = 64, kRH = 16;  // replacement tile
 const ReplaceFn kReplace = crb::replace_kernel<kRW, kRH>;
@@ -112,7 +122,7 @@ enum QK {
 };
 
 struct GraphKey {
-  int n, niter, shape;
+  int n, niter, shape, rows;
   bool fuse, fuse2, queue;
   int seg_from;
   long long occ_sig;  // the queue kernels' blocks per SM, packed
@@ -124,7 +134,7 @@ struct GraphKey {
   void* frames;
   void* tab;
   bool operator==(const GraphKey& o) const {
-    return n == o.n && niter == o.niter && shape == o.shape && fuse == o.fuse && fuse2 == o.fuse2 && queue == o.queue &&
+    return n == o.n && niter == o.niter && shape == o.shape && rows == o.rows && fuse == o.fuse && fuse2 == o.fuse2 && queue == o.queue &&
            seg_from == o.seg_from && occ_sig == o.occ_sig &&
            tiles == o.tiles && nblocks == o.nblocks && ncells == o.ncells && npix == o.npix &&
            rtiles == o.rtiles && bits_total == o.bits_total && ncounters == o.ncounters && dgrid == o.dgrid &&
@@ -263,6 +273,12 @@ int init_ctx(crb_ctx* c) {
     c->occ_detect_maps.push_back(occm > 0 ? occm : 1);
     c->occ_fused.push_back(occf > 0 ? occf : 1);
   }
+  for (const auto& t : kTileKernels)
+    for (auto fn : t.fn) {  // four blocks per SM need the largest shared-memory carveout
+      CRB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, t.smem));
+      CRB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                    int(cudaSharedmemCarveoutMaxShared)));
+    }
   {
     const void* fns[kQKernels] = {
         reinterpret_cast<const void*>(crb::bound_dense_kernel),      reinterpret_cast<const void*>(crb::need_kernel),
@@ -414,6 +430,7 @@ struct Plan {
   int n = 0, niter = 0, shape = 0;
   bool maps = false, fuse = false, queue = false;
   bool fuse2 = false;  // tile pipeline: iterations 2 and 3 in one launch
+  int rows = -1;       // tile pipeline: the row kernels' variant (kTileKernels), or -1 for the detect kernels
   long long tiles = 0, rtiles = 0;
   size_t bits_total = 0;  // bytes from the start of the workspace that start at zero
   int ncounters = 0;
@@ -568,6 +585,17 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
           crb::mask_kernel<<<grid(kQMask, P.nblocks), 256, 0, stream>>>(c->d_frames, P.n, P.nblocks);
         });
       timed(c, kPWork, stream, [&] { crb::queue_work_kernel<<<1, 32, 0, stream>>>(c->d_frames, P.Q, k, P.npix); });
+    }
+    CRB_CUDA(cudaGetLastError());
+    return CRB_OK;
+  }
+  if (P.rows >= 0) {  // an upload, then one launch per iteration and the last replacement
+    const TileKernels& t = kTileKernels[P.rows];
+    for (int k = 1; k <= P.niter + 1; ++k) {
+      const int mode = k == 1 ? 0 : k <= P.niter ? 1 : 2;
+      timed(c, mode == 2 ? kPTileReplace : kPTileDetect, stream, [&] {
+        t.fn[mode]<<<unsigned(P.tiles), 256, t.smem, stream>>>(c->d_frames, P.n, c->p, k, P.niter);
+      });
     }
     CRB_CUDA(cudaGetLastError());
     return CRB_OK;
@@ -816,6 +844,64 @@ const CUtensorMap* encode_tile_maps(const crb::Frame& f, const DetectShape& ds, 
   return dev;
 }
 
+// Workspace and descriptors of the row kernels: three flag planes per frame
+// (zeroed at the start of a call), then the second image buffers.
+int prepare_tile(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Plan& P) {
+  const int n = int(specs.size());
+  auto plane = [](const FrameSpec& s) { return align256(size_t(crb::tile_wps(s.w)) * 2 * size_t(s.h) * 4); };
+  size_t bits = 0, total = 0;
+  for (const auto& s : specs) bits += 3 * plane(s);
+  total = bits;
+  if (niter >= 2)
+    for (const auto& s : specs) total += align256(size_t(s.w) * size_t(s.h) * 4);
+  const int nit = niter > 0 ? niter : 1;
+  const int ncounters = (2 + crb::kWork) * nit * n;
+  int rc = ensure_ws(c, total, ncounters);
+  if (rc) return rc;
+  rc = next_desc_slot(c, n, 0);
+  if (rc) return rc;
+  const int v = 0;
+  const int th = kTileKernels[v].th;
+  char* pb = static_cast<char*>(c->ws);
+  char* pi = pb + bits;
+  long long tiles = 0;
+  for (int i = 0; i < n; ++i) {
+    const auto& s = specs[size_t(i)];
+    crb::Frame& f = c->h_frames[i];
+    f = crb::Frame{};
+    f.img = s.img;
+    f.out_clean = s.out_clean;
+    f.out_mask = s.out_mask;
+    if (niter >= 2) {
+      f.ws = reinterpret_cast<float*>(pi);
+      pi += align256(size_t(s.w) * size_t(s.h) * 4);
+    }
+    for (auto& m : f.mp) {
+      m = reinterpret_cast<uint32_t*>(pb);
+      pb += plane(s);
+    }
+    f.wps = crb::tile_wps(s.w);
+    f.counters = c->d_counters + size_t(2 + crb::kWork) * nit * i;
+    f.work = f.counters + size_t(2) * nit;
+    f.w = s.w;
+    f.h = s.h;
+    f.gain = s.gain;
+    f.rn = s.rn;
+    crb::bound_thresholds(c->p, s.gain, f.bkl, f.bkh);
+    f.tiles_x = (s.w + crb::kT2W - 1) / crb::kT2W;
+    f.tile0 = tiles;
+    tiles += (long long)f.tiles_x * ((s.h + th - 1) / th);
+  }
+  P.n = n;
+  P.niter = niter;
+  P.fuse = true;
+  P.rows = v;
+  P.tiles = tiles;
+  P.bits_total = bits;
+  P.ncounters = ncounters;
+  return CRB_OK;
+}
+
 // Lays out the workspace and writes the descriptors (host), for tile shape `shape`.
 int prepare(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool maps, int shape, Plan& P) {
   const int n = int(specs.size());
@@ -935,7 +1021,7 @@ int upload(crb_ctx* c, const Plan& P, cudaStream_t stream) {
 int launch_graph(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs, cudaStream_t stream) {
   long long occ_sig = 0;
   for (int i = 0; i < kQKernels; ++i) occ_sig = occ_sig * 31 + P.occ[i];
-  GraphKey key{P.n,      P.niter,      P.shape,      P.fuse,  P.fuse2, P.queue, P.seg_from,  occ_sig,      P.tiles,
+  GraphKey key{P.n,      P.niter,      P.shape,      P.rows,  P.fuse,  P.fuse2, P.queue, P.seg_from,  occ_sig,      P.tiles,
                P.rtiles, P.nblocks,    P.ncells,     P.npix,  P.bits_total, P.ncounters, P.dgrid, P.fgrid,
                P.rgrid,  c->ws,        c->d_counters, c->d_frames, P.queue ? c->d_tab : nullptr};
   for (auto& g : c->graphs)
@@ -1020,25 +1106,24 @@ int trial_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, cons
   return CRB_OK;
 }
 
-// The tile shape that tile_shape 0 takes for a call (see kOneRoundShape).
-int default_shape(const crb_ctx* c, const std::vector<FrameSpec>& specs) {
-  const auto& v = detect_shapes();
-  auto tiles = [&](const DetectShape& d) {
-    long long t = 0;
-    for (const auto& s : specs) t += (long long)((s.w + d.tw - 1) / d.tw) * ((s.h + d.th - 1) / d.th);
-    return t;
-  };
-  auto slots = [&](int i) {
-    return (long long)c->num_sms * std::min(c->occ_detect[size_t(i)], c->occ_fused[size_t(i)]);
-  };
-  return (tiles(v[kOneRoundShape]) <= slots(kOneRoundShape) && tiles(v[0]) > slots(0)) ? kOneRoundShape : 0;
+// Whether a tile-pipeline call takes the row kernels (tile.cuh): tile_shape 0
+// without map export, a given mask or the options that ask for other launches.
+// The tile count must fit a grid.
+bool takes_rows(const crb_ctx* c, const std::vector<FrameSpec>& specs, bool maps) {
+  if (maps || c->opt.no_fusion || c->opt.fuse2 || c->opt.tile_shape != 0) return false;
+  long long tiles = 0;
+  for (const auto& s : specs) {
+    if (s.mprev) return false;
+    tiles += (long long)((s.w + crb::kT2W - 1) / crb::kT2W) * ((s.h + 13) / 14);
+  }
+  return tiles < (1LL << 31);
 }
 
-// Times one tile-pipeline clean (with the shape tile_shape 0 takes when that is
-// the option, else 64 x 32), synchronising `stream`.
+// Times one tile-pipeline clean (with the kernels tile_shape 0 takes when that
+// is the option, else 64 x 32 tiles), synchronising `stream`.
 int trial_tile(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, cudaStream_t stream, float* ms) {
   Plan P;
-  int rc = prepare(c, specs, niter, false, c->opt.tile_shape == 0 ? default_shape(c, specs) : 0, P);
+  int rc = takes_rows(c, specs, false) ? prepare_tile(c, specs, niter, P) : prepare(c, specs, niter, false, 0, P);
   if (rc == CRB_OK) rc = upload(c, P, stream);
   if (rc) return rc;
   cudaEvent_t a = take_event(c), b = take_event(c);
@@ -1054,7 +1139,7 @@ int trial_tile(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, cudaS
 }
 
 // Calls below this many pixels also try the tile pipeline.
-constexpr long long kTuneTilePixels = 1LL << 25;
+constexpr long long kTuneTilePixels = 10000000;
 
 // Tunes the queue pipeline for specs: (1) four occupancy levels (all, 3/4, 1/2,
 // 1/4 of each kernel's largest blocks per SM), each kernel keeping the level at
@@ -1192,9 +1277,10 @@ int run(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool maps, c
     }
   }
   if (shape < 0) shape = 0;
-  if (shape == 0 && c->opt.tile_shape == 0 && !maps && !queue) shape = default_shape(c, specs);
   Plan P;
-  int rc = queue ? prepare_queue(c, specs, niter, P) : prepare(c, specs, niter, maps, shape, P);
+  int rc = queue ? prepare_queue(c, specs, niter, P)
+                 : takes_rows(c, specs, maps) ? prepare_tile(c, specs, niter, P)
+                                              : prepare(c, specs, niter, maps, shape, P);
   if (rc) return rc;
   if (queue && tuned) {
     std::copy(tuned->occ, tuned->occ + kQKernels, P.occ);

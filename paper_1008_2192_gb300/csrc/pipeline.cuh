@@ -152,61 +152,6 @@ __device__ __forceinline__ void group_append(uint32_t g, uint32_t* q, unsigned i
 // four word columns, two rows per step, keeping the rows of its columns (and of
 // the halo columns, held by lanes 0-3) in registers.
 //
-// Sliding column medians: the windows of rows y and y+1 share the four values
-// of rows y-1..y+2. With c1 <= c2 the two middle values of those four, the
-// median of the four and one more value e is min(max(e, c1), c2).
-
-__device__ __forceinline__ float clamp_med(float e, float c1, float c2) { return fminf(fmaxf(e, c1), c2); }
-
-// Thresholds of the bound test of a frame: S+ = L+ / (2 N-) with N- from the
-// floored lower bound mlow of m5, so S+ > t is L+^2 > 4 t^2 / gain^2 * (gain *
-// max(mlow, 0) + rn^2). kh uses t = sigclip (hot), kl t = min(sigclip,
-// sigfrac*sigclip) (act); the factor 0.9999 keeps the test conservative
-// against the roundings of both sides. Computed once per frame on the host,
-// so the dense pass and the re-test compare against the same values.
-__host__ __device__ inline void bound_thresholds(const Params& p, float gain, float& kl, float& kh) {
-  const float sigclip = p.sigclip, tlow = fminf(p.sigfrac * p.sigclip, sigclip), g2 = gain * gain;
-  kh = 4.f * sigclip * sigclip * 0.9999f / g2;
-  kl = 4.f * tlow * tlow * 0.9999f / g2;
-}
-
-// The two bound tests of one pixel from its L+ and the smallest of its five
-// column medians, with every rounding spelled out: the dense pass and the
-// re-test share it, so a pixel re-tested with an unchanged window keeps its
-// bits exactly.
-__device__ __forceinline__ void bound_test(float lp, float mlow, float gain, float rn2, float kl, float kh, bool& act,
-                                           bool& hot) {
-  const float den = __fmaf_rn(gain, mlow > 0.f ? mlow : 0.f, rn2);
-  const float lhs = __fmul_rn(lp, lp);
-  act = lhs > __fmul_rn(kl, den);
-  hot = lhs > __fmul_rn(kh, den);
-}
-
-// Sliding column-median state of one column: rows r-2 .. r+1 of the current step.
-struct Col4 {
-  float a, b, c, d;
-};
-
-// Advances a column by the two rows (e, g) below it: the medians of the five
-// rows around the first and the second row of the step.
-__device__ __forceinline__ void col_step(Col4& s, float e, float g, float& m0, float& m1) {
-  const float l1 = fminf(s.b, s.c), h1 = fmaxf(s.b, s.c), l2 = fminf(s.d, e), h2 = fmaxf(s.d, e);
-  const float u = fmaxf(l1, l2), v = fminf(h1, h2);
-  const float c1 = fminf(u, v), c2 = fmaxf(u, v);
-  m0 = clamp_med(s.a, c1, c2);
-  m1 = clamp_med(g, c1, c2);
-}
-
-// The three values sorted: lo <= mi <= hi.
-__device__ __forceinline__ void sort3(float a, float b, float c, float& lo, float& mi, float& hi) {
-  const float s0 = fminf(a, b), s1 = fmaxf(a, b);
-  hi = fmaxf(s1, c);
-  const float t = fminf(s1, c);
-  lo = fminf(s0, t);
-  mi = fmaxf(s0, t);
-}
-__device__ __forceinline__ float med3f(float a, float b, float c) { return fmaxf(fminf(a, b), fminf(fmaxf(a, b), c)); }
-
 // hot/act/lpz bits of the NP word columns wc .. wc+NP-1 (wc a multiple of NP),
 // rows [y0, y1), of frame f (whole warp), NP pixels per lane (NP = 4 or 8):
 // lane l holds x0+NP*l .. x0+NP*l+NP-1 (16-byte loads per row when the row

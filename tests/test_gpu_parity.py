@@ -423,3 +423,22 @@ def test_two_iteration_fusion(niter):
     for a, o, m in zip(imgs, outs, masks):
         r = oracle.clean(a, params_of({}), niter, precision="f32")
         assert np.array_equal(host(m), r.mask) and np.array_equal(host(o), r.clean), a.shape
+
+
+@pytest.mark.parametrize("w,h", [(47, 29), (48, 30), (49, 31), (56, 38), (95, 60), (97, 61), (145, 22), (8, 90), (257, 91)])
+@pytest.mark.parametrize("pset", [dict(), dict(sigclip=1.2, sigfrac=0.3, objlim=0.05), dict(sigclip=5.0, objlim=500.0)],
+                         ids=["default", "dense-flags", "floored-objlim"])
+def test_row_tiles_edges(w, h, pset):
+    """The tile pipeline's row kernels at the edges of their 48-px tiles, of the flag planes' 64-px words and
+    of the frame: masks, images and counters equal the FP32 oracle's. dense-flags: fully flagged windows and
+    many new flags in every iteration; floored-objlim: S'/objlim around 0.01, where the objlim test is not
+    decided by counting."""
+    img = scene(w, h, seed=3 * w + h)
+    img[h // 2, :] += np.float32(4000.0)  # hits across every tile edge of a row and a column
+    img[:, w // 2] += np.float32(1500.0)
+    for niter in (1, 2, 5):
+        c = Cleaner(niter=niter, pipeline="tile", **pset)
+        out, mask = gpu_clean(c, img)
+        r32 = oracle.clean(img, params_of(pset), niter, precision="f32")
+        assert np.array_equal(mask, r32.mask) and np.array_equal(out, r32.clean), niter
+        assert c.last_counts() == list(zip(r32.n_new, r32.n_none_left)), niter
