@@ -40,6 +40,36 @@ def test_rects_equal_whole_frame(w, h, n, cols, niter):
     assert torch.equal(mask, ref_mask) and torch.equal(out, ref_out)
 
 
+@pytest.mark.parametrize("w,h,n", [(701, 403, 70), (97, 300, 65), (64, 33, 1)])
+def test_many_rects_in_one_call(w, h, n):
+    """More rectangles than one copy launch carries, widths off every alignment: equal to the whole frame."""
+    img = torch.from_numpy(synth.frame(w, h, seed=w)).cuda()
+    c = Cleaner(niter=2)
+    ref_out, ref_mask = c.clean(img)
+    out, mask = c.clean_rects(img, partition.plan(w, h, n, 16)[2])
+    c.sync()
+    assert torch.equal(mask, ref_mask) and torch.equal(out, ref_out)
+
+
+def test_overlapping_interiors_keep_their_order():
+    """Interiors that overlap, with too little context for equal results: each pixel is the last rectangle's, as
+    one call per rectangle leaves it."""
+    img = torch.from_numpy(synth.frame(300, 200, seed=4, ncr=900)).cuda()
+    R = partition.Rect
+    rects = [R(0, 0, 200, 200, 0, 0, 200, 200), R(100, 0, 200, 120, 100, 0, 200, 120),
+             R(150, 50, 100, 100, 150, 50, 100, 100), R(0, 150, 300, 50, 0, 150, 300, 50)]
+    c = Cleaner(niter=3)
+    out, mask = c.clean_rects(img, rects)
+    ref_out, ref_mask = torch.empty_like(out), torch.empty_like(mask)
+    for r in rects:
+        c.clean_rects_into(img, [r], ref_out, ref_mask)
+    c.sync()
+    done = torch.zeros_like(mask, dtype=torch.bool)
+    for r in rects:
+        done[r.interior()] = True
+    assert torch.equal(mask[done], ref_mask[done]) and torch.equal(out[done], ref_out[done])
+
+
 def test_mosaic_in_four_quadrants():
     """The 16384x16384 mosaic (1 GiB) as the paper's 2x2 segmentation with a 32-pixel context."""
     rec = workloads.mosaic_16384()
