@@ -173,7 +173,7 @@ struct crb_ctx {
   size_t ws_bytes = 0;
   // Descriptors (and the queue pipeline's frame table: frame of each
   // 2^kTabShift pixels) are staged in a ring of kDescSlots page-locked host
-  // buffers, so that a call waits only for the upload of the call kDescSlots
+  // buffers, so that a call waits only for the end of the call kDescSlots
   // back before refilling one, and uploaded into one device buffer of the
   // context: calls on a context are ordered (each starts after the previous
   // one's completion event), so no kernel still reads the device copy when the
@@ -186,7 +186,7 @@ struct crb_ctx {
     CUtensorMap* h_maps = nullptr;  // tile pipeline: 3 per frame (capacity 3 * frames_cap)
     int frames_cap = 0;
     size_t tab_cap = 0;
-    cudaEvent_t upload_ev = nullptr;
+    cudaEvent_t ev = nullptr;  // the end of the last call that used the slot
   } slot[kDescSlots];
   int cur = 0;
   crb::Frame* d_frames = nullptr;  // device descriptors (capacity d_frames_cap)
@@ -206,7 +206,8 @@ struct crb_ctx {
   int last_launches = 0;  // kernels the work of the last call launches
   int mprev_frames = 0;   // crb_iterate: frames given an explicit M_{k-1}
   int last_nframes = 0;
-  cudaEvent_t upload_ev = nullptr, done_ev = nullptr;  // upload_ev: the current slot's
+  // done_ev: the end of the last call, the event of its slot (not owned)
+  cudaEvent_t done_ev = nullptr;
   bool any_call = false;
   int latched = CRB_OK;
 
@@ -307,9 +308,8 @@ int init_ctx(crb_ctx* c) {
   CRB_CUDA(cudaFuncSetAttribute(kReplace, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kReplaceSmem)));
   CRB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c->occ_replace, kReplace, crb::kThreads, kReplaceSmem));
   if (c->occ_replace < 1) c->occ_replace = 1;
-  for (auto& sl : c->slot) CRB_CUDA(cudaEventCreateWithFlags(&sl.upload_ev, cudaEventDisableTiming));
-  c->upload_ev = c->slot[0].upload_ev;
-  CRB_CUDA(cudaEventCreateWithFlags(&c->done_ev, cudaEventDisableTiming));
+  for (auto& sl : c->slot) CRB_CUDA(cudaEventCreateWithFlags(&sl.ev, cudaEventDisableTiming));
+  c->done_ev = c->slot[0].ev;
   CRB_CUDA(cudaMalloc(&c->d_status, 256));
   CRB_CUDA(cudaMemset(c->d_status, 0, 256));
   return CRB_OK;
@@ -347,7 +347,7 @@ bool overlaps(const void* a, size_t na, const void* b, size_t nb) {
 }
 
 // Moves to the next descriptor slot, with room for n frames and tab_entries
-// table entries, once the slot's previous upload has run; sets the views and
+// table entries, once the slot's previous call has ended; sets the views and
 // grows the device copies if needed.
 int next_desc_slot(crb_ctx* c, int n, size_t tab_entries) {
   c->cur = (c->cur + 1) % kDescSlots;
@@ -392,12 +392,11 @@ int next_desc_slot(crb_ctx* c, int n, size_t tab_entries) {
       c->d_tab_cap = tab_entries;
     }
   }
-  CRB_CUDA(cudaEventSynchronize(S.upload_ev));  // the staging buffers are free again
+  CRB_CUDA(cudaEventSynchronize(S.ev));  // the staging buffers are free again
   c->h_frames = S.h_frames;
   c->h_maps = S.h_maps;
   c->maps_n = 0;
   c->h_tab = S.h_tab;
-  c->upload_ev = S.upload_ev;
   return CRB_OK;
 }
 
@@ -446,9 +445,36 @@ struct Plan {
   int seg_from = crb::kSegFrom;  // queue pipeline: first iteration of the segment-list forms
 };
 
+// Launches fn so that it may start before the kernel ahead of it in the stream
+// has ended (it waits for it in crb::pdl_wait).
+template <typename... P, typename... A>
+void launch_pdl(void (*fn)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, fn, P(args)...);
+}
+
+// The end of the work of a call on `stream`: the descriptor slot and the next
+// call wait for it.
+int finish(crb_ctx* c, cudaStream_t stream) {
+  c->done_ev = c->slot[c->cur].ev;
+  CRB_CUDA(cudaEventRecord(c->done_ev, stream));
+  c->any_call = true;
+  return CRB_OK;
+}
+
 int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs, cudaStream_t stream) {
   const DetectShape& ds = detect_shapes()[size_t(P.shape)];
-  CRB_CUDA(cudaMemsetAsync(c->d_counters, 0, sizeof(unsigned long long) * size_t(P.ncounters), stream));
+  if (P.rows < 0)  // else the upload zeroed them
+    CRB_CUDA(cudaMemsetAsync(c->d_counters, 0, sizeof(unsigned long long) * size_t(P.ncounters), stream));
   if (P.niter == 0) {
     for (const auto& s : specs) {
       CRB_CUDA(cudaMemcpyAsync(s.out_clean, s.img, size_t(s.w) * s.h * 4, cudaMemcpyDeviceToDevice, stream));
@@ -456,7 +482,7 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
     }
     return CRB_OK;
   }
-  CRB_CUDA(cudaMemsetAsync(c->ws, 0, P.bits_total, stream));
+  if (P.rows < 0) CRB_CUDA(cudaMemsetAsync(c->ws, 0, P.bits_total, stream));
   if (P.queue) {
     // the image buffer starts as I0 (copied by the first bound pass): every
     // replacement then writes only its flagged pixels
@@ -594,7 +620,7 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
     for (int k = 1; k <= P.niter + 1; ++k) {
       const int mode = k == 1 ? 0 : k <= P.niter ? 1 : 2;
       timed(c, mode == 2 ? kPTileReplace : kPTileDetect, stream, [&] {
-        t.fn[mode]<<<unsigned(P.tiles), 256, t.smem, stream>>>(c->d_frames, P.n, c->p, k, P.niter);
+        launch_pdl(t.fn[mode], unsigned(P.tiles), 256, t.smem, stream, c->d_frames, P.n, c->p, k, P.niter);
       });
     }
     CRB_CUDA(cudaGetLastError());
@@ -978,13 +1004,20 @@ int prepare(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool map
   return CRB_OK;
 }
 
-// Copies n0 4-byte words src0 -> dst0 and n1 words src1 -> dst1 from
+// Zeroes nz 16-byte vectors at z and nc 8-byte words at zc (the row kernels'
+// flag planes and the counters: one launch in the place of two memsets), and
+// copies n0 4-byte words src0 -> dst0 and n1 words src1 -> dst1 from
 // page-locked host memory, read directly by the kernel: the descriptors reach
 // the device without a copy engine, so they do not queue behind large
 // transfers of other streams (crb_clean_batch_host), and one launch carries
 // them all.
 __global__ void upload_kernel(uint32_t* __restrict__ dst0, const uint32_t* __restrict__ src0, size_t n0,
-                              uint32_t* __restrict__ dst1, const uint32_t* __restrict__ src1, size_t n1) {
+                              uint32_t* __restrict__ dst1, const uint32_t* __restrict__ src1, size_t n1,
+                              uint4* __restrict__ z, size_t nz, unsigned long long* __restrict__ zc, size_t nc) {
+  crb::pdl_launch();
+  const size_t t = size_t(blockIdx.x) * blockDim.x + threadIdx.x, step = size_t(gridDim.x) * blockDim.x;
+  for (size_t i = t; i < nz; i += step) z[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (size_t i = t; i < nc; i += step) zc[i] = 0ull;
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n0 + n1; i += size_t(gridDim.x) * blockDim.x)
     if (i < n0)
       dst0[i] = src0[i];
@@ -1065,10 +1098,13 @@ int upload(crb_ctx* c, const Plan& P, cudaStream_t stream) {
   uint32_t* d1 = P.queue ? c->d_tab : reinterpret_cast<uint32_t*>(c->d_maps);
   const uint32_t* h1 = P.queue ? c->h_tab : reinterpret_cast<const uint32_t*>(c->h_maps);
   const size_t n1 = P.queue ? c->tab_n : sizeof(CUtensorMap) * c->maps_n / 4;
-  upload_kernel<<<int(std::min<size_t>((nf + n1 + 255) / 256, 64)), 256, 0, stream>>>(
-      reinterpret_cast<uint32_t*>(c->d_frames), reinterpret_cast<const uint32_t*>(c->h_frames), nf, d1, h1, n1);
+  const size_t nz = P.rows >= 0 && P.niter > 0 ? P.bits_total / 16 : 0, nc = P.rows >= 0 ? size_t(P.ncounters) : 0;
+  const size_t blocks = std::max(std::min<size_t>((nf + n1 + 255) / 256, 64),
+                                 std::min<size_t>((nz + 1023) / 1024, size_t(c->num_sms) * 4));
+  upload_kernel<<<int(blocks), 256, 0, stream>>>(reinterpret_cast<uint32_t*>(c->d_frames),
+                                                 reinterpret_cast<const uint32_t*>(c->h_frames), nf, d1, h1, n1,
+                                                 static_cast<uint4*>(c->ws), nz, c->d_counters, nc);
   CRB_CUDA(cudaGetLastError());
-  CRB_CUDA(cudaEventRecord(c->upload_ev, stream));
   c->last_niter = P.niter;
   c->last_nframes = P.n;
   // the launches of this upload and of enqueue_work for this plan (memsets and copies not counted)
@@ -1335,9 +1371,7 @@ int run(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool maps, c
       cudaEventDestroy(b);
       c->tuned.emplace_back(sig, best_shape);
       // every trial produced the same outputs; the last one stays
-      CRB_CUDA(cudaEventRecord(c->done_ev, stream));
-      c->any_call = true;
-      return CRB_OK;
+      return finish(c, stream);
     }
   }
   if (shape < 0) shape = 0;
@@ -1363,10 +1397,8 @@ int run(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool maps, c
     rc = launch_graph(c, P, specs, stream);
   else
     rc = enqueue_work(c, P, specs, stream);
-  if (rc) return rc;
-  CRB_CUDA(cudaEventRecord(c->done_ev, stream));
-  c->any_call = true;
-  return CRB_OK;
+  const int re = finish(c, stream);
+  return rc ? rc : re;
 }
 
 bool valid_params(float gain, float rn, float sigclip, float sigfrac, float objlim, int niter) {
@@ -1448,10 +1480,9 @@ void crb_destroy(crb_ctx* c) {
     if (sl.h_frames) cudaFreeHost(sl.h_frames);
     if (sl.h_maps) cudaFreeHost(sl.h_maps);
     if (sl.h_tab) cudaFreeHost(sl.h_tab);
-    if (sl.upload_ev) cudaEventDestroy(sl.upload_ev);
+    if (sl.ev) cudaEventDestroy(sl.ev);
   }
   cudaFree(c->d_counters);
-  if (c->done_ev) cudaEventDestroy(c->done_ev);
   delete c;
 }
 

@@ -315,6 +315,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, unsign
   }
   return false;
 }
+// Programmatic dependent launch: a kernel launched with the attribute may start
+// while the kernel before it in the stream still runs. pdl_wait returns once
+// that kernel has completed and its writes are visible; pdl_launch allows the next
+// kernel to start (once every block has called it or ended). Both do nothing in
+// a kernel launched without the attribute. Every kernel of a chain waits before it
+// lets the next one start, so what an earlier kernel of the chain than the
+// previous one wrote is visible before the wait too.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // Polls of a TMA wait before it gives up (each poll suspends the thread for a
 // while in hardware; a box lands in microseconds).
 constexpr unsigned kTmaWaitPolls = 1u << 22;

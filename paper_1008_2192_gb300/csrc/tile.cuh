@@ -234,7 +234,21 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
   int* cnt = reinterpret_cast<int*>(smem + L::oCnt);  // 0 replacement, 1 S, 2 S', 3 tests, 4 full windows, 5.. work
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-  const Frame& f = frames[frame_of<false>(frames, nframes, blockIdx.x)];
+  // the bit maps and counters; then the frame's descriptor, which in the later iterations does not depend
+  // on the kernel before this one (pdl_wait)
+  for (int i = tid; i < 6 * R; i += 256) mC[i] = make_uint2(0u, 0u);
+  if (tid < 16) cnt[tid] = 0;
+  if (kMode == 0) {
+    pdl_wait();
+    pdl_launch();
+  }
+  __shared__ Frame sf;
+  {
+    const uint32_t* d = reinterpret_cast<const uint32_t*>(frames + frame_of<false>(frames, nframes, blockIdx.x));
+    for (int i = tid; i < int(sizeof(Frame) / 4); i += 256) reinterpret_cast<uint32_t*>(&sf)[i] = d[i];
+  }
+  __syncthreads();
+  const Frame& f = sf;
   const int w = f.w, h = f.h, wps = f.wps;
   TilePos T;
   {
@@ -248,6 +262,10 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
     T.edge = T.c0 > 2 || T.r0 > 2 || T.c1 < 62 || T.r1 < R - 2;
   }
   const float* src = kMode == 0 ? f.img : iter_src(f, k - 1, niter);
+  if (kMode != 0) {
+    pdl_wait();
+    pdl_launch();
+  }
 
   // the image region (mode 2: the tile and the 2 rows around it), clamped into the frame
   {
@@ -274,8 +292,6 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
     }
     cp_async_commit();
   }
-  for (int i = tid; i < 6 * R; i += 256) mC[i] = make_uint2(0u, 0u);
-  if (tid < 16) cnt[tid] = 0;
   const uint2 own = T.cols(0);
 
   if (kMode != 0) {
