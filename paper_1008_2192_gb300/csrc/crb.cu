@@ -86,8 +86,11 @@ constexpr TileKernels make_tile() {
   return TileKernels{TH, {crb::tile_kernel<TH, 0>, crb::tile_kernel<TH, 1>, crb::tile_kernel<TH, 2>},
                      crb::TileLayout<TH>::bytes};
 }
-const TileKernels kTileKernels[] = {make_tile<30>(), make_tile<22>()};
-constexpr int kNumTileKernels = 2;
+// Tiles of 30 rows: the time of a call by height, 14 / 22 / 30 / 38 rows: 70 / 61 / 60 / 61 us on 800 x 800,
+// 299 / 238 / 213 / 219 us on 2048 x 2048 (fewer rows: more of them recomputed around the tile; 38: three
+// blocks per SM). Tiles of 14 rows where they number at most one per SM: a block's latency is all there is,
+// and fewer rows per warp shorten it (137 x 137: 41 / 43 / 47 / 50 us).
+const TileKernels kTileKernels[] = {make_tile<30>(), make_tile<14>()};
 
 constexpr int kRW = 64, kRH = 16;  // replacement tile
 const ReplaceFn kReplace = crb::replace_kernel<kRW, kRH>;
@@ -886,7 +889,12 @@ int prepare_tile(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pla
   if (rc) return rc;
   rc = next_desc_slot(c, n, 0);
   if (rc) return rc;
-  const int v = 0;
+  auto tiles_of = [&](const FrameSpec& s, int h) {
+    return (long long)((s.w + crb::kT2W - 1) / crb::kT2W) * ((s.h + h - 1) / h);
+  };
+  long long small = 0;
+  for (const auto& s : specs) small += tiles_of(s, kTileKernels[1].th);
+  const int v = small <= c->num_sms ? 1 : 0;
   const int th = kTileKernels[v].th;
   char* pb = static_cast<char*>(c->ws);
   char* pi = pb + bits;
@@ -916,7 +924,7 @@ int prepare_tile(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pla
     crb::bound_thresholds(c->p, s.gain, f.bkl, f.bkh);
     f.tiles_x = (s.w + crb::kT2W - 1) / crb::kT2W;
     f.tile0 = tiles;
-    tiles += (long long)f.tiles_x * ((s.h + th - 1) / th);
+    tiles += tiles_of(s, th);
   }
   P.n = n;
   P.niter = niter;

@@ -56,8 +56,8 @@ struct TileLayout {
   static constexpr int oN = oS + RS * kT2P;
   static constexpr int oM3 = oN + R2 * kT2P;
   static constexpr int nF = oM3 + RB * kT2P;
-  static constexpr int kListR = (TH + 12) * 60;  // flagged pixels to replace: values over the S map
-  static_assert(kListR <= RS * kT2P, "replacement values fit in the S map");
+  static constexpr int kListR = (TH + 12) * 60;  // flagged pixels to replace: values over the S and N maps
+  static_assert(kListR <= (RS + R2) * kT2P, "replacement values fit in the S and N maps");
   static constexpr int kListS = imax(RS * 28, (kListR + 1) / 2 * 2);  // pairs of S; or the replacement list
   static constexpr int kListP = R2 * 26;  // pairs of S'
   static_assert(R2 * 52 <= kListS, "the tests take the place of the pairs of S");
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
   float* sS = reinterpret_cast<float*>(smem) + L::oS - 4 * kT2P;  // rows 4 .. R-5
   float* sN = reinterpret_cast<float*>(smem) + L::oN - 6 * kT2P;  // rows 6 .. R-7; the test scale where tested
   float* sM3 = reinterpret_cast<float*>(smem) + L::oM3 - 3 * kT2P;  // rows 3 .. R-4
-  float* val = reinterpret_cast<float*>(smem) + L::oS;            // replacement values (before S)
+  float* val = reinterpret_cast<float*>(smem) + L::oS;            // replacement values (before S and N)
   uint2* mM = reinterpret_cast<uint2*>(smem + L::oMask);          // M_{k-1}
   uint2* mF = mM + R;                                             // new in M_{k-1}; then the pixels near a change
   uint2* mC = mF + R;                                             // changed pixels
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
   const float* src = kMode == 0 ? f.img : iter_src(f, k - 1, niter);
   if (kMode != 0) {
     pdl_wait();
-    pdl_launch();
+    if (kMode == 1) pdl_launch();  // the last kernel's results are the caller's: nothing starts before they are whole
   }
 
   // the image region (mode 2: the tile and the 2 rows around it), clamped into the frame
