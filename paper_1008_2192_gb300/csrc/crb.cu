@@ -126,7 +126,7 @@ enum QK {
 
 struct GraphKey {
   int n, niter, shape, rows;
-  bool fuse, fuse2, queue;
+  bool fuse, fuse2, queue, pdl, row_form;
   int seg_from;
   long long occ_sig;  // the queue kernels' blocks per SM, packed
   long long tiles, rtiles, nblocks, ncells, npix;
@@ -137,7 +137,7 @@ struct GraphKey {
   void* frames;
   void* tab;
   bool operator==(const GraphKey& o) const {
-    return n == o.n && niter == o.niter && shape == o.shape && rows == o.rows && fuse == o.fuse && fuse2 == o.fuse2 && queue == o.queue &&
+    return n == o.n && niter == o.niter && shape == o.shape && rows == o.rows && fuse == o.fuse && fuse2 == o.fuse2 && queue == o.queue && pdl == o.pdl && row_form == o.row_form &&
            seg_from == o.seg_from && occ_sig == o.occ_sig &&
            tiles == o.tiles && nblocks == o.nblocks && ncells == o.ncells && npix == o.npix &&
            rtiles == o.rtiles && bits_total == o.bits_total && ncounters == o.ncounters && dgrid == o.dgrid &&
@@ -430,7 +430,9 @@ int ensure_ws(crb_ctx* c, size_t bytes, int ncounters) {
 // and kernel launches. Issued on `stream` directly, or into a CUDA graph.
 struct Plan {
   int n = 0, niter = 0, shape = 0;
-  bool maps = false, fuse = false, queue = false;
+  bool maps = false, fuse = false, queue = false, pdl = false;
+  bool row_form = false;  // the row forms of the bit-plane kernels
+  bool zeroed = false;  // the upload zeroes the planes and counters (else two memsets do)
   bool fuse2 = false;  // tile pipeline: iterations 2 and 3 in one launch
   int rows = -1;       // tile pipeline: the row kernels' variant (kTileKernels), or -1 for the detect kernels
   long long tiles = 0, rtiles = 0;
@@ -476,7 +478,7 @@ int finish(crb_ctx* c, cudaStream_t stream) {
 
 int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs, cudaStream_t stream) {
   const DetectShape& ds = detect_shapes()[size_t(P.shape)];
-  if (P.rows < 0)  // else the upload zeroed them
+  if (!P.zeroed)
     CRB_CUDA(cudaMemsetAsync(c->d_counters, 0, sizeof(unsigned long long) * size_t(P.ncounters), stream));
   if (P.niter == 0) {
     for (const auto& s : specs) {
@@ -485,7 +487,7 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
     }
     return CRB_OK;
   }
-  if (P.rows < 0) CRB_CUDA(cudaMemsetAsync(c->ws, 0, P.bits_total, stream));
+  if (!P.zeroed) CRB_CUDA(cudaMemsetAsync(c->ws, 0, P.bits_total, stream));
   if (P.queue) {
     // the image buffer starts as I0 (copied by the first bound pass): every
     // replacement then writes only its flagged pixels
@@ -505,115 +507,142 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
       cudaEventRecord(b, stream);
       c->tune_ev.push_back({kernel, {a, b}});
     };
+    // Below kPdlPixels every kernel may start while the one ahead of it ends.
+    auto go = [&](auto fn, auto grid, int block, auto... args) {
+      if (P.pdl)
+        launch_pdl(fn, unsigned(grid), unsigned(block), 0, stream, args...);
+      else
+        fn<<<unsigned(grid), unsigned(block), 0, stream>>>(args...);
+    };
     const size_t cells_bytes = size_t(P.ncells) * 4;
     for (int k = 1; k <= P.niter; ++k) {
       uint32_t* cls = P.cells[k & 1];
       uint32_t* cls_next = (k < P.niter) ? P.cells[(k + 1) & 1] : nullptr;
       const uint32_t* kcls = (k == 1) ? nullptr : cls;
+      // the classes and changed pixels of iteration k+1 start at zero (those of iteration k-1 were read by then)
+      const bool clear = k >= 3 && cls_next;
       const long long ucol = (P.nunits + crb::kColWarps - 1) / crb::kColWarps;
       const int gcol = grid(kQNeed, ucol);
       const int gcolm = grid(kQM3need, ucol), gcol1m = grid(kQM3needAll, ucol);
       const bool seg = k >= P.seg_from;  // the column kernels walk the listed segments only
       const int tcol = crb::kColWarps * 32;
+      const long long grow = std::min<long long>(P.nunits, 64LL * c->num_sms), gseg = 8LL * c->num_sms;  // row forms
       timed(c, kPBound, stream, [&] {
         if (k == 1) {
           tq(kQBound, [&] {
-            crb::bound_dense_kernel<<<grid(kQBound, P.nblocks), crb::kBoundThreads, 0, stream>>>(c->d_frames, P.n,
+            go(crb::bound_dense_kernel, grid(kQBound, P.nblocks), crb::kBoundThreads, c->d_frames, P.n,
                                                                                          P.nblocks, c->p);
           });
         } else {  // the pixels within 2 px of a change, re-tested one by one
           if (seg) {
             tq(kQSegList, [&] {
-              crb::seg_list_kernel<<<grid(kQSegList, (P.nunits + 7) / 8), crb::kThreads, 0, stream>>>(
+              go(crb::seg_list_kernel, grid(kQSegList, (P.nunits + 7) / 8), crb::kThreads, 
                   c->d_frames, P.n, P.nunits, P.Q, cls);
             });
             tq(kQD2Seg, [&] {
-              crb::d2_seg_kernel<<<gq * P.occ[kQD2Seg], tcol, 0, stream>>>(c->d_frames, P.n, P.Q, k);
+              if (P.row_form)
+                go(crb::d2_segrow_kernel, gseg, 256, c->d_frames, P.n, P.Q, k);
+              else
+                go(crb::d2_seg_kernel, gq * P.occ[kQD2Seg], tcol, c->d_frames, P.n, P.Q, k);
             });
           } else {
             tq(kQD2, [&] {
-              crb::d2_kernel<<<grid(kQD2, ucol), tcol, 0, stream>>>(c->d_frames, P.n, P.nunits, P.Q, k);
+              if (P.row_form)
+                go(crb::d2_row_kernel, grow, 256, c->d_frames, P.n, P.nunits, P.Q, k);
+              else
+                go(crb::d2_kernel, grid(kQD2, ucol), tcol, c->d_frames, P.n, P.nunits, P.Q, k);
             });
           }
           tq(kQBoundSparse, [&] {
-            crb::bound_sparse_kernel<<<gq * P.occ[kQBoundSparse], 256, 0, stream>>>(c->d_frames, P.n, P.Q, c->p);
+            go(crb::bound_sparse_kernel, gq * P.occ[kQBoundSparse], 256, c->d_frames, P.n, P.Q, c->p);
           });
         }
       });
       timed(c, kPNeed, stream, [&] {
         if (seg)
           tq(kQNeedSeg, [&] {
-            crb::need_seg_kernel<<<gq * P.occ[kQNeedSeg], tcol, 0, stream>>>(c->d_frames, P.n, P.Q, cls);
+            if (P.row_form)
+              go(crb::need_segrow_kernel, gseg, 256, c->d_frames, P.n, P.Q, cls);
+            else
+              go(crb::need_seg_kernel, gq * P.occ[kQNeedSeg], tcol, c->d_frames, P.n, P.Q, cls);
           });
         else
           tq(kQNeed, [&] {
-            crb::need_kernel<<<gcol, tcol, 0, stream>>>(c->d_frames, P.n, P.nunits, P.Q, kcls);
+            if (P.row_form)
+              go(crb::need_row_kernel, grow, 256, c->d_frames, P.n, P.nunits, P.Q, kcls);
+            else
+              go(crb::need_kernel, gcol, tcol, c->d_frames, P.n, P.nunits, P.Q, kcls);
           });
       });
       timed(c, kPS, stream, [&] {
-        tq(kQS, [&] { crb::s_kernel<<<gq * P.occ[kQS], 256, 0, stream>>>(c->d_frames, P.n, P.Q, k); });
+        tq(kQS, [&] { go(crb::s_kernel, gq * P.occ[kQS], 256, c->d_frames, P.n, P.Q, k); });
       });
       timed(c, kPSp, stream, [&] {
-        tq(kQSp, [&] { crb::sp_kernel<<<gq * P.occ[kQSp], 256, 0, stream>>>(c->d_frames, P.n, P.Q, c->p, k); });
+        tq(kQSp, [&] { go(crb::sp_kernel, gq * P.occ[kQSp], 256, c->d_frames, P.n, P.Q, c->p, k); });
       });
       timed(c, kPM3need, stream, [&] {
         if (seg)
           tq(kQM3needSeg, [&] {
-            crb::m3need_seg_kernel<<<gq * P.occ[kQM3needSeg], tcol, 0, stream>>>(c->d_frames, P.n, P.Q, cls);
+            if (P.row_form)
+              go(crb::m3need_segrow_kernel, gseg, 256, c->d_frames, P.n, P.Q, cls);
+            else
+              go(crb::m3need_seg_kernel, gq * P.occ[kQM3needSeg], tcol, c->d_frames, P.n, P.Q, cls);
           });
         else if (k == 1)
           tq(kQM3needAll, [&] {
-            crb::m3need_kernel<true><<<gcol1m, tcol, 0, stream>>>(c->d_frames, P.n, P.nunits, P.Q, nullptr);
+            go(crb::m3need_kernel<true>, gcol1m, tcol, c->d_frames, P.n, P.nunits, P.Q, nullptr);
           });
         else
           tq(kQM3need, [&] {
-            crb::m3need_kernel<false><<<gcolm, tcol, 0, stream>>>(c->d_frames, P.n, P.nunits, P.Q, kcls);
+            if (P.row_form)
+              go(crb::m3need_row_kernel, grow, 256, c->d_frames, P.n, P.nunits, P.Q, kcls);
+            else
+              go(crb::m3need_kernel<false>, gcolm, tcol, c->d_frames, P.n, P.nunits, P.Q, kcls);
           });
       });
       timed(c, kPM3, stream, [&] {
-        tq(kQM3, [&] { crb::m3_kernel<<<gq * P.occ[kQM3], 256, 0, stream>>>(c->d_frames, P.n, P.Q, k); });
+        tq(kQM3, [&] { go(crb::m3_kernel, gq * P.occ[kQM3], 256, c->d_frames, P.n, P.Q, k); });
       });
       timed(c, kPCand, stream, [&] {
         tq(kQCand, [&] {
-          crb::cand_test_kernel<<<gq * P.occ[kQCand], 256, 0, stream>>>(c->d_frames, P.n, P.Q, c->p, k);
+          go(crb::cand_test_kernel, gq * P.occ[kQCand], 256, c->d_frames, P.n, P.Q, c->p, k);
         });
         tq(kQCandFull, [&] {
-          crb::cand_full_kernel<<<gq * P.occ[kQCandFull], 256, 0, stream>>>(c->d_frames, P.n, P.Q, c->p, k);
+          go(crb::cand_full_kernel, gq * P.occ[kQCandFull], 256, c->d_frames, P.n, P.Q, c->p, k, reinterpret_cast<uint4*>(cls_next), clear ? (cells_bytes + 15) / 16 : 0,
+             reinterpret_cast<uint4*>(P.chg[(k + 1) & 1]), clear ? P.chg_bytes / 16 : 0);
         });
       });
       timed(c, kPGrow, stream, [&] {
         if (k == 1)  // both growths from the bit planes; flags counted and queued for the replacement
           tq(kQGrowFirst, [&] {
-            crb::grow_first_kernel<<<grid(kQGrowFirst, ucol), tcol, 0, stream>>>(c->d_frames, P.n, P.nunits, P.Q);
+            if (P.row_form)
+              go(crb::grow_first_row_kernel, grow, 256, c->d_frames, P.n, P.nunits, P.Q);
+            else
+              go(crb::grow_first_kernel, grid(kQGrowFirst, ucol), tcol, c->d_frames, P.n, P.nunits, P.Q);
           });
         else
           tq(kQGrow, [&] {
-            crb::grow_kernel<<<gq * P.occ[kQGrow], 256, 0, stream>>>(c->d_frames, P.n, P.Q, c->p, k);
+            go(crb::grow_kernel, gq * P.occ[kQGrow], 256, c->d_frames, P.n, P.Q, c->p, k);
           });
       });
-      // the classes and changed pixels of iteration k+1 start at zero (those of iteration k-1 were read by now)
-      if (k >= 3 && cls_next) {
-        CRB_CUDA(cudaMemsetAsync(cls_next, 0, cells_bytes, stream));
-        CRB_CUDA(cudaMemsetAsync(P.chg[(k + 1) & 1], 0, P.chg_bytes, stream));
-      }
       timed(c, kPRep, stream, [&] {
         if (k >= 2)
-          tq(kQRq, [&] { crb::rq_kernel<<<gq * P.occ[kQRq], 256, 0, stream>>>(c->d_frames, P.n, P.Q); });
+          tq(kQRq, [&] { go(crb::rq_kernel, gq * P.occ[kQRq], 256, c->d_frames, P.n, P.Q); });
         tq(kQRepCompute, [&] {
-          crb::rep_compute_kernel<<<gq * P.occ[kQRepCompute], 256, 0, stream>>>(c->d_frames, P.n, P.Q, k,
+          go(crb::rep_compute_kernel, gq * P.occ[kQRepCompute], 256, c->d_frames, P.n, P.Q, k,
                                                                                 cls_next);
         });
         if (k >= 2)
           tq(kQRepWrite, [&] {
-            crb::rep_write_kernel<<<gq * P.occ[kQRepWrite], 256, 0, stream>>>(c->d_frames, P.n, P.Q, cls_next,
+            go(crb::rep_write_kernel, gq * P.occ[kQRepWrite], 256, c->d_frames, P.n, P.Q, cls_next,
                                                                               k + 1, 1);
           });
       });
       if (k == P.niter)
         timed(c, kPMask, stream, [&] {
-          crb::mask_kernel<<<grid(kQMask, P.nblocks), 256, 0, stream>>>(c->d_frames, P.n, P.nblocks);
+          go(crb::mask_kernel, grid(kQMask, P.nblocks), 256, c->d_frames, P.n, P.nblocks);
         });
-      timed(c, kPWork, stream, [&] { crb::queue_work_kernel<<<1, 32, 0, stream>>>(c->d_frames, P.Q, k, P.npix); });
+      timed(c, kPWork, stream, [&] { go(crb::queue_work_kernel, 1, 32, c->d_frames, P.Q, k, P.npix); });
     }
     CRB_CUDA(cudaGetLastError());
     return CRB_OK;
@@ -667,6 +696,17 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
   CRB_CUDA(cudaGetLastError());
   return CRB_OK;
 }
+
+// Calls below this many pixels, not replayed from a graph, launch the queue kernels so that each may start
+// while the one ahead ends (about 2 us of each of the 57 launches): 721 -> 615 us on 4146 x 2051, 782 -> 682
+// on 4096^2, 1517 -> 1466 on 8192^2, no gain on 16384^2. In a graph the same edges are slower than plain ones
+// (650 -> 677 us on 4096^2).
+constexpr long long kPdlPixels = 1LL << 27;
+
+// Calls below this many pixels take the row forms of the bit-plane kernels (pipeline.cuh): 522 -> 447 us on
+// 2048 x 3100, 573 -> 484 on 4146 x 2051, 685 -> 622 on 4096^2 (643 -> 581 in a graph), 986 -> 920 on 6000^2;
+// level on 8192^2 (1462, 1460), slower above (4532 -> 4844 on 16384^2).
+constexpr long long kRowFormPixels = 1LL << 26;
 
 // Queue pipeline: workspace = [queue counters | per frame: bit planes M, rq, fb |
 // cell classes x 2 | changed-pixel planes x 2] (zeroed at the start of a call)
@@ -798,6 +838,9 @@ int prepare_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pl
   P.maps = false;
   P.fuse = false;
   P.queue = true;
+  P.zeroed = npix < kPdlPixels;
+  P.row_form = npix < kRowFormPixels;
+  P.pdl = npix < kPdlPixels && !c->opt.use_graphs;
   P.rtiles = rtiles;
   P.bits_total = zero_bytes;
   P.ncounters = ncounters;
@@ -930,6 +973,7 @@ int prepare_tile(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pla
   P.niter = niter;
   P.fuse = true;
   P.rows = v;
+  P.zeroed = true;
   P.tiles = tiles;
   P.bits_total = bits;
   P.ncounters = ncounters;
@@ -1106,7 +1150,7 @@ int upload(crb_ctx* c, const Plan& P, cudaStream_t stream) {
   uint32_t* d1 = P.queue ? c->d_tab : reinterpret_cast<uint32_t*>(c->d_maps);
   const uint32_t* h1 = P.queue ? c->h_tab : reinterpret_cast<const uint32_t*>(c->h_maps);
   const size_t n1 = P.queue ? c->tab_n : sizeof(CUtensorMap) * c->maps_n / 4;
-  const size_t nz = P.rows >= 0 && P.niter > 0 ? P.bits_total / 16 : 0, nc = P.rows >= 0 ? size_t(P.ncounters) : 0;
+  const size_t nz = P.zeroed && P.niter > 0 ? P.bits_total / 16 : 0, nc = P.zeroed ? size_t(P.ncounters) : 0;
   const size_t blocks = std::max(std::min<size_t>((nf + n1 + 255) / 256, 64),
                                  std::min<size_t>((nz + 1023) / 1024, size_t(c->num_sms) * 4));
   upload_kernel<<<int(blocks), 256, 0, stream>>>(reinterpret_cast<uint32_t*>(c->d_frames),
@@ -1129,7 +1173,7 @@ int upload(crb_ctx* c, const Plan& P, cudaStream_t stream) {
 int launch_graph(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs, cudaStream_t stream) {
   long long occ_sig = 0;
   for (int i = 0; i < kQKernels; ++i) occ_sig = occ_sig * 31 + P.occ[i];
-  GraphKey key{P.n,      P.niter,      P.shape,      P.rows,  P.fuse,  P.fuse2, P.queue, P.seg_from,  occ_sig,      P.tiles,
+  GraphKey key{P.n,      P.niter,      P.shape,      P.rows,  P.fuse,  P.fuse2, P.queue, P.pdl, P.row_form, P.seg_from,  occ_sig,      P.tiles,
                P.rtiles, P.nblocks,    P.ncells,     P.npix,  P.bits_total, P.ncounters, P.dgrid, P.fgrid,
                P.rgrid,  c->ws,        c->d_counters, c->d_frames, P.queue ? c->d_tab : nullptr};
   for (auto& g : c->graphs)

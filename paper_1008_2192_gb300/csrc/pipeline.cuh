@@ -364,6 +364,8 @@ constexpr int kBoundThreads = 32 * kBW / kBoundNP;
 
 __global__ void __launch_bounds__(kBoundThreads, kBoundNP == 4 ? 12 : 16)
     bound_dense_kernel(const Frame* __restrict__ frames, int nframes, long long nblocks, Params p) {
+  pdl_wait();
+  pdl_launch();
   const int warp = threadIdx.x >> 5;
   for (long long b = blockIdx.x; b < nblocks; b += gridDim.x) {
     const int fi = frame_of_block(frames, nframes, b);
@@ -501,6 +503,8 @@ __device__ __forceinline__ bool strip_has_class2(const uint32_t* __restrict__ cl
 __global__ void __launch_bounds__(kColWarps * 32) need_kernel(const Frame* __restrict__ frames, int nframes,
                                                               long long nunits, Queues Q,
                                                               const uint32_t* __restrict__ cls) {
+  pdl_wait();
+  pdl_launch();
   __shared__ ColWords sw;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (long long u = (long long)blockIdx.x * kColWarps + warp; u < nunits; u += (long long)gridDim.x * kColWarps) {
@@ -602,6 +606,8 @@ template <bool kAll>
 __global__ void __launch_bounds__(kColWarps * 32) m3need_kernel(const Frame* __restrict__ frames, int nframes,
                                                                 long long nunits, Queues Q,
                                                                 const uint32_t* __restrict__ cls_in) {
+  pdl_wait();
+  pdl_launch();
   const uint32_t* __restrict__ cls = kAll ? nullptr : cls_in;
   __shared__ ColWords sw;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -697,6 +703,8 @@ __global__ void __launch_bounds__(kColWarps * 32) m3need_kernel(const Frame* __r
 // y0-2 .. y0+kSH+1 feed the five-row window.
 __global__ void __launch_bounds__(kColWarps * 32) d2_kernel(const Frame* __restrict__ frames, int nframes,
                                                             long long nunits, Queues Q, int k) {
+  pdl_wait();
+  pdl_launch();
   __shared__ ColWords sw;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (long long u = (long long)blockIdx.x * kColWarps + warp; u < nunits; u += (long long)gridDim.x * kColWarps) {
@@ -767,6 +775,8 @@ constexpr int kSegFrom = 3;
 __global__ void __launch_bounds__(kThreads) seg_list_kernel(const Frame* __restrict__ frames, int nframes,
                                                             long long nunits, Queues Q,
                                                             const uint32_t* __restrict__ cls) {
+  pdl_wait();
+  pdl_launch();
   __shared__ int ws[kThreads / 32 + 1];
   __shared__ unsigned int sbase[3];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -837,6 +847,8 @@ __device__ __forceinline__ SegLane seg_lane(const Frame* __restrict__ frames, in
 // d2_seg_kernel: d2_kernel over the listed segments.
 __global__ void __launch_bounds__(kColWarps * 32) d2_seg_kernel(const Frame* __restrict__ frames, int nframes,
                                                                 Queues Q, int k) {
+  pdl_wait();
+  pdl_launch();
   __shared__ ColWords sw;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned int nseg = Q.n[kNSegD];
@@ -885,6 +897,8 @@ __global__ void __launch_bounds__(kColWarps * 32) d2_seg_kernel(const Frame* __r
 // need_seg_kernel: need_kernel over the listed segments.
 __global__ void __launch_bounds__(kColWarps * 32) need_seg_kernel(const Frame* __restrict__ frames, int nframes,
                                                                   Queues Q, const uint32_t* __restrict__ cls) {
+  pdl_wait();
+  pdl_launch();
   __shared__ ColWords sw;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned int nseg = Q.n[kNSegN];
@@ -975,6 +989,8 @@ __global__ void __launch_bounds__(kColWarps * 32) need_seg_kernel(const Frame* _
 // m3need_seg_kernel: m3need_kernel over the listed segments.
 __global__ void __launch_bounds__(kColWarps * 32) m3need_seg_kernel(const Frame* __restrict__ frames, int nframes,
                                                                     Queues Q, const uint32_t* __restrict__ cls) {
+  pdl_wait();
+  pdl_launch();
   __shared__ ColWords sw;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned int nseg = Q.n[kNSeg];
@@ -1037,6 +1053,478 @@ __global__ void __launch_bounds__(kColWarps * 32) m3need_seg_kernel(const Frame*
     col_write(sw, warp, 1, S.gw0, wpr, base[1], reinterpret_cast<uint2*>(Q.q2));
     __syncwarp();
   }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Row forms of the bit-plane kernels, for calls below kRowFormPixels (crb.cu): a strip's rows (or a
+// segment's) are taken side by side instead of one after another. A strip walk is a chain of 24 rows of
+// loads on one warp, and a call of 8 to 17 Mpix has 4 to 7 such warps per SM: its time is that chain's
+// latency. Here a warp takes two rows of a strip (lane = word) and loads all the rows their windows need at
+// once, or a segment (lane = row), for about 1.5 times the instructions per word; larger calls, which fill
+// the chip with strips, keep the walks. The outputs are those of the strip and segment kernels (the queues
+// in another order).
+
+constexpr int kRowWarps = kSH / 2;
+static_assert(kRowWarps == 8, "256 threads: two rows of a strip per warp");
+
+// One value per warp and queue -> exclusive prefix over the block's warps, the total appended to the queue's
+// counter. Every thread calls it.
+struct RowTotals {
+  unsigned int e[kRowWarps][2], p[kRowWarps][2], base[2];
+};
+
+__device__ __forceinline__ void rows_reserve(RowTotals& T, const unsigned int (&ents)[2], const unsigned int (&pix)[2],
+                                             unsigned int* ne0, unsigned int* ne1, unsigned int* np0,
+                                             unsigned int* np1, unsigned int (&base)[2]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane < 2) {
+    T.e[warp][lane] = lane ? ents[1] : ents[0];
+    T.p[warp][lane] = lane ? pix[1] : pix[0];
+  }
+  __syncthreads();
+  unsigned int before[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const unsigned int e = lane < kRowWarps ? T.e[lane][j] : 0u;
+    before[j] = __reduce_add_sync(0xffffffffu, lane < warp ? e : 0u);
+    if (warp == j) {
+      const unsigned int n = __reduce_add_sync(0xffffffffu, e);
+      const unsigned int px = __reduce_add_sync(0xffffffffu, lane < kRowWarps ? T.p[lane][j] : 0u);
+      if (lane == 0) {
+        T.base[j] = n ? atomicAdd(j ? ne1 : ne0, n) : 0u;
+        if (px) atomicAdd(j ? np1 : np0, px);
+      }
+    }
+  }
+  __syncthreads();
+  base[0] = T.base[0] + before[0];
+  base[1] = T.base[1] + before[1];
+}
+
+// Writes the nonzero words of a warp as entries: word v of each lane is global word gw.
+__device__ __forceinline__ void row_write(uint32_t v, uint32_t gw, unsigned int& base, uint2* q) {
+  const unsigned bal = __ballot_sync(0xffffffffu, v != 0u);
+  if (v) q[base + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u))] = make_uint2(gw, v);
+  base += __popc(bal);
+}
+
+// A warp's place in a strip: word column wc (lane), first row ya of its two, halo word hw of lanes 0 and 31.
+struct RowLane {
+  const Frame* f;
+  int wc, hw, ya, wpr, h;
+  bool inw, hin;
+  uint32_t fmask, gw;  // in-frame bits of the word; global word of row ya
+};
+
+__device__ __forceinline__ RowLane row_lane(const Frame* __restrict__ frames, int nframes, long long u) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  RowLane L;
+  L.f = frames + frame_of_unit(frames, nframes, u);
+  const Frame& f = *L.f;
+  const long long lu = u - f.u0;
+  const int uy = int(lu / f.ugx), ux = int(lu - (long long)uy * f.ugx);
+  L.wpr = f.wpr;
+  L.h = f.h;
+  L.wc = ux * 32 + lane;
+  L.hw = lane == 0 ? ux * 32 - 1 : ux * 32 + 32;
+  L.ya = uy * kSH + 2 * warp;
+  L.inw = L.wc < L.wpr;
+  L.hin = (lane == 0 || lane == 31) && L.hw >= 0 && L.hw < L.wpr;
+  L.fmask = L.inw ? frame_word(L.wc, f.w) : 0u;
+  L.gw = uint32_t(f.word0 + (long long)L.ya * L.wpr + L.wc);
+  return L;
+}
+
+// Rows ya+r0 .. ya+r0+N-1 of a plane: the lane's word and its halo word (0 outside the frame).
+template <int N>
+__device__ __forceinline__ void row_load(const uint32_t* __restrict__ plane, const RowLane& L, int r0, uint32_t (&v)[N],
+                                         uint32_t (&g)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const int r = L.ya + r0 + i;
+    const bool rin = r >= 0 && r < L.h;
+    const size_t ro = size_t(rin ? r : 0) * L.wpr;
+    v[i] = (rin && L.inw) ? plane[ro + L.wc] : 0u;
+    g[i] = (rin && L.hin) ? plane[ro + L.hw] : 0u;
+  }
+}
+
+// The lane's word v dilated by R columns, from the neighbour lanes' words (the halo word g at the strip's ends);
+// row_dil_halo: the halo word itself (its bits next to the strip).
+template <int R>
+__device__ __forceinline__ uint32_t row_dil(uint32_t v, uint32_t g) {
+  const int lane = threadIdx.x & 31;
+  uint32_t l = __shfl_up_sync(0xffffffffu, v, 1), r = __shfl_down_sync(0xffffffffu, v, 1);
+  if (lane == 0) l = g;
+  if (lane == 31) r = g;
+  return hdil<R>(l, v, r);
+}
+template <int R>
+__device__ __forceinline__ uint32_t row_dil_halo(uint32_t v, uint32_t g) {
+  const bool first = (threadIdx.x & 31) == 0;
+  return hdil<R>(first ? 0u : v, g, first ? v : 0u);
+}
+
+// need_kernel, row form.
+__global__ void __launch_bounds__(256) need_row_kernel(const Frame* __restrict__ frames, int nframes, long long nunits,
+                                                       Queues Q, const uint32_t* __restrict__ cls) {
+  pdl_wait();
+  pdl_launch();
+  __shared__ RowTotals tot;
+  for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
+    const RowLane L = row_lane(frames, nframes, u);
+    const Frame& f = *L.f;
+    uint32_t h[10], gh[10], a[6], ga[6], sv[2], lz[2];
+    row_load<10>(f.hot, L, -4, h, gh);
+    row_load<6>(f.act, L, -2, a, ga);
+    const bool out = L.inw && L.ya < L.h;
+    const uint32_t cl = out ? cell_class(cls, f, L.wc, L.ya) : 0u;  // both rows lie in one cell
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const bool o = out && L.ya + j < L.h;
+      const size_t wo = size_t(o ? L.ya + j : 0) * L.wpr + (o ? L.wc : 0);
+      sv[j] = (o && cls) ? f.sval[wo] : 0u;
+      lz[j] = o ? f.lpz[wo] : 0u;
+    }
+    uint32_t n[6], gn[6];  // nsp, rows ya-2 .. ya+3
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const uint32_t v = h[i] | h[i + 1] | h[i + 2] | h[i + 3] | h[i + 4];
+      const uint32_t g = gh[i] | gh[i + 1] | gh[i + 2] | gh[i + 3] | gh[i + 4];
+      n[i] = row_dil<2>(v, g) & a[i];
+      gn[i] = row_dil_halo<2>(v, g) & ga[i];
+    }
+    uint32_t qs[2], qsp[2];
+    unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const uint32_t needS =
+          row_dil<2>(n[j] | n[j + 1] | n[j + 2] | n[j + 3] | n[j + 4], gn[j] | gn[j + 1] | gn[j + 2] | gn[j + 3] | gn[j + 4]) &
+          L.fmask;
+      qs[j] = qsp[j] = 0u;
+      if (cl >= 2u && L.ya + j < L.h) {
+        const size_t o = size_t(L.ya + j) * L.wpr + L.wc;
+        if (cl >= 3u) {
+          qsp[j] = n[j + 2];
+          f.nsp[o] = qsp[j];
+          f.test[o] = 0u;
+        }
+        const uint32_t s = cl >= 4u ? 0u : sv[j];
+        qs[j] = needS & ~s & ~lz[j];
+        if ((s | needS) != s || cl >= 4u) f.sval[o] = s | needS;
+      }
+      col_count(qs[j], ents[0], pix[0]);
+      col_count(qsp[j], ents[1], pix[1]);
+    }
+    unsigned int base[2];
+    rows_reserve(tot, ents, pix, Q.n + kNS, Q.n + kNSP, Q.n + kNSpx, Q.n + kNSPpx, base);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      row_write(qs[j], L.gw + uint32_t(j) * L.wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
+      row_write(qsp[j], L.gw + uint32_t(j) * L.wpr, base[1], reinterpret_cast<uint2*>(Q.q1));
+    }
+  }
+}
+
+// m3need_kernel<false>, row form.
+__global__ void __launch_bounds__(256) m3need_row_kernel(const Frame* __restrict__ frames, int nframes,
+                                                         long long nunits, Queues Q, const uint32_t* __restrict__ cls) {
+  pdl_wait();
+  pdl_launch();
+  __shared__ RowTotals tot;
+  for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
+    const RowLane L = row_lane(frames, nframes, u);
+    const Frame& f = *L.f;
+    uint32_t q[8], g[8], m[2];
+    row_load<8>(f.test, L, -3, q, g);
+    // rows ya-3 .. ya+4 lie in two cell rows at most
+    const int clo = max(L.ya - 3, 0) / kCH, chi = min(L.ya + 4, L.h - 1) / kCH;
+    const uint32_t* cr = cls + f.cell0;
+    const bool any = L.ya < L.h;
+    const uint32_t c0 = (any && L.inw) ? cr[(long long)clo * L.wpr + L.wc] : 0u;
+    const uint32_t c1 = (any && L.inw) ? cr[(long long)chi * L.wpr + L.wc] : 0u;
+    const uint32_t g0 = (any && L.hin) ? cr[(long long)clo * L.wpr + L.hw] : 0u;
+    const uint32_t g1 = (any && L.hin) ? cr[(long long)chi * L.wpr + L.hw] : 0u;
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      m[j] = (L.inw && L.ya + j < L.h) ? f.m3val[size_t(L.ya + j) * L.wpr + L.wc] : 0u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const bool lo = max(L.ya - 3 + i, 0) / kCH == clo;
+      if ((lo ? c0 : c1) < 2u) q[i] = 0u;
+      if ((lo ? g0 : g1) < 2u) g[i] = 0u;
+    }
+    const bool c4 = (L.ya / kCH == clo ? c0 : c1) >= 4u;
+    uint32_t qm[2], qt[2];
+    unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      uint32_t v = 0, gv = 0;
+#pragma unroll
+      for (int i = 0; i < 7; ++i) v |= q[j + i], gv |= g[j + i];
+      const uint32_t need = row_dil<3>(v, gv) & L.fmask;
+      qm[j] = qt[j] = 0u;
+      if (L.ya + j < L.h && L.inw) {
+        if (need || c4) {
+          const uint32_t old = c4 ? 0u : m[j];
+          qm[j] = need & ~old;
+          if (c4 || qm[j]) f.m3val[size_t(L.ya + j) * L.wpr + L.wc] = old | need;
+        }
+        qt[j] = q[j + 3];
+      }
+      col_count(qm[j], ents[0], pix[0]);
+      col_count(qt[j], ents[1], pix[1]);
+    }
+    unsigned int base[2];
+    rows_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, Q.n + kNM3px, Q.n + kNTpx, base);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      row_write(qm[j], L.gw + uint32_t(j) * L.wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
+      row_write(qt[j], L.gw + uint32_t(j) * L.wpr, base[1], reinterpret_cast<uint2*>(Q.q2));
+    }
+  }
+}
+
+// d2_kernel, row form.
+__global__ void __launch_bounds__(256) d2_row_kernel(const Frame* __restrict__ frames, int nframes, long long nunits,
+                                                     Queues Q, int k) {
+  pdl_wait();
+  pdl_launch();
+  __shared__ RowTotals tot;
+  for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
+    const RowLane L = row_lane(frames, nframes, u);
+    uint32_t c[6], g[6], d[2];
+    row_load<6>(L.f->chg[k & 1], L, -2, c, g);
+    unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      d[j] = row_dil<2>(c[j] | c[j + 1] | c[j + 2] | c[j + 3] | c[j + 4], g[j] | g[j + 1] | g[j + 2] | g[j + 3] | g[j + 4]);
+      d[j] = L.ya + j < L.h ? d[j] & L.fmask : 0u;
+      col_count(d[j], ents[0], pix[0]);
+    }
+    unsigned int base[2];
+    rows_reserve(tot, ents, pix, Q.n + kNB, Q.n + kNB, Q.n + kNBpx, Q.n + kNBpx, base);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) row_write(d[j], L.gw + uint32_t(j) * L.wpr, base[0], reinterpret_cast<uint2*>(Q.q2));
+  }
+}
+
+// grow_first_kernel, row form.
+__global__ void __launch_bounds__(256) grow_first_row_kernel(const Frame* __restrict__ frames, int nframes,
+                                                             long long nunits, Queues Q) {
+  pdl_wait();
+  pdl_launch();
+  __shared__ RowTotals tot;
+  const int lane = threadIdx.x & 31;
+  for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
+    const RowLane L = row_lane(frames, nframes, u);
+    const Frame& f = *L.f;
+    uint32_t c[6], e[6], t[4], et[4], low[2];
+    row_load<6>(f.cand, L, -2, c, e);
+    row_load<4>(f.test, L, -1, t, et);
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      low[j] = (L.inw && L.ya + j < L.h) ? f.low[size_t(L.ya + j) * L.wpr + L.wc] & L.fmask : 0u;
+    uint32_t g1[4], eg[4];  // the first growth, rows ya-1 .. ya+2
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t v = c[i] | c[i + 1] | c[i + 2], ev = e[i] | e[i + 1] | e[i + 2];
+      g1[i] = row_dil<1>(v, ev) & t[i];
+      eg[i] = row_dil_halo<1>(v, ev) & et[i];
+    }
+    uint32_t m[2];
+    unsigned int cnt = 0;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      m[j] = row_dil<1>(g1[j] | g1[j + 1] | g1[j + 2], eg[j] | eg[j + 1] | eg[j + 2]) & low[j];
+      if (L.inw && L.ya + j < L.h) f.bits_a[size_t(L.ya + j) * L.wpr + L.wc] = m[j];
+      cnt += unsigned(__popc(m[j]));
+    }
+    unsigned int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const unsigned int n = __shfl_sync(0xffffffffu, incl, 31);
+    const unsigned int ents[2] = {n, 0u}, pix[2] = {0u, 0u};
+    unsigned int base[2];
+    rows_reserve(tot, ents, pix, Q.n + kNRep, Q.n + kNRep, nullptr, nullptr, base);
+    if (lane == 0 && n) atomicAdd(f.counters + 0, (unsigned long long)n);
+    unsigned int o = base[0] + incl - cnt;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const uint32_t row = uint32_t(f.pix0 + (long long)(L.ya + j) * f.w + 32 * L.wc);
+      for (uint32_t v = m[j]; v; v &= v - 1u) Q.q1[o++] = row + unsigned(__ffs(v) - 1);
+    }
+  }
+}
+
+// Segments, lane = row: rows y0-4 .. y0+19 of the listed segment in lanes 0 .. 23.
+constexpr int kSegPerWarp = 4;  // segments per warp and append
+
+struct SegRow {
+  const Frame* f;
+  int wc, y;   // the lane's row
+  size_t ro;   // its word
+  bool rin, inl, inr, out;
+  uint32_t fmask, gw;
+};
+
+__device__ __forceinline__ SegRow seg_row(const Frame* __restrict__ frames, int nframes, const uint32_t* seg,
+                                          unsigned int i, unsigned int nseg) {
+  const int lane = threadIdx.x & 31;
+  SegRow S;
+  const bool ok = i < nseg;
+  const uint32_t s = seg[ok ? i : 0];
+  const long long u = s >> 5;
+  S.f = frames + frame_of_unit(frames, nframes, u);
+  const Frame& f = *S.f;
+  const long long lu = u - f.u0;
+  const int uy = int(lu / f.ugx), ux = int(lu - (long long)uy * f.ugx);
+  S.wc = ux * 32 + int(s & 31u);
+  S.y = uy * kSH - 4 + lane;
+  S.rin = ok && lane < kSH + 8 && S.y >= 0 && S.y < f.h;
+  S.out = S.rin && lane >= 4 && lane < kSH + 4;
+  S.ro = S.rin ? size_t(S.y) * f.wpr + S.wc : 0;
+  S.inl = S.rin && S.wc > 0;
+  S.inr = S.rin && S.wc + 1 < f.wpr;
+  S.fmask = frame_word(S.wc, f.w);
+  S.gw = uint32_t(f.word0 + (long long)S.ro);
+  return S;
+}
+
+// OR of the words of rows r-R .. r+R (lane = row; lanes whose window leaves the warp are not used)
+template <int R>
+__device__ __forceinline__ uint32_t vor(uint32_t v) {
+  uint32_t o = v;
+#pragma unroll
+  for (int d = 1; d <= R; ++d) o |= __shfl_up_sync(0xffffffffu, v, d) | __shfl_down_sync(0xffffffffu, v, d);
+  return o;
+}
+
+// A block's listed segments from b on: body(j, segment) for the warp's kSegPerWarp of them, then the append.
+template <typename F>
+__device__ __forceinline__ void seg_blocks(unsigned int nseg, F&& body) {
+  constexpr unsigned int kPer = kRowWarps * kSegPerWarp;
+  for (unsigned int b = blockIdx.x * kPer; b < nseg; b += gridDim.x * kPer)
+    body(b + (threadIdx.x >> 5) * kSegPerWarp);
+}
+
+__global__ void __launch_bounds__(256) d2_segrow_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
+                                                        int k) {
+  pdl_wait();
+  pdl_launch();
+  __shared__ RowTotals tot;
+  const unsigned int nseg = Q.n[kNSegD];
+  seg_blocks(nseg, [&](unsigned int i0) {
+    uint32_t d[kSegPerWarp], gw[kSegPerWarp];
+    unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
+#pragma unroll
+    for (int j = 0; j < kSegPerWarp; ++j) {
+      const SegRow S = seg_row(frames, nframes, Q.seg[2], i0 + j, nseg);
+      const uint32_t* chg = S.f->chg[k & 1];
+      const uint32_t c = S.rin ? chg[S.ro] : 0u, l = S.inl ? chg[S.ro - 1] : 0u, r = S.inr ? chg[S.ro + 1] : 0u;
+      d[j] = hdil<2>(vor<2>(l), vor<2>(c), vor<2>(r)) & S.fmask;
+      if (!S.out) d[j] = 0u;
+      gw[j] = S.gw;
+      col_count(d[j], ents[0], pix[0]);
+    }
+    unsigned int base[2];
+    rows_reserve(tot, ents, pix, Q.n + kNB, Q.n + kNB, Q.n + kNBpx, Q.n + kNBpx, base);
+#pragma unroll
+    for (int j = 0; j < kSegPerWarp; ++j) row_write(d[j], gw[j], base[0], reinterpret_cast<uint2*>(Q.q2));
+  });
+}
+
+__global__ void __launch_bounds__(256) need_segrow_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
+                                                          const uint32_t* __restrict__ cls) {
+  pdl_wait();
+  pdl_launch();
+  __shared__ RowTotals tot;
+  const unsigned int nseg = Q.n[kNSegN];
+  seg_blocks(nseg, [&](unsigned int i0) {
+    uint32_t qs[kSegPerWarp], qsp[kSegPerWarp], gw[kSegPerWarp];
+    unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
+#pragma unroll
+    for (int j = 0; j < kSegPerWarp; ++j) {
+      const SegRow S = seg_row(frames, nframes, Q.seg[1], i0 + j, nseg);
+      const Frame& f = *S.f;
+      const uint32_t hc = S.rin ? f.hot[S.ro] : 0u, hl = S.inl ? f.hot[S.ro - 1] : 0u, hr = S.inr ? f.hot[S.ro + 1] : 0u;
+      const uint32_t ac = S.rin ? f.act[S.ro] : 0u, al = S.inl ? f.act[S.ro - 1] : 0u, ar = S.inr ? f.act[S.ro + 1] : 0u;
+      const uint32_t cl = S.out ? cls[f.cell0 + (long long)(S.y / kCH) * f.wpr + S.wc] : 0u;
+      const uint32_t sval = S.out ? f.sval[S.ro] : 0u, lz = S.out ? f.lpz[S.ro] : 0u;
+      // nsp: exact in the own word, and in the two bits of each side word next to it
+      const uint32_t vl = vor<2>(hl), vc = vor<2>(hc), vr = vor<2>(hr);
+      const uint32_t nl = hdil<2>(0u, vl, vc) & al, nc = hdil<2>(vl, vc, vr) & ac, nr = hdil<2>(vc, vr, 0u) & ar;
+      const uint32_t needS = hdil<2>(vor<2>(nl), vor<2>(nc), vor<2>(nr)) & S.fmask;
+      qs[j] = qsp[j] = 0u;
+      gw[j] = S.gw;
+      if (cl >= 2u) {
+        if (cl >= 3u) {
+          qsp[j] = nc;
+          f.nsp[S.ro] = nc;
+          f.test[S.ro] = 0u;
+        }
+        const uint32_t s = cl < 4u ? sval : 0u;  // S is not current anywhere in cells of class 4
+        qs[j] = needS & ~s & ~lz;
+        if ((s | needS) != s || cl >= 4u) f.sval[S.ro] = s | needS;
+      }
+      col_count(qs[j], ents[0], pix[0]);
+      col_count(qsp[j], ents[1], pix[1]);
+    }
+    unsigned int base[2];
+    rows_reserve(tot, ents, pix, Q.n + kNS, Q.n + kNSP, Q.n + kNSpx, Q.n + kNSPpx, base);
+#pragma unroll
+    for (int j = 0; j < kSegPerWarp; ++j) {
+      row_write(qs[j], gw[j], base[0], reinterpret_cast<uint2*>(Q.q0));
+      row_write(qsp[j], gw[j], base[1], reinterpret_cast<uint2*>(Q.q1));
+    }
+  });
+}
+
+__global__ void __launch_bounds__(256) m3need_segrow_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
+                                                            const uint32_t* __restrict__ cls) {
+  pdl_wait();
+  pdl_launch();
+  __shared__ RowTotals tot;
+  const unsigned int nseg = Q.n[kNSeg];
+  seg_blocks(nseg, [&](unsigned int i0) {
+    uint32_t qm[kSegPerWarp], qt[kSegPerWarp], gw[kSegPerWarp];
+    unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
+#pragma unroll
+    for (int j = 0; j < kSegPerWarp; ++j) {
+      const SegRow S = seg_row(frames, nframes, Q.seg[0], i0 + j, nseg);
+      const Frame& f = *S.f;
+      const uint32_t* cr = cls + f.cell0 + (long long)((S.rin ? S.y : 0) / kCH) * f.wpr + S.wc;
+      const uint32_t cl = S.rin ? cr[0] : 0u;
+      const uint32_t c = (S.rin ? f.test[S.ro] : 0u) & (cl >= 2u ? ~0u : 0u);
+      const uint32_t l = S.inl ? f.test[S.ro - 1] & (cr[-1] >= 2u ? ~0u : 0u) : 0u;
+      const uint32_t r = S.inr ? f.test[S.ro + 1] & (cr[1] >= 2u ? ~0u : 0u) : 0u;
+      const uint32_t m = S.out ? f.m3val[S.ro] : 0u;
+      const uint32_t need = hdil<3>(vor<3>(l), vor<3>(c), vor<3>(r)) & S.fmask;
+      qm[j] = qt[j] = 0u;
+      gw[j] = S.gw;
+      if (S.out) {
+        const bool c4 = cl >= 4u;
+        if (need || c4) {
+          const uint32_t old = c4 ? 0u : m;  // M3 is not current anywhere in cells of class 4
+          qm[j] = need & ~old;
+          if (c4 || qm[j]) f.m3val[S.ro] = old | need;
+        }
+        qt[j] = c;
+      }
+      col_count(qm[j], ents[0], pix[0]);
+      col_count(qt[j], ents[1], pix[1]);
+    }
+    unsigned int base[2];
+    rows_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, Q.n + kNM3px, Q.n + kNTpx, base);
+#pragma unroll
+    for (int j = 0; j < kSegPerWarp; ++j) {
+      row_write(qm[j], gw[j], base[0], reinterpret_cast<uint2*>(Q.q0));
+      row_write(qt[j], gw[j], base[1], reinterpret_cast<uint2*>(Q.q2));
+    }
+  });
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1291,6 +1779,8 @@ __device__ __forceinline__ void load_pair_span(const float* __restrict__ a, int 
 // groups of four would hold 1.9 listed pixels on average, and measured slower
 // than single medians; a run of five listed pixels fills three pairs.)
 __global__ void __launch_bounds__(256, 4) s_kernel(const Frame* __restrict__ frames, int nframes, Queues Q, int k) {
+  pdl_wait();
+  pdl_launch();
   expand_words<2, true>(frames, nframes, reinterpret_cast<const uint2*>(Q.q0), Q.n[kNS],
                   [&](bool valid, int fi, int x0, int y, uint32_t bits) {
                     if (!valid) return;
@@ -1328,6 +1818,8 @@ __device__ __forceinline__ uint32_t plane_bits8(const uint32_t* __restrict__ pla
 // per SM (80 registers, 20 B of spills) measured 4 % faster than two (103).
 __global__ void __launch_bounds__(256, 3) sp_kernel(const Frame* __restrict__ frames, int nframes, Queues Q, Params p,
                                                     int k) {
+  pdl_wait();
+  pdl_launch();
   const float siglow = __fmul_rn(p.sigfrac, p.sigclip);
   expand_words<2, true>(frames, nframes, reinterpret_cast<const uint2*>(Q.q1), Q.n[kNSP],
                   [&](bool valid, int fi, int x0, int y, uint32_t bits) {
@@ -1376,6 +1868,8 @@ __global__ void __launch_bounds__(256, 3) sp_kernel(const Frame* __restrict__ fr
 // largest of its column minima, the median of its column medians and the
 // smallest of its column maxima (an exact selection of the fifth of nine).
 __global__ void __launch_bounds__(256) m3_kernel(const Frame* __restrict__ frames, int nframes, Queues Q, int k) {
+  pdl_wait();
+  pdl_launch();
   expand_words<4, true>(frames, nframes, reinterpret_cast<const uint2*>(Q.q0), Q.n[kNM3],
                   [&](bool valid, int fi, int x0, int y, uint32_t bits) {
                     if (!valid) return;
@@ -1415,6 +1909,8 @@ __global__ void __launch_bounds__(256) m3_kernel(const Frame* __restrict__ frame
 // XORs of disjoint bits by other groups of the word commute with it.
 __global__ void __launch_bounds__(256, 4) bound_sparse_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
                                                            Params p) {
+  pdl_wait();
+  pdl_launch();
   expand_words<4, true>(frames, nframes, reinterpret_cast<const uint2*>(Q.q2), Q.n[kNB],
                   [&](bool valid, int fi, int x0, int y, uint32_t) {
                     if (!valid) return;
@@ -1495,6 +1991,8 @@ __device__ __forceinline__ void load_pair_span7(const float* __restrict__ a, int
 // two (102 registers).
 __global__ void __launch_bounds__(256, 3) cand_test_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
                                                            Params p, int k) {
+  pdl_wait();
+  pdl_launch();
   __shared__ WarpLists<2, 128> wl;
   wl.init();
   uint32_t* const lists[2] = {Q.q0, Q.q1};
@@ -1554,9 +2052,16 @@ __global__ void __launch_bounds__(256, 3) cand_test_kernel(const Frame* __restri
 }
 
 // cand_full_kernel: at the open tests, the exact F = m3 - med7(m3) and the
-// objlim test -> candidates.
+// objlim test -> candidates. It also clears the cell classes and changed pixels
+// the replacement will mark (n0 and n1 16-byte vectors at z0 and z1), last read
+// in the previous iteration.
 __global__ void __launch_bounds__(256) cand_full_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
-                                                        Params p, int k) {
+                                                        Params p, int k, uint4* z0, size_t n0, uint4* z1, size_t n1) {
+  pdl_wait();
+  pdl_launch();
+  const size_t zt = size_t(blockIdx.x) * blockDim.x + threadIdx.x, zs = size_t(gridDim.x) * blockDim.x;
+  for (size_t i = zt; i < n0; i += zs) z0[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (size_t i = zt; i < n1; i += zs) z1[i] = make_uint4(0u, 0u, 0u, 0u);
   __shared__ WarpLists<1, 128> wl;
   wl.init();
   uint32_t* const lists[1] = {Q.q0};
@@ -1596,6 +2101,8 @@ __global__ void __launch_bounds__(256) cand_full_kernel(const Frame* __restrict_
 // replacement, all of them being new.
 __global__ void __launch_bounds__(kColWarps * 32) grow_first_kernel(const Frame* __restrict__ frames, int nframes,
                                                                     long long nunits, Queues Q) {
+  pdl_wait();
+  pdl_launch();
   __shared__ ColWords sw;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (long long u = (long long)blockIdx.x * kColWarps + warp; u < nunits; u += (long long)gridDim.x * kColWarps) {
@@ -1683,6 +2190,8 @@ __global__ void __launch_bounds__(kColWarps * 32) grow_first_kernel(const Frame*
 // either threshold.
 __global__ void __launch_bounds__(256, 4) grow_kernel(const Frame* __restrict__ frames, int nframes, Queues Q, Params p,
                                                    int k) {
+  pdl_wait();
+  pdl_launch();
   const unsigned int n = Q.n[kNPass];
   const float sigclip = p.sigclip, siglow = __fmul_rn(p.sigfrac, p.sigclip);
   const unsigned int stride = gridDim.x * blockDim.x;
@@ -1831,6 +2340,8 @@ __device__ __forceinline__ uint32_t or_window(uint32_t* plane, int wpr, int h, i
 // may have changed in it) -> the replacement queue, each once (bit plane rq;
 // one append atomic per block).
 __global__ void __launch_bounds__(256) rq_kernel(const Frame* __restrict__ frames, int nframes, Queues Q) {
+  pdl_wait();
+  pdl_launch();
   __shared__ int ws[kThreads / 32 + 1];
   __shared__ unsigned int sbase;
   const unsigned int nf = Q.n[kNFresh], n = nf + Q.n[kNFb];
@@ -1898,6 +2409,8 @@ __device__ __forceinline__ void mark_change(const Frame& f, int x, int y, uint32
 // directly (`cls_next`: cell classes to mark, or nullptr).
 __global__ void __launch_bounds__(256) rep_compute_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
                                                           int k, uint32_t* cls_next) {
+  pdl_wait();
+  pdl_launch();
   const unsigned int n = Q.n[kNRep];
   float* __restrict__ vals = reinterpret_cast<float*>(Q.q0);
   for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -1957,6 +2470,8 @@ __global__ void __launch_bounds__(256) rep_compute_kernel(const Frame* __restric
 // Clears the queued bits.
 __global__ void __launch_bounds__(256) rep_write_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
                                                         uint32_t* cls_next, int knext, int clear_rq) {
+  pdl_wait();
+  pdl_launch();
   const unsigned int n = Q.n[kNRep];
   const float* __restrict__ vals = reinterpret_cast<const float*>(Q.q0);
   for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -1977,30 +2492,61 @@ __global__ void __launch_bounds__(256) rep_write_kernel(const Frame* __restrict_
 // thread; two 16-byte stores when the 32 bytes are aligned).
 __device__ __forceinline__ uint32_t nibble_bytes(uint32_t nib) { return (nib * 0x00204081u) & 0x01010101u; }
 
+// 16 mask bytes from 16 flag bits
+__device__ __forceinline__ uint4 mask16(uint32_t v) {
+  return make_uint4(nibble_bytes(v & 15u), nibble_bytes((v >> 4) & 15u), nibble_bytes((v >> 8) & 15u),
+                    nibble_bytes((v >> 12) & 15u));
+}
+
 __global__ void __launch_bounds__(256) mask_kernel(const Frame* __restrict__ frames, int nframes, long long nblocks) {
+  pdl_wait();
+  pdl_launch();
   const int t = threadIdx.x;
   for (long long b = blockIdx.x; b < nblocks; b += gridDim.x) {
     const int fi = frame_of_block(frames, nframes, b);
     const Frame& f = frames[fi];
     const long long lb = b - f.blk0;
+    if (!f.out_mask) continue;
+    const int w = f.w, wpr = f.wpr;
+    const unsigned int npix = unsigned(w) * unsigned(f.h);
+    if (((w & 15) != 0 || (reinterpret_cast<uintptr_t>(f.out_mask) & 15u) != 0) && w >= 32) {
+      // Rows off the 16-byte boundaries: the frame's mask as one array, the block taking the 16-byte vectors
+      // of kBW x kBH words' worth of bytes from its first aligned address on; a vector holds the end of one
+      // row and the start of the next at most (one word and 32 byte stores per thread took 48 us on
+      // 4146 x 2051, 8 us so).
+      const unsigned int head = unsigned(-reinterpret_cast<uintptr_t>(f.out_mask) & 15u);  // bytes before it
+      auto bits = [&](unsigned int o, int n) {  // flags of the n <= 16 pixels from o on
+        unsigned int y = o / unsigned(w), x = o - y * unsigned(w);
+        const uint32_t* p = f.bits_a + size_t(y) * wpr;
+        auto word = [&](const uint32_t* q, unsigned int i) { return int(i) < wpr ? q[i] : 0u; };
+        uint32_t v = __funnelshift_r(word(p, x >> 5), word(p, (x >> 5) + 1), x & 31u);
+        const int left = w - int(x);  // pixels of this row
+        if (left < n) v = (v & ((1u << left) - 1u)) | (p[wpr] << left);
+        return v;
+      };
+      constexpr unsigned int kPer = kBW * kBH * 2;  // vectors per block
+      for (unsigned int i = t; i < kPer; i += 256) {
+        const unsigned long long o = head + ((unsigned long long)lb * kPer + i) * 16u;
+        if (o >= npix) break;
+        const int n = int(min(16ull, npix - o));
+        const uint32_t v = bits(unsigned(o), n);
+        if (n == 16)
+          *reinterpret_cast<uint4*>(f.out_mask + o) = mask16(v);
+        else
+          for (int j = 0; j < n; ++j) f.out_mask[o + j] = uint8_t((v >> j) & 1u);
+      }
+      if (lb == 0 && t < int(min(head, npix))) f.out_mask[t] = uint8_t(bits(unsigned(t), 1) & 1u);
+      continue;
+    }
     const int bys = int(lb / f.bx), bxs = int(lb - (long long)bys * f.bx);
     const int y = bys * kBH + t / kBW, wc = bxs * kBW + t % kBW;
-    if (y >= f.h || wc >= f.wpr || !f.out_mask) continue;
-    const uint32_t v = f.bits_a[size_t(y) * f.wpr + wc];
-    uint8_t* o = f.out_mask + size_t(y) * f.w + 32 * wc;
-    const int nb = min(32, f.w - 32 * wc);
+    if (y >= f.h || wc >= wpr) continue;
+    const uint32_t v = f.bits_a[size_t(y) * wpr + wc];
+    uint8_t* o = f.out_mask + size_t(y) * w + 32 * wc;
+    const int nb = min(32, w - 32 * wc);
     if (nb == 32 && (reinterpret_cast<uintptr_t>(o) & 15u) == 0) {
-      uint4 q0, q1;
-      q0.x = nibble_bytes(v & 15u);
-      q0.y = nibble_bytes((v >> 4) & 15u);
-      q0.z = nibble_bytes((v >> 8) & 15u);
-      q0.w = nibble_bytes((v >> 12) & 15u);
-      q1.x = nibble_bytes((v >> 16) & 15u);
-      q1.y = nibble_bytes((v >> 20) & 15u);
-      q1.z = nibble_bytes((v >> 24) & 15u);
-      q1.w = nibble_bytes(v >> 28);
-      reinterpret_cast<uint4*>(o)[0] = q0;
-      reinterpret_cast<uint4*>(o)[1] = q1;
+      reinterpret_cast<uint4*>(o)[0] = mask16(v);
+      reinterpret_cast<uint4*>(o)[1] = mask16(v >> 16);
     } else {
       for (int bb = 0; bb < nb; ++bb) o[bb] = uint8_t((v >> bb) & 1u);
     }
@@ -2011,6 +2557,7 @@ __global__ void __launch_bounds__(256) mask_kernel(const Frame* __restrict__ fra
 // totals of the call) and clears the per-iteration counters. Bound tests:
 // `dense` positions in iteration 1, the re-tested pixels after it.
 __global__ void queue_work_kernel(const Frame* __restrict__ frames, Queues Q, int k, long long dense) {
+  pdl_wait();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     unsigned long long* wk = frames[0].work + kWork * (k - 1);
     wk[0] += Q.n[kNSpx];

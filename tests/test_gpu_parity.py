@@ -442,3 +442,37 @@ def test_row_tiles_edges(w, h, pset):
         r32 = oracle.clean(img, params_of(pset), niter, precision="f32")
         assert np.array_equal(mask, r32.mask) and np.array_equal(out, r32.clean), niter
         assert c.last_counts() == list(zip(r32.n_new, r32.n_none_left)), niter
+
+
+@pytest.mark.parametrize("w,h", [(32, 40), (33, 40), (47, 33), (50, 17), (1040, 37), (1025, 18)])
+def test_queue_masks_off_alignment(w, h):
+    """The u8 mask of rows off the 16-byte boundaries, at every offset of the mask's first byte: 16-byte vectors
+    over row ends, and the bytes before the first and after the last."""
+    img = scene(w, h, seed=w + h)
+    r32 = oracle.clean(img, params_of({}), 2, precision="f32")
+    c = Cleaner(niter=2, pipeline="queue")
+    x = dev(img)
+    for off in (0, 1, 7, 15):
+        buf = torch.full((w * h + 32,), 9, dtype=torch.uint8, device="cuda")
+        out, mask = torch.empty_like(x), buf[off:off + w * h].view(h, w)
+        c.clean_into(x, out, mask)
+        c.sync()
+        assert np.array_equal(host(mask), r32.mask) and np.array_equal(host(out), r32.clean), off
+        assert (buf[:off] == 9).all() and (buf[off + w * h:] == 9).all(), off
+
+
+@pytest.mark.parametrize("niter", [1, 2, 3, 5])
+def test_row_and_strip_forms_agree(niter):
+    """A batch above the size from which the bit-plane kernels walk strips and segments gives each frame what the
+    row forms (a call of its own) give: strip tails in both directions, frames narrower than a strip."""
+    sizes = [(8200, 8200), (1056, 33), (31, 500), (2080, 47), (993, 129)]  # the first alone is above the limit
+    imgs = [dev(synth.frame(w, h, seed=61, index=i) if w * h < 10**7 else
+                np.tile(synth.frame(820, 820, seed=61), (10, 10))) for i, (w, h) in enumerate(sizes)]
+    c = Cleaner(niter=niter, pipeline="queue")
+    outs, masks = c.clean_batch(imgs)
+    crops = [x if i else x[:3000, :2500].contiguous() for i, x in enumerate(imgs)]
+    for i, x in enumerate(crops):
+        o, m = c.clean(x)
+        a, b = (slice(None), slice(None)) if i else (slice(0, 2900), slice(0, 2400))  # away from the crop's cut
+        c.sync()
+        assert torch.equal(o[a, b], outs[i][a, b]) and torch.equal(m[a, b], masks[i][a, b]), sizes[i]
