@@ -78,7 +78,7 @@ constexpr int kOneRoundShape = 5;
 // The row kernels (tile.cuh) by tile height.
 struct TileKernels {
   int th;
-  void (*fn[3])(const crb::Frame*, int, crb::Params, int, int);  // iteration 1, later ones, the last replacement
+  void (*fn[3])(const crb::Frame*, int, crb::Params, int, int, const crb::Frame);  // iteration 1, later ones, the last replacement
   int smem;
 };
 template <int TH>
@@ -434,6 +434,7 @@ struct Plan {
   bool row_form = false;  // the row forms of the bit-plane kernels
   bool zeroed = false;  // the upload zeroes the planes and counters (else two memsets do)
   bool fuse2 = false;  // tile pipeline: iterations 2 and 3 in one launch
+  bool one = false;    // row kernels: one frame, whose descriptor iteration 1 takes with its launch (not in a graph)
   int rows = -1;       // tile pipeline: the row kernels' variant (kTileKernels), or -1 for the detect kernels
   long long tiles = 0, rtiles = 0;
   size_t bits_total = 0;  // bytes from the start of the workspace that start at zero
@@ -652,7 +653,8 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
     for (int k = 1; k <= P.niter + 1; ++k) {
       const int mode = k == 1 ? 0 : k <= P.niter ? 1 : 2;
       timed(c, mode == 2 ? kPTileReplace : kPTileDetect, stream, [&] {
-        launch_pdl(t.fn[mode], unsigned(P.tiles), 256, t.smem, stream, c->d_frames, P.n, c->p, k, P.niter);
+        launch_pdl(t.fn[mode], unsigned(P.tiles), 256, t.smem, stream, c->d_frames, k == 1 && P.one ? 0 : P.n, c->p, k, P.niter,
+                   c->h_frames[0]);
       });
     }
     CRB_CUDA(cudaGetLastError());
@@ -973,6 +975,7 @@ int prepare_tile(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pla
   P.niter = niter;
   P.fuse = true;
   P.rows = v;
+  P.one = n == 1 && !c->opt.use_graphs;
   P.zeroed = true;
   P.tiles = tiles;
   P.bits_total = bits;

@@ -191,6 +191,15 @@ __device__ __noinline__ float median25_at(const float* a, int r, int c, int rlo,
   return a[r * kT2P + c];
 }
 
+// med3 at (r, c) of the image region.
+__device__ __noinline__ float med3_at(const float* a, int r, int c) {
+  const float* p = a + (r - 1) * kT2P + c - 1;
+  float lo[3], mi[3], hi[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) sort3(p[d], p[d + kT2P], p[d + 2 * kT2P], lo[d], mi[d], hi[d]);
+  return med3f(max3f(lo[0], lo[1], lo[2]), med3f(mi[0], mi[1], mi[2]), min3f(hi[0], hi[1], hi[2]));
+}
+
 // Scale of the objlim test of a pixel: the test holds for a value v of the 7x7
 // window in the place of the median exactly where S'/max(F/N, 0.01) > objlim
 // with F = m3 - v (article form: 2S for S'), that is where F < X up to
@@ -208,11 +217,16 @@ __device__ __forceinline__ bool test_holds(const Params& p, float fval, float nn
   return __fdiv_rn(num, fmaxf(__fdiv_rn(fval, nn), 0.01f)) > p.objlim;
 }
 
+// What a launch does before pdl_wait depends on nothing the launch ahead of it
+// writes: iteration 1 of a call of one frame (nframes 0: its descriptor `one`
+// comes with the launch) needs only the input until it writes its flags, so it
+// runs beside the upload; later launches load M_{k-2}, and iteration 2 the
+// input, while the launch ahead ends.
 // kMode 0: iteration 1. 1: the replacement of iteration k-1, then iteration k.
 // 2: the replacement of iteration niter (k = niter + 1) and the u8 mask.
 template <int TH, int kMode>
 __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ frames, int nframes, Params p, int k,
-                                                      int niter) {
+                                                      int niter, const __grid_constant__ Frame one) {
   using L = TileLayout<TH>;
   constexpr int R = L::R;
   extern __shared__ __align__(128) char smem[];
@@ -238,13 +252,14 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
   // on the kernel before this one (pdl_wait)
   for (int i = tid; i < 6 * R; i += 256) mC[i] = make_uint2(0u, 0u);
   if (tid < 16) cnt[tid] = 0;
-  if (kMode == 0) {
+  if (kMode == 0 && nframes) {
     pdl_wait();
     pdl_launch();
   }
   __shared__ Frame sf;
   {
-    const uint32_t* d = reinterpret_cast<const uint32_t*>(frames + frame_of<false>(frames, nframes, blockIdx.x));
+    const uint32_t* d = reinterpret_cast<const uint32_t*>(
+        (kMode == 0 && !nframes) ? &one : frames + frame_of<false>(frames, nframes, blockIdx.x));
     for (int i = tid; i < int(sizeof(Frame) / 4); i += 256) reinterpret_cast<uint32_t*>(&sf)[i] = d[i];
   }
   __syncthreads();
@@ -262,13 +277,9 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
     T.edge = T.c0 > 2 || T.r0 > 2 || T.c1 < 62 || T.r1 < R - 2;
   }
   const float* src = kMode == 0 ? f.img : iter_src(f, k - 1, niter);
-  if (kMode != 0) {
-    pdl_wait();
-    if (kMode == 1) pdl_launch();  // the last kernel's results are the caller's: nothing starts before they are whole
-  }
 
   // the image region (mode 2: the tile and the 2 rows around it), clamped into the frame
-  {
+  auto load_image = [&] {
     constexpr int ra = kMode == 2 ? 6 : kMode == 0 ? 2 : 0, rb = R - ra;
     if ((w & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
       for (int i = tid; i < (rb - ra) * 16; i += 256) {
@@ -291,17 +302,24 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
       }
     }
     cp_async_commit();
-  }
+  };
   const uint2 own = T.cols(0);
+  if (kMode == 0 || k == 2) load_image();
 
   if (kMode != 0) {
     const int kr = k - 1;  // the iteration whose replacement this is
-    for (int r = tid; r < R; r += 256) {
-      const int gy = clampi(T.y0 - 8 + r, 0, h - 1);
-      const uint2 a = plane_row(f.mp[kr % 3], wps, gy, T), b = plane_row(f.mp[(kr + 2) % 3], wps, gy, T);
-      mM[r] = a;
-      mF[r] = make_uint2(a.x & ~b.x, a.y & ~b.y);
+    static_assert(R <= 256, "a thread per row");
+    const int gy = clampi(T.y0 - 8 + tid, 0, h - 1);
+    uint2 before = make_uint2(0u, 0u);
+    if (tid < R) before = plane_row(f.mp[(kr + 2) % 3], wps, gy, T);
+    pdl_wait();
+    if (kMode == 1) pdl_launch();  // the last kernel's results are the caller's: nothing starts before they are whole
+    if (tid < R) {
+      const uint2 a = plane_row(f.mp[kr % 3], wps, gy, T);
+      mM[tid] = a;
+      mF[tid] = make_uint2(a.x & ~before.x, a.y & ~before.y);
     }
+    if (k != 2) load_image();
     __syncthreads();
     // list the flagged pixels whose value can change
     constexpr int kReach = kMode == 2 ? 0 : 6;
@@ -329,6 +347,37 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
         for (uint32_t v = j ? m.y : m.x; v; v &= v - 1u) L0[o++] = uint16_t((tid << 6) | (2 * (__ffs(v) - 1) + j));
     }
   }
+  // I_{k-1} of the tile, by the threads from `first` on: the first write into each image buffer is whole,
+  // later ones the flagged pixels
+  auto write_image = [&](int first) {
+    float* __restrict__ dst = iter_dst(f, k - 1, niter);
+    if (k - 1 <= 2) {
+      if ((w & 3) == 0 && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
+        for (int i = tid - first; i < TH * 12; i += 256 - first) {
+          const int r = 8 + i / 12, c = 8 + (i % 12) * 4;
+          if (r < T.r1 && c < T.c1)
+            *reinterpret_cast<float4*>(dst + size_t(T.y0 - 8 + r) * w + T.x0 - 8 + c) =
+                *reinterpret_cast<const float4*>(sJ + r * kT2P + c);
+        }
+      } else {
+        for (int i = tid - first; i < TH * kT2W; i += 256 - first) {
+          const int r = 8 + i / kT2W, c = 8 + i % kT2W;
+          if (r < T.r1 && c < T.c1) dst[size_t(T.y0 - 8 + r) * w + T.x0 - 8 + c] = sJ[r * kT2P + c];
+        }
+      }
+    } else if (tid - first < 2 * TH) {  // a thread per row and parity
+      const int r = 8 + ((tid - first) >> 1), j = (tid - first) & 1;
+      if (r < T.r1) {
+        const uint2 m = and2(mM[r], own);
+        uint32_t v = j ? m.y : m.x;
+        while (v) {
+          const int c = 2 * (__ffs(v) - 1) + j;
+          v &= v - 1u;
+          dst[size_t(T.y0 - 8 + r) * w + T.x0 - 8 + c] = sJ[r * kT2P + c];
+        }
+      }
+    }
+  };
   cp_async_wait_all();
   __syncthreads();
 
@@ -380,35 +429,8 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
       for (int j = tid; j < nR; j += 256) sJ[(L0[j] >> 6) * kT2P + (L0[j] & 63)] = val[j];
     }
     const bool any = __syncthreads_or(changed);
-    // I_{k-1} of the tile: the first write into each image buffer is whole, later ones the flagged pixels
-    float* __restrict__ dst = iter_dst(f, k - 1, niter);
-    if (k - 1 <= 2) {
-      if ((w & 3) == 0 && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
-        for (int i = tid; i < TH * 12; i += 256) {
-          const int r = 8 + i / 12, c = 8 + (i % 12) * 4;
-          if (r < T.r1 && c < T.c1)
-            *reinterpret_cast<float4*>(dst + size_t(T.y0 - 8 + r) * w + T.x0 - 8 + c) =
-                *reinterpret_cast<const float4*>(sJ + r * kT2P + c);
-        }
-      } else {
-        for (int i = tid; i < TH * kT2W; i += 256) {
-          const int r = 8 + i / kT2W, c = 8 + i % kT2W;
-          if (r < T.r1 && c < T.c1) dst[size_t(T.y0 - 8 + r) * w + T.x0 - 8 + c] = sJ[r * kT2P + c];
-        }
-      }
-    } else if (tid < 2 * TH) {  // a thread per row and parity
-      const int r = 8 + (tid >> 1), j = tid & 1;
-      if (r < T.r1) {
-        const uint2 m = and2(mM[r], own);
-        uint32_t v = j ? m.y : m.x;
-        while (v) {
-          const int c = 2 * (__ffs(v) - 1) + j;
-          v &= v - 1u;
-          dst[size_t(T.y0 - 8 + r) * w + T.x0 - 8 + c] = sJ[r * kT2P + c];
-        }
-      }
-    }
     if (kMode == 2) {
+      write_image(0);
       uint8_t* __restrict__ om = f.out_mask;
       if (!om) return;
       if ((w & 15) == 0 && (reinterpret_cast<uintptr_t>(om) & 15u) == 0) {
@@ -437,6 +459,7 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
       return;
     }
     if (!any) {  // J did not change within 6 px: no new flag
+      write_image(0);
       if (tid < 2 * TH) {
         const int r = 8 + (tid >> 1), j = tid & 1;
         if (r < T.r1) {
@@ -454,26 +477,31 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
       }
       __syncthreads();
     }
-    // the pixels within 6 px of a change
-    if (tid < R) {
-      uint2 z = make_uint2(0u, 0u);
-#pragma unroll
-      for (int d = -6; d <= 6; ++d)
-        if (tid + d >= 0 && tid + d < R) z = or2(z, mC[tid + d]);
-      mF[tid] = hdil6(z);
-    }
   }
 
   const float gain = f.gain, rn2 = __fmul_rn(f.rn, f.rn);
   // ---- rows: a warp per band
   {
     const float kl = f.bkl, kh = f.bkh;
-    constexpr int BR = L::BR;
-    const int ra = 3 + warp * BR;
+    // iteration 1: bands of the rows of med3; later ones, with few tests, form med3 at the tests and take the
+    // rows of the bound test only, warp 7 meanwhile the pixels within 6 px of a change
+    constexpr int BR = kMode == 0 ? L::BR : (L::R2 + 6) / 7;
+    const int ra = (kMode == 0 ? 3 : 6) + warp * BR;
     bool work = true;
-    if (kMode == 1) {  // a change within 9 rows: 3 of the med3 windows and 6
-      const int rr = ra - 9 + lane;
-      work = __any_sync(0xffffffffu, lane < BR + 18 && rr >= 0 && rr < R && any2(mC[rr]));
+    if (kMode == 1) {
+      if (warp == 7) {
+        for (int r = lane; r < R; r += 32) {
+          uint2 z = make_uint2(0u, 0u);
+#pragma unroll
+          for (int d = -6; d <= 6; ++d)
+            if (r + d >= 0 && r + d < R) z = or2(z, mC[r + d]);
+          mF[r] = hdil6(z);
+        }
+        work = false;
+      } else {  // a change within 8 rows
+        const int rr = ra - 8 + lane;
+        work = __any_sync(0xffffffffu, lane < BR + 16 && rr >= 0 && rr < R && any2(mC[rr]));
+      }
     }
     if (work) {
       const uint2 cm = T.cols(2);
@@ -498,7 +526,7 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
       for (int j = 0; j < BR; ++j) {
         const int r = ra + j;
         const float2 up = v[j + 1], ce = v[j + 2], dn = v[j + 3];
-        {  // med3: as m3_kernel, from the sorted columns
+        if (kMode == 0) {  // med3: as m3_kernel, from the sorted columns
           float le, ne, he, lo, no, ho;
           sort3(up.x, ce.x, dn.x, le, ne, he);
           sort3(up.y, ce.y, dn.y, lo, no, ho);
@@ -535,7 +563,7 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
   __syncthreads();
 
   // ---- need: nsp = dilate5(hot) & act, needS = dilate5(nsp), as lists of pairs
-  if (T.edge) {  // med3 outside the frame: the value at the frame's edge
+  if (kMode == 0 && T.edge) {  // med3 outside the frame: the value at the frame's edge
     for (int i = tid; i < L::RB * 64; i += 256) {
       const int r = 3 + (i >> 6), c = i & 63;
       const int rr = clampi(r, T.r0, T.r1 - 1), cc = clampi(c, T.c0, T.c1 - 1);
@@ -598,7 +626,9 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
   }
   __syncthreads();
 
-  // ---- S' and the thresholds; the tests with their scale
+  // ---- S' and the thresholds; the tests with their scale. S' takes the first warps (few pairs): the others
+  // write the image meanwhile
+  if (kMode == 1 && warp >= 2) write_image(64);
   const float sigclip = p.sigclip, siglow = __fmul_rn(p.sigfrac, p.sigclip);
   for (int j = tid; j < nP; j += 256) {
     const int e = L1[j], r = e >> 7, c0 = ((e >> 2) & 31) * 2;
@@ -637,14 +667,36 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
     const int t = t0 + (lane >> 3), q = lane & 7;
     const bool on = t < nT;
     const int r = on ? L0[t] >> 6 : 8, c = on ? L0[t] & 63 : 8;
-    const float x = sN[r * kT2P + c], mc = sM3[r * kT2P + c];
+    const float x = sN[r * kT2P + c];
     const float xl = x * (1.f - 2e-6f), xh = x * (1.f + 2e-6f);
+    float v[7], mc;  // the window's row r-3+q of med3, and its centre
+    if (kMode == 0) {
+      const float* row = sM3 + (r - 3 + (q < 7 ? q : 0)) * kT2P + c - 3;
+#pragma unroll
+      for (int d = 0; d < 7; ++d) v[d] = row[d];
+      mc = sM3[r * kT2P + c];
+    } else {
+      if (!T.edge) {
+        const float* row = sJ + (r - 4 + (q < 7 ? q : 0)) * kT2P + c - 4;
+        float lo[9], mi[9], hi[9];
+#pragma unroll
+        for (int d = 0; d < 9; ++d) sort3(row[d], row[d + kT2P], row[d + 2 * kT2P], lo[d], mi[d], hi[d]);
+#pragma unroll
+        for (int d = 0; d < 7; ++d)
+          v[d] = med3f(max3f(lo[d], lo[d + 1], lo[d + 2]), med3f(mi[d], mi[d + 1], mi[d + 2]),
+                       min3f(hi[d], hi[d + 1], hi[d + 2]));
+      } else {
+#pragma unroll
+        for (int d = 0; d < 7; ++d)
+          v[d] = med3_at(sJ, clampi(r - 3 + (q < 7 ? q : 0), T.r0, T.r1 - 1), clampi(c - 3 + d, T.c0, T.c1 - 1));
+      }
+      mc = __shfl_sync(0xffffffffu, v[3], (lane & 24) | 3);
+    }
     int n = 0;  // values that pass; values that do not fail, in the upper half
     if (on && q < 7) {
-      const float* row = sM3 + (r - 3 + q) * kT2P + c - 3;
 #pragma unroll
       for (int d = 0; d < 7; ++d) {
-        const float fv = __fsub_rn(mc, row[d]);
+        const float fv = __fsub_rn(mc, v[d]);
         n += (fv < xl ? 1 : 0) + (fv <= xh ? 65536 : 0);
       }
     }
@@ -660,7 +712,9 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
       const float num = p.objlim_form == 1 ? __fmul_rn(2.f, s) : __fsub_rn(s, median25_at(sS, r, c, rl, rh, cl, ch));
       int m = 0;
       for (int i = 0; i < 49; ++i)
-        m += test_holds(p, __fsub_rn(mc, sM3[(r - 3 + i / 7) * kT2P + c - 3 + i % 7]), nn, num);
+        m += test_holds(p, __fsub_rn(mc, kMode == 0 ? sM3[(r - 3 + i / 7) * kT2P + c - 3 + i % 7]
+                                                     : med3_at(sJ, clampi(r - 3 + i / 7, rl, rh), clampi(c - 3 + i % 7, cl, ch))),
+                        nn, num);
       cand = m >= 25;
       if (f.work) atomicAdd(&cnt[7], 1);
     }
@@ -669,6 +723,10 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
   __syncthreads();
 
   // ---- both growths; M_k = M_{k-1} | g2
+  if (kMode == 0 && !nframes) {
+    pdl_wait();
+    pdl_launch();
+  }
   if (warp * 32 < TH) {
     const int r = 8 + tid;
     int fresh = 0;
@@ -697,7 +755,7 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
       atomicAdd(wk + 0, (unsigned long long)cnt[5]);
       atomicAdd(wk + 1, (unsigned long long)cnt[6]);
     }
-    atomicAdd(wk + 2, (unsigned long long)span(5));
+    atomicAdd(wk + 2, (unsigned long long)(kMode == 0 ? span(5) : 49ll * nT));
     if (nT) atomicAdd(wk + 3, (unsigned long long)nT);
     if (cnt[7]) atomicAdd(wk + 4, (unsigned long long)cnt[7]);
     atomicAdd(wk + 5, (unsigned long long)span(2));
