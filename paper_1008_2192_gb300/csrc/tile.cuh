@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
   uint2* mG = mLow + R;  // candidates
   uint16_t* L0 = reinterpret_cast<uint16_t*>(smem + L::oL0);
   uint16_t* L1 = reinterpret_cast<uint16_t*>(smem + L::oL1);
-  int* cnt = reinterpret_cast<int*>(smem + L::oCnt);  // 0 replacement, 1 S, 2 S', 3 tests, 4 full windows, 5.. work
+  int* cnt = reinterpret_cast<int*>(smem + L::oCnt);  // 0 replacement, 1 S and S', 3 tests, 4 full windows, 5.. work
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
   // the bit maps and counters; then the frame's descriptor, which in the later iterations does not depend
@@ -570,10 +570,11 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
       if (rr != r || cc != c) sM3[r * kT2P + c] = sM3[rr * kT2P + cc];
     }
   }
-  if (warp * 32 < L::RS) {
-    const int r = 4 + tid;
+  if (warp * 32 < 2 * L::RS) {  // two lanes per row, each listing half of its pairs
+    const int r = 4 + (tid >> 1);
+    const uint32_t half = (tid & 1) ? 0xffff0000u : 0x0000ffffu;
     uint2 hv[9], nsp = make_uint2(0u, 0u), need = nsp, mine = nsp;
-    if (tid < L::RS) {
+    if (tid < 2 * L::RS) {
 #pragma unroll
       for (int j = 0; j < 9; ++j)
         hv[j] = (r - 4 + j >= 6 && r - 4 + j < R - 6) ? mHot[r - 4 + j] : make_uint2(0u, 0u);
@@ -589,26 +590,27 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
       }
       if (T.row_in<TH>(r, 4)) need = and2(hdil2(nsp), T.cols(4));
     }
-    const uint32_t ps = need.x | need.y, pp = mine.x | mine.y;
-    int os = warp_reserve(__popc(ps), &cnt[1]), op = warp_reserve(__popc(pp), &cnt[2]);
+    const uint32_t ps = (need.x | need.y) & half, pp = (mine.x | mine.y) & half;
+    const int o = warp_reserve(__popc(ps) | __popc(pp) << 16, &cnt[1]);  // both lists at once, 16 bits each
+    int os = o & 0xffff, op = o >> 16;
     for (uint32_t v = ps; v; v &= v - 1u) L0[os++] = uint16_t((r << 6) | ((__ffs(v) - 1) << 1));
     for (uint32_t v = pp; v; v &= v - 1u) {
       const int b = __ffs(v) - 1;
       L1[op++] = uint16_t((r << 7) | (b << 2) | ((mine.x >> b) & 1u) | ((mine.y >> b) & 1u) << 1);
     }
     if (f.work) {
-      const int ns = __reduce_add_sync(0xffffffffu, unsigned(popc2(need)));
-      const int np = __reduce_add_sync(0xffffffffu, unsigned(popc2(mine)));
-      if (lane == 0 && ns) {
-        atomicAdd(&cnt[5], ns);
-        atomicAdd(&cnt[6], np);
+      const uint2 hm = make_uint2(half, half);
+      const int n = __reduce_add_sync(0xffffffffu, unsigned(popc2(and2(need, hm))) | unsigned(popc2(and2(mine, hm))) << 16);
+      if (lane == 0 && n) {
+        atomicAdd(&cnt[5], n & 0xffff);
+        atomicAdd(&cnt[6], n >> 16);
       }
     }
   }
   __syncthreads();
 
   // ---- S and N
-  const int nS = cnt[1], nP = cnt[2];
+  const int nS = cnt[1] & 0xffff, nP = cnt[1] >> 16;
   for (int j = tid; j < nS; j += 256) {
     const int r = L0[j] >> 6, c0 = L0[j] & 63;
     float v[5][6], m5[2];
