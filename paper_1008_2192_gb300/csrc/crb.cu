@@ -79,18 +79,21 @@ constexpr int kOneRoundShape = 5;
 struct TileKernels {
   int th;
   void (*fn[3])(const crb::Frame*, int, crb::Params, int, int, const crb::Frame);  // iteration 1, later ones, the last replacement
-  int smem;
+  int smem[3];
 };
-template <int TH>
+template <int TH, bool kMany>
 constexpr TileKernels make_tile() {
-  return TileKernels{TH, {crb::tile_kernel<TH, 0>, crb::tile_kernel<TH, 1>, crb::tile_kernel<TH, 2>},
-                     crb::TileLayout<TH>::bytes};
+  return TileKernels{TH,
+                     {crb::tile_kernel<TH, 0, false>, crb::tile_kernel<TH, 1, kMany>, crb::tile_kernel<TH, 2, false>},
+                     {crb::TileLayout<TH, 0>::bytes, crb::TileLayout<TH, 1>::bytes, crb::TileLayout<TH, 2>::bytes}};
 }
 // Tiles of 30 rows: the time of a call by height, 14 / 22 / 30 / 38 rows: 70 / 61 / 60 / 61 us on 800 x 800,
 // 299 / 238 / 213 / 219 us on 2048 x 2048 (fewer rows: more of them recomputed around the tile; 38: three
 // blocks per SM). Tiles of 14 rows where they number at most one per SM: a block's latency is all there is,
 // and fewer rows per warp shorten it (137 x 137: 41 / 43 / 47 / 50 us).
-const TileKernels kTileKernels[] = {make_tile<30>(), make_tile<14>()};
+// More tiles than one round of four blocks per SM: iterations 2 on at five blocks (1024 x 1024: 73.1 -> 67.1 us,
+// 2048 x 2048: 199 -> 187; 800 x 800, one round: 52.7 -> 53.6).
+const TileKernels kTileKernels[] = {make_tile<30, false>(), make_tile<14, false>(), make_tile<30, true>()};
 
 constexpr int kRW = 64, kRH = 16;  // replacement tile
 const ReplaceFn kReplace = crb::replace_kernel<kRW, kRH>;
@@ -278,9 +281,9 @@ int init_ctx(crb_ctx* c) {
     c->occ_fused.push_back(occf > 0 ? occf : 1);
   }
   for (const auto& t : kTileKernels)
-    for (auto fn : t.fn) {  // four blocks per SM need the largest shared-memory carveout
-      CRB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, t.smem));
-      CRB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+    for (int m = 0; m < 3; ++m) {  // the blocks per SM need the largest shared-memory carveout
+      CRB_CUDA(cudaFuncSetAttribute(t.fn[m], cudaFuncAttributeMaxDynamicSharedMemorySize, t.smem[m]));
+      CRB_CUDA(cudaFuncSetAttribute(t.fn[m], cudaFuncAttributePreferredSharedMemoryCarveout,
                                     int(cudaSharedmemCarveoutMaxShared)));
     }
   {
@@ -653,7 +656,7 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
     for (int k = 1; k <= P.niter + 1; ++k) {
       const int mode = k == 1 ? 0 : k <= P.niter ? 1 : 2;
       timed(c, mode == 2 ? kPTileReplace : kPTileDetect, stream, [&] {
-        launch_pdl(t.fn[mode], unsigned(P.tiles), 256, t.smem, stream, c->d_frames, k == 1 && P.one ? 0 : P.n, c->p, k, P.niter,
+        launch_pdl(t.fn[mode], unsigned(P.tiles), 256, t.smem[mode], stream, c->d_frames, k == 1 && P.one ? 0 : P.n, c->p, k, P.niter,
                    c->h_frames[0]);
       });
     }
@@ -937,9 +940,12 @@ int prepare_tile(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pla
   auto tiles_of = [&](const FrameSpec& s, int h) {
     return (long long)((s.w + crb::kT2W - 1) / crb::kT2W) * ((s.h + h - 1) / h);
   };
-  long long small = 0;
-  for (const auto& s : specs) small += tiles_of(s, kTileKernels[1].th);
-  const int v = small <= c->num_sms ? 1 : 0;
+  long long low = 0, high = 0;
+  for (const auto& s : specs) {
+    high += tiles_of(s, kTileKernels[0].th);
+    low += tiles_of(s, kTileKernels[1].th);
+  }
+  const int v = low <= c->num_sms ? 1 : high > 4LL * c->num_sms ? 2 : 0;
   const int th = kTileKernels[v].th;
   char* pb = static_cast<char*>(c->ws);
   char* pi = pb + bits;

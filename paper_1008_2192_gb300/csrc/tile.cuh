@@ -43,26 +43,30 @@ constexpr int kT2P = 68;  // row pitch in shared memory: rows of a column fall o
 // words per bit stream of a plane row
 __host__ __device__ inline int tile_wps(int w) { return ((w + 1) / 2 + 31) / 32; }
 
-template <int TH>
+// kMode as tile_kernel: iteration 1 keeps med3, the later ones the image region and the maps of S and N (whose
+// place the replacement values take before), the last replacement the image region and those values.
+// 53, 42 and 24 KB: 4, 5 and 6 blocks per SM, the second at 48 registers with 40 B of spills (kMany), the third at
+// 40. Calls whose tiles take one round of blocks keep 64 registers and 4 blocks in mode 1.
+template <int TH, int kMode>
 struct TileLayout {
   static constexpr int R = TH + 16;   // rows of the image region
-  static constexpr int RB = TH + 10;  // rows of the row stage (med3: the tile and 5 rows each side)
+  static constexpr int RB = TH + 10;  // rows of med3: the tile and 5 rows each side
   static constexpr int BR = RB / 8;   // rows per warp
   static_assert(RB % 8 == 0 && R <= 64 && TH >= 8, "whole bands of rows, 6-bit rows in list entries");
   static constexpr int RS = TH + 8;   // rows of S
   static constexpr int R2 = TH + 4;   // rows of S' and N
+  static constexpr int kListR = kMode == 2 ? TH * kT2W : (TH + 12) * 60;  // flagged pixels to replace at most
   static constexpr int oJ = 0;
   static constexpr int oS = oJ + R * kT2P;
-  static constexpr int oN = oS + RS * kT2P;
-  static constexpr int oM3 = oN + R2 * kT2P;
-  static constexpr int nF = oM3 + RB * kT2P;
-  static constexpr int kListR = (TH + 12) * 60;  // flagged pixels to replace: values over the S and N maps
-  static_assert(kListR <= (RS + R2) * kT2P, "replacement values fit in the S and N maps");
-  static constexpr int kListS = imax(RS * 28, (kListR + 1) / 2 * 2);  // pairs of S; or the replacement list
-  static constexpr int kListP = R2 * 26;  // pairs of S'
-  static_assert(R2 * 52 <= kListS, "the tests take the place of the pairs of S");
-  static constexpr int oMask = nF * 4;    // bytes: 8 bit maps of R rows x 2 words
-  static constexpr int oL0 = oMask + 8 * R * 8;
+  static constexpr int oN = oS + (kMode == 2 ? 0 : RS * kT2P);
+  static constexpr int oM3 = oN + (kMode == 2 ? kListR : R2 * kT2P);
+  static_assert(oS + kListR <= oM3, "replacement values fit in the S and N maps");
+  static constexpr int nF = oM3 + (kMode == 0 ? RB * kT2P : 0);
+  static constexpr int kListS = kMode == 2 ? kListR : imax(RS * 28, (kListR + 1) / 2 * 2);  // pairs of S; or the replacement list
+  static constexpr int kListP = kMode == 2 ? 0 : R2 * 26;                                   // pairs of S'
+  static_assert(kMode == 2 || R2 * 52 <= kListS, "the tests take the place of the pairs of S");
+  static constexpr int oMask = nF * 4;  // bytes: bit maps of R rows x 2 words (mode 2: M and its new flags)
+  static constexpr int oL0 = round16(oMask + (kMode == 2 ? 2 : 8) * R * 8);
   static constexpr int oL1 = oL0 + round16(kListS * 2);
   static constexpr int oCnt = oL1 + round16(kListP * 2);
   static constexpr int bytes = oCnt + 64;
@@ -224,10 +228,10 @@ __device__ __forceinline__ bool test_holds(const Params& p, float fval, float nn
 // input, while the launch ahead ends.
 // kMode 0: iteration 1. 1: the replacement of iteration k-1, then iteration k.
 // 2: the replacement of iteration niter (k = niter + 1) and the u8 mask.
-template <int TH, int kMode>
-__global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ frames, int nframes, Params p, int k,
+template <int TH, int kMode, bool kMany>
+__global__ void __launch_bounds__(256, kMode == 1 && !kMany ? 4 : 4 + kMode) tile_kernel(const Frame* __restrict__ frames, int nframes, Params p, int k,
                                                       int niter, const __grid_constant__ Frame one) {
-  using L = TileLayout<TH>;
+  using L = TileLayout<TH, kMode>;
   constexpr int R = L::R;
   extern __shared__ __align__(128) char smem[];
   float* sJ = reinterpret_cast<float*>(smem) + L::oJ;             // rows 0 .. R-1
@@ -250,7 +254,7 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
 
   // the bit maps and counters; then the frame's descriptor, which in the later iterations does not depend
   // on the kernel before this one (pdl_wait)
-  for (int i = tid; i < 6 * R; i += 256) mC[i] = make_uint2(0u, 0u);
+  for (int i = tid; i < (kMode == 2 ? 0 : 6 * R); i += 256) mC[i] = make_uint2(0u, 0u);
   if (tid < 16) cnt[tid] = 0;
   if (kMode == 0 && nframes) {
     pdl_wait();
@@ -415,7 +419,7 @@ __global__ void __launch_bounds__(256, 4) tile_kernel(const Frame* __restrict__ 
       }
       float out = sel_med25(v);
       if (n == 0) out = floor_m5(out);
-      if (__float_as_uint(out) != __float_as_uint(sJ[r * kT2P + c])) {
+      if (kMode == 1 && __float_as_uint(out) != __float_as_uint(sJ[r * kT2P + c])) {
         changed = true;
         set_bit2(&mC[r], c);
       }
