@@ -299,10 +299,11 @@ __global__ void __launch_bounds__(256, kMode == 1 && !kMany ? 4 : 4 + kMode) til
         }
       }
     } else {
-      for (int i = tid; i < (rb - ra) * 64; i += 256) {
-        const int r = ra + (i >> 6), c = i & 63;
-        cp_async4(sJ + r * kT2P + c,
-                  src + size_t(clampi(T.y0 - 8 + r, 0, h - 1)) * w + clampi(T.x0 - 8 + c, 0, w - 1));
+      const int ca = clampi(T.x0 - 8 + lane, 0, w - 1), cb = clampi(T.x0 + 24 + lane, 0, w - 1);
+      for (int r = ra + warp; r < rb; r += 8) {  // a row per warp
+        const float* row = src + size_t(clampi(T.y0 - 8 + r, 0, h - 1)) * w;
+        cp_async4(sJ + r * kT2P + lane, row + ca);
+        cp_async4(sJ + r * kT2P + lane + 32, row + cb);
       }
     }
     cp_async_commit();
@@ -364,9 +365,10 @@ __global__ void __launch_bounds__(256, kMode == 1 && !kMany ? 4 : 4 + kMode) til
                 *reinterpret_cast<const float4*>(sJ + r * kT2P + c);
         }
       } else {
-        for (int i = tid - first; i < TH * kT2W; i += 256 - first) {
-          const int r = 8 + i / kT2W, c = 8 + i % kT2W;
-          if (r < T.r1 && c < T.c1) dst[size_t(T.y0 - 8 + r) * w + T.x0 - 8 + c] = sJ[r * kT2P + c];
+        for (int r = 8 + (tid - first) / 32; r < min(8 + TH, T.r1); r += (256 - first) / 32) {  // a row per warp
+          float* row = dst + size_t(T.y0 - 8 + r) * w + T.x0 - 8;
+          if (8 + lane < T.c1) row[8 + lane] = sJ[r * kT2P + 8 + lane];
+          if (lane < kT2W - 32 && 40 + lane < T.c1) row[40 + lane] = sJ[r * kT2P + 40 + lane];
         }
       }
     } else if (tid - first < 2 * TH) {  // a thread per row and parity
@@ -452,12 +454,11 @@ __global__ void __launch_bounds__(256, kMode == 1 && !kMany ? 4 : 4 + kMode) til
           *reinterpret_cast<uint4*>(om + size_t(T.y0 - 8 + r) * w + T.x0 - 8 + c) = make_uint4(q[0], q[1], q[2], q[3]);
         }
       } else {
-        for (int i = tid; i < TH * kT2W; i += 256) {
-          const int r = 8 + i / kT2W, c = 8 + i % kT2W;
-          if (r < T.r1 && c < T.c1) {
-            const uint2 m = mM[r];
-            om[size_t(T.y0 - 8 + r) * w + T.x0 - 8 + c] = uint8_t((((c & 1) ? m.y : m.x) >> (c >> 1)) & 1u);
-          }
+        for (int r = 8 + warp; r < min(8 + TH, T.r1); r += 8) {  // a row per warp
+          uint8_t* row = om + size_t(T.y0 - 8 + r) * w + T.x0 - 8;
+          const uint32_t m = (lane & 1) ? mM[r].y : mM[r].x;
+          if (8 + lane < T.c1) row[8 + lane] = uint8_t((m >> (4 + (lane >> 1))) & 1u);
+          if (lane < kT2W - 32 && 40 + lane < T.c1) row[40 + lane] = uint8_t((m >> (20 + (lane >> 1))) & 1u);
         }
       }
       return;
