@@ -72,22 +72,24 @@ constexpr int kTabShift = 16;  // pixels per entry of the frame table: 2^kTabShi
 
 // queue counters (Queues::n)
 enum : int {
-  kNS = 0,      // QS (word entries)
-  kNSP = 1,     // QSP (word entries)
-  kNM3 = 2,     // QM3 (word entries)
-  kNT = 3,      // QT (word entries)
-  kNRep = 4,    // replacement queue
-  kNFresh = 5,  // new flags of this iteration
-  kNFb = 6,     // pixels with a fully flagged window (kept over the iterations)
-  kNReserved = 7,  // (not used)
-  kNPass = 8,   // candidates (passed the objlim test)
-  kNAmb = 9,    // tests the column-median bounds leave open
-  kNSpx = 10,   // positions in QS, QSP, QM3, QT (work counters)
-  kNSPpx = 11,
-  kNM3px = 12,
-  kNTpx = 13,
-  kNB = 14,     // pixels to re-test in the bound pass (word entries)
-  kNBpx = 15,
+  // word entries of a queue and, in the next counter, the positions they list (work counters): one 64-bit
+  // atomic adds both
+  kNS = 0,      // QS
+  kNSpx = 1,
+  kNSP = 2,     // QSP
+  kNSPpx = 3,
+  kNM3 = 4,     // QM3
+  kNM3px = 5,
+  kNT = 6,      // QT
+  kNTpx = 7,
+  kNB = 8,      // pixels to re-test in the bound pass
+  kNBpx = 9,
+  kNRep = 10,   // replacement queue (pixels; its second counter is not used)
+  kNRep2 = 11,
+  kNPass = 12,  // candidates (passed the objlim test)
+  kNAmb = 13,   // tests the column-median bounds leave open
+  kNFresh = 14, // new flags of this iteration
+  kNFb = 15,    // pixels with a fully flagged window (kept over the iterations)
   kNSeg = 16,   // segments (1 word x kSH rows) listed for m3need_seg_kernel,
   kNSegN = 17,  // for need_seg_kernel,
   kNSegD = 18,  // for d2_seg_kernel (the three in Queues::seg order)
@@ -463,21 +465,46 @@ __device__ __forceinline__ void col_write(const ColWords& sw, int warp, int j, u
   }
 }
 
-// Reserves the strip's entries and positions of two queues (counters ne[0..1],
-// np[0..1]); returns the entry bases to every lane.
-__device__ __forceinline__ void col_reserve(const unsigned int (&ents)[2], const unsigned int (&pix)[2],
-                                            unsigned int* ne0, unsigned int* ne1, unsigned int* np0,
-                                            unsigned int* np1, unsigned int (&base)[2]) {
-  const int lane = threadIdx.x & 31;
-  unsigned int b0 = 0, b1 = 0;
-  if (lane == 0) {
-    if (ents[0]) b0 = atomicAdd(ne0, ents[0]);
-    if (ents[1]) b1 = atomicAdd(ne1, ents[1]);
-    if (pix[0]) atomicAdd(np0, pix[0]);
-    if (pix[1]) atomicAdd(np1, pix[1]);
+// Reserves the entries and positions of two queues (counter pairs at c0, c1) for
+// the block's NW warps: each warp's bases. One atomic per block and queue: the
+// queues' counters lie in one line, where an atomic takes about 1.7 ns: with two per
+// warp and queue, m3need in iteration 1 of 430 Mpix took 80 us (52,000 atomics) against
+// 44, d2 84 against 64, a whole 16384 x 16384 clean 4558 against 4468. Every thread of the
+// block calls it.
+template <int NW>
+struct Totals {
+  unsigned int e[NW][2], p[NW][2], base[2], sum[2];
+};
+
+template <int NW>
+__device__ __forceinline__ void block_reserve(Totals<NW>& T, const unsigned int (&ents)[2], const unsigned int (&pix)[2],
+                                              unsigned int* c0, unsigned int* c1, unsigned int (&base)[2]) {
+  static_assert(NW >= 2 && NW <= 32, "a warp per queue");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane < 2) {
+    T.e[warp][lane] = lane ? ents[1] : ents[0];
+    T.p[warp][lane] = lane ? pix[1] : pix[0];
   }
-  base[0] = __shfl_sync(0xffffffffu, b0, 0);
-  base[1] = __shfl_sync(0xffffffffu, b1, 0);
+  __syncthreads();
+  unsigned int before[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const unsigned int e = lane < NW ? T.e[lane][j] : 0u;
+    before[j] = __reduce_add_sync(0xffffffffu, lane < warp ? e : 0u);
+    if (warp == j) {
+      const unsigned int n = __reduce_add_sync(0xffffffffu, e);
+      const unsigned int px = __reduce_add_sync(0xffffffffu, lane < NW ? T.p[lane][j] : 0u);
+      if (lane == 0) {
+        unsigned int b = 0;
+        if (n) b = (unsigned int)atomicAdd(reinterpret_cast<unsigned long long*>(j ? c1 : c0), n | (unsigned long long)px << 32);
+        T.base[j] = b;
+        T.sum[j] = n;
+      }
+    }
+  }
+  __syncthreads();
+  base[0] = T.base[0] + before[0];
+  base[1] = T.base[1] + before[1];
 }
 
 // Whether this lane's word (and halo word) has a cell of class >= 2 among the
@@ -506,8 +533,10 @@ __global__ void __launch_bounds__(kColWarps * 32) need_kernel(const Frame* __res
   pdl_wait();
   pdl_launch();
   __shared__ ColWords sw;
+  __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (long long u = (long long)blockIdx.x * kColWarps + warp; u < nunits; u += (long long)gridDim.x * kColWarps) {
+  for (long long ub = (long long)blockIdx.x * kColWarps; ub < nunits; ub += (long long)gridDim.x * kColWarps) {  // whole blocks
+    const long long u = min(ub + warp, nunits - 1);
     const Frame& f = frames[frame_of_unit(frames, nframes, u)];
     const long long lu = u - f.u0;
     const int uy = int(lu / f.ugx), ux = int(lu - (long long)uy * f.ugx);
@@ -516,7 +545,7 @@ __global__ void __launch_bounds__(kColWarps * 32) need_kernel(const Frame* __res
     const int hw = lane == 0 ? wc0 - 1 : wc0 + 32;  // halo word (lanes 0 and 31)
     const bool hin = (lane == 0 || lane == 31) && hw >= 0 && hw < f.wpr;
     const uint32_t fmask = inw ? frame_word(wc, f.w) : 0u;
-    if (cls && !__any_sync(0xffffffffu, strip_has_class2(cls, f, wc, inw, -1, false, y0, 0))) continue;
+    const bool on = ub + warp < nunits && !(cls && !__any_sync(0xffffffffu, strip_has_class2(cls, f, wc, inw, -1, false, y0, 0)));
     uint32_t h0 = 0, h1 = 0, h2 = 0, h3 = 0, h4 = 0;  // own hot, rows r-4 .. r
     uint32_t g0 = 0, g1 = 0, g2 = 0, g3 = 0, g4 = 0;  // halo hot
     uint32_t a0 = 0, a1 = 0, a2 = 0, b0 = 0, b1 = 0, b2 = 0;  // act, rows r-2 .. r (own, halo)
@@ -525,7 +554,7 @@ __global__ void __launch_bounds__(kColWarps * 32) need_kernel(const Frame* __res
     unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
     // rows y0-4 .. y0+kSH+3 in chunks of kColChunk: the chunk's loads are issued together
     static_assert((kSH + 8) % kColChunk == 0, "whole chunks");
-    for (int rc = y0 - 4; rc < y0 + kSH + 4; rc += kColChunk) {
+    for (int rc = y0 - 4; on && rc < y0 + kSH + 4; rc += kColChunk) {
       uint32_t Lh[kColChunk], La[kColChunk], Lgh[kColChunk], Lga[kColChunk], Lc[kColChunk], Ls[kColChunk],
           Lz[kColChunk];
 #pragma unroll
@@ -588,10 +617,10 @@ __global__ void __launch_bounds__(kColWarps * 32) need_kernel(const Frame* __res
       }
     }
     unsigned int base[2];
-    col_reserve(ents, pix, Q.n + kNS, Q.n + kNSP, Q.n + kNSpx, Q.n + kNSPpx, base);
+    block_reserve(tot, ents, pix, Q.n + kNS, Q.n + kNSP, base);
     __syncwarp();
-    col_write(sw, warp, 0, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
-    col_write(sw, warp, 1, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[1], reinterpret_cast<uint2*>(Q.q1));
+    if (on) col_write(sw, warp, 0, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
+    if (on) col_write(sw, warp, 1, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[1], reinterpret_cast<uint2*>(Q.q1));
     __syncwarp();  // the shared words are refilled for the next strip
   }
 }
@@ -610,8 +639,10 @@ __global__ void __launch_bounds__(kColWarps * 32) m3need_kernel(const Frame* __r
   pdl_launch();
   const uint32_t* __restrict__ cls = kAll ? nullptr : cls_in;
   __shared__ ColWords sw;
+  __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (long long u = (long long)blockIdx.x * kColWarps + warp; u < nunits; u += (long long)gridDim.x * kColWarps) {
+  for (long long ub = (long long)blockIdx.x * kColWarps; ub < nunits; ub += (long long)gridDim.x * kColWarps) {  // whole blocks
+    const long long u = min(ub + warp, nunits - 1);
     const Frame& f = frames[frame_of_unit(frames, nframes, u)];
     const long long lu = u - f.u0;
     const int uy = int(lu / f.ugx), ux = int(lu - (long long)uy * f.ugx);
@@ -620,25 +651,25 @@ __global__ void __launch_bounds__(kColWarps * 32) m3need_kernel(const Frame* __r
     const int hw = lane == 0 ? wc0 - 1 : wc0 + 32;
     const bool hin = (lane == 0 || lane == 31) && hw >= 0 && hw < f.wpr;
     const uint32_t fmask = inw ? frame_word(wc, f.w) : 0u;
-    if (cls && !__any_sync(0xffffffffu, strip_has_class2(cls, f, wc, inw, hw, hin, y0, 1))) continue;
+    const bool on = ub + warp < nunits && !(cls && !__any_sync(0xffffffffu, strip_has_class2(cls, f, wc, inw, hw, hin, y0, 1)));
     if constexpr (kAll) {
       // iteration 1: the dense bound pass wrote M3 everywhere, so M3 is current on the whole frame and
       // nothing is queued for m3; QT = the test words
       unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
       uint32_t tq[kSH];
 #pragma unroll
-      for (int t = 0; t < kSH; ++t) tq[t] = (inw && y0 + t < f.h) ? f.test[size_t(y0 + t) * f.wpr + wc] : 0u;
+      for (int t = 0; t < kSH; ++t) tq[t] = (on && inw && y0 + t < f.h) ? f.test[size_t(y0 + t) * f.wpr + wc] : 0u;
 #pragma unroll
       for (int t = 0; t < kSH; ++t) {
-        if (inw && y0 + t < f.h) f.m3val[size_t(y0 + t) * f.wpr + wc] = fmask;
+        if (on && inw && y0 + t < f.h) f.m3val[size_t(y0 + t) * f.wpr + wc] = fmask;
         sw.w[warp][t][0][lane] = 0u;
         sw.w[warp][t][1][lane] = tq[t];
         col_count(tq[t], ents[1], pix[1]);
       }
       unsigned int base[2];
-      col_reserve(ents, pix, Q.n + kNM3, Q.n + kNT, Q.n + kNM3px, Q.n + kNTpx, base);
+      block_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, base);
       __syncwarp();
-      col_write(sw, warp, 1, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[1],
+      if (on) col_write(sw, warp, 1, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[1],
                 reinterpret_cast<uint2*>(Q.q2));
       __syncwarp();
       continue;
@@ -647,7 +678,7 @@ __global__ void __launch_bounds__(kColWarps * 32) m3need_kernel(const Frame* __r
     uint32_t s0 = 0, s1 = 0, s2 = 0, s3 = 0, s4 = 0, s5 = 0, s6 = 0;  // halo QT words
     unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
     // rows y0-3 .. y0+kSH+2 in chunks of kColChunk (the last chunk runs past the end)
-    for (int rc = y0 - 3; rc < y0 + kSH + 3; rc += kColChunk) {
+    for (int rc = y0 - 3; on && rc < y0 + kSH + 3; rc += kColChunk) {
       uint32_t Lq[kColChunk], Lg[kColChunk], Lm[kColChunk], Lc4[kColChunk];
 #pragma unroll
       for (int i = 0; i < kColChunk; ++i) {
@@ -689,10 +720,10 @@ __global__ void __launch_bounds__(kColWarps * 32) m3need_kernel(const Frame* __r
       }
     }
     unsigned int base[2];
-    col_reserve(ents, pix, Q.n + kNM3, Q.n + kNT, Q.n + kNM3px, Q.n + kNTpx, base);
+    block_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, base);
     __syncwarp();
-    col_write(sw, warp, 0, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
-    col_write(sw, warp, 1, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[1], reinterpret_cast<uint2*>(Q.q2));
+    if (on) col_write(sw, warp, 0, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
+    if (on) col_write(sw, warp, 1, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[1], reinterpret_cast<uint2*>(Q.q2));
     __syncwarp();
   }
 }
@@ -706,8 +737,10 @@ __global__ void __launch_bounds__(kColWarps * 32) d2_kernel(const Frame* __restr
   pdl_wait();
   pdl_launch();
   __shared__ ColWords sw;
+  __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (long long u = (long long)blockIdx.x * kColWarps + warp; u < nunits; u += (long long)gridDim.x * kColWarps) {
+  for (long long ub = (long long)blockIdx.x * kColWarps; ub < nunits; ub += (long long)gridDim.x * kColWarps) {  // whole blocks
+    const long long u = min(ub + warp, nunits - 1);
     const Frame& f = frames[frame_of_unit(frames, nframes, u)];
     const uint32_t* __restrict__ chg = f.chg[k & 1];
     const long long lu = u - f.u0;
@@ -717,9 +750,10 @@ __global__ void __launch_bounds__(kColWarps * 32) d2_kernel(const Frame* __restr
     const int hw = lane == 0 ? wc0 - 1 : wc0 + 32;
     const bool hin = (lane == 0 || lane == 31) && hw >= 0 && hw < f.wpr;
     const uint32_t fmask = inw ? frame_word(wc, f.w) : 0u;
+    const bool on = ub + warp < nunits;
     uint32_t c0 = 0, c1 = 0, c2 = 0, c3 = 0, c4 = 0, e0 = 0, e1 = 0, e2 = 0, e3 = 0, e4 = 0;
     unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
-    for (int rc = y0 - 2; rc < y0 + kSH + 2; rc += kColChunk) {  // the last chunk may run past the end
+    for (int rc = y0 - 2; on && rc < y0 + kSH + 2; rc += kColChunk) {  // the last chunk may run past the end
       uint32_t L[kColChunk], G[kColChunk];
 #pragma unroll
       for (int i = 0; i < kColChunk; ++i) {
@@ -746,9 +780,9 @@ __global__ void __launch_bounds__(kColWarps * 32) d2_kernel(const Frame* __restr
       }
     }
     unsigned int base[2];
-    col_reserve(ents, pix, Q.n + kNB, Q.n + kNB, Q.n + kNBpx, Q.n + kNBpx, base);
+    block_reserve(tot, ents, pix, Q.n + kNB, Q.n + kNB, base);
     __syncwarp();
-    col_write(sw, warp, 0, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[0], reinterpret_cast<uint2*>(Q.q2));
+    if (on) col_write(sw, warp, 0, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[0], reinterpret_cast<uint2*>(Q.q2));
     __syncwarp();
   }
 }
@@ -850,9 +884,12 @@ __global__ void __launch_bounds__(kColWarps * 32) d2_seg_kernel(const Frame* __r
   pdl_wait();
   pdl_launch();
   __shared__ ColWords sw;
+  __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned int nseg = Q.n[kNSegD];
-  for (unsigned int b = (blockIdx.x * kColWarps + warp) * 32u; b < nseg; b += gridDim.x * kColWarps * 32u) {
+  for (unsigned int bb = blockIdx.x * kColWarps * 32u; bb < nseg; bb += gridDim.x * kColWarps * 32u) {  // whole blocks
+    const bool on = bb + warp * 32u < nseg;
+    const unsigned int b = on ? bb + warp * 32u : bb;
     const SegLane S = seg_lane(frames, nframes, Q.seg[2], b, nseg);
     const Frame& f = *S.f;
     const int wc = S.wc, y0 = S.y0, wpr = S.wpr, h = S.h;
@@ -862,7 +899,7 @@ __global__ void __launch_bounds__(kColWarps * 32) d2_seg_kernel(const Frame* __r
     uint32_t cc0 = 0, cc1 = 0, cc2 = 0, cc3 = 0, cc4 = 0;
     uint32_t cr0 = 0, cr1 = 0, cr2 = 0, cr3 = 0, cr4 = 0;
     unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
-    for (int tc = -2; tc < kSH + 2; tc += 8) {  // rows y0-2 .. y0+kSH+1 (the last chunk runs past them)
+    for (int tc = -2; on && tc < kSH + 2; tc += 8) {  // rows y0-2 .. y0+kSH+1 (the last chunk runs past them)
       uint32_t L[8], C[8], R[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
@@ -887,9 +924,9 @@ __global__ void __launch_bounds__(kColWarps * 32) d2_seg_kernel(const Frame* __r
       }
     }
     unsigned int base[2];
-    col_reserve(ents, pix, Q.n + kNB, Q.n + kNB, Q.n + kNBpx, Q.n + kNBpx, base);
+    block_reserve(tot, ents, pix, Q.n + kNB, Q.n + kNB, base);
     __syncwarp();
-    col_write(sw, warp, 0, S.gw0, wpr, base[0], reinterpret_cast<uint2*>(Q.q2));
+    if (on) col_write(sw, warp, 0, S.gw0, wpr, base[0], reinterpret_cast<uint2*>(Q.q2));
     __syncwarp();
   }
 }
@@ -900,9 +937,12 @@ __global__ void __launch_bounds__(kColWarps * 32) need_seg_kernel(const Frame* _
   pdl_wait();
   pdl_launch();
   __shared__ ColWords sw;
+  __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned int nseg = Q.n[kNSegN];
-  for (unsigned int b = (blockIdx.x * kColWarps + warp) * 32u; b < nseg; b += gridDim.x * kColWarps * 32u) {
+  for (unsigned int bb = blockIdx.x * kColWarps * 32u; bb < nseg; bb += gridDim.x * kColWarps * 32u) {  // whole blocks
+    const bool on = bb + warp * 32u < nseg;
+    const unsigned int b = on ? bb + warp * 32u : bb;
     const SegLane S = seg_lane(frames, nframes, Q.seg[1], b, nseg);
     const Frame& f = *S.f;
     const int wc = S.wc, y0 = S.y0, wpr = S.wpr, h = S.h;
@@ -915,7 +955,7 @@ __global__ void __launch_bounds__(kColWarps * 32) need_seg_kernel(const Frame* _
     uint32_t nl[5] = {}, nc[5] = {}, nr[5] = {};  // nsp, rows r-6 .. r-2
     unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
     constexpr int kC = 4;  // rows per chunk of loads
-    for (int tc = -4; tc < kSH + 4; tc += kC) {  // rows y0-4 .. y0+kSH+3
+    for (int tc = -4; on && tc < kSH + 4; tc += kC) {  // rows y0-4 .. y0+kSH+3
       uint32_t Hl[kC], Hc[kC], Hr[kC], Al[kC], Ac[kC], Ar[kC], Cl[kC], Sv[kC], Lz[kC];
 #pragma unroll
       for (int i = 0; i < kC; ++i) {
@@ -978,10 +1018,10 @@ __global__ void __launch_bounds__(kColWarps * 32) need_seg_kernel(const Frame* _
       }
     }
     unsigned int base[2];
-    col_reserve(ents, pix, Q.n + kNS, Q.n + kNSP, Q.n + kNSpx, Q.n + kNSPpx, base);
+    block_reserve(tot, ents, pix, Q.n + kNS, Q.n + kNSP, base);
     __syncwarp();
-    col_write(sw, warp, 0, S.gw0, wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
-    col_write(sw, warp, 1, S.gw0, wpr, base[1], reinterpret_cast<uint2*>(Q.q1));
+    if (on) col_write(sw, warp, 0, S.gw0, wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
+    if (on) col_write(sw, warp, 1, S.gw0, wpr, base[1], reinterpret_cast<uint2*>(Q.q1));
     __syncwarp();
   }
 }
@@ -992,9 +1032,12 @@ __global__ void __launch_bounds__(kColWarps * 32) m3need_seg_kernel(const Frame*
   pdl_wait();
   pdl_launch();
   __shared__ ColWords sw;
+  __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned int nseg = Q.n[kNSeg];
-  for (unsigned int b = (blockIdx.x * kColWarps + warp) * 32u; b < nseg; b += gridDim.x * kColWarps * 32u) {
+  for (unsigned int bb = blockIdx.x * kColWarps * 32u; bb < nseg; bb += gridDim.x * kColWarps * 32u) {  // whole blocks
+    const bool on = bb + warp * 32u < nseg;
+    const unsigned int b = on ? bb + warp * 32u : bb;
     const SegLane S = seg_lane(frames, nframes, Q.seg[0], b, nseg);
     const Frame& f = *S.f;
     const int wc = S.wc, y0 = S.y0, wpr = S.wpr, h = S.h;
@@ -1003,7 +1046,7 @@ __global__ void __launch_bounds__(kColWarps * 32) m3need_seg_kernel(const Frame*
     const long long cb = f.cell0 + wc;
     uint32_t ql[7] = {}, qc[7] = {}, qr[7] = {};  // QT, rows r-6 .. r: left, own, right words
     unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
-    for (int tc = -3; tc < kSH + 3; tc += 8) {  // rows y0-3 .. y0+kSH+2 (the last chunk runs past them)
+    for (int tc = -3; on && tc < kSH + 3; tc += 8) {  // rows y0-3 .. y0+kSH+2 (the last chunk runs past them)
       uint32_t Ql[8], Qc[8], Qr[8], Lm[8], Lc4[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
@@ -1047,10 +1090,10 @@ __global__ void __launch_bounds__(kColWarps * 32) m3need_seg_kernel(const Frame*
       }
     }
     unsigned int base[2];
-    col_reserve(ents, pix, Q.n + kNM3, Q.n + kNT, Q.n + kNM3px, Q.n + kNTpx, base);
+    block_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, base);
     __syncwarp();
-    col_write(sw, warp, 0, S.gw0, wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
-    col_write(sw, warp, 1, S.gw0, wpr, base[1], reinterpret_cast<uint2*>(Q.q2));
+    if (on) col_write(sw, warp, 0, S.gw0, wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
+    if (on) col_write(sw, warp, 1, S.gw0, wpr, base[1], reinterpret_cast<uint2*>(Q.q2));
     __syncwarp();
   }
 }
@@ -1066,40 +1109,6 @@ __global__ void __launch_bounds__(kColWarps * 32) m3need_seg_kernel(const Frame*
 
 constexpr int kRowWarps = kSH / 2;
 static_assert(kRowWarps == 8, "256 threads: two rows of a strip per warp");
-
-// One value per warp and queue -> exclusive prefix over the block's warps, the total appended to the queue's
-// counter. Every thread calls it.
-struct RowTotals {
-  unsigned int e[kRowWarps][2], p[kRowWarps][2], base[2];
-};
-
-__device__ __forceinline__ void rows_reserve(RowTotals& T, const unsigned int (&ents)[2], const unsigned int (&pix)[2],
-                                             unsigned int* ne0, unsigned int* ne1, unsigned int* np0,
-                                             unsigned int* np1, unsigned int (&base)[2]) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane < 2) {
-    T.e[warp][lane] = lane ? ents[1] : ents[0];
-    T.p[warp][lane] = lane ? pix[1] : pix[0];
-  }
-  __syncthreads();
-  unsigned int before[2];
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const unsigned int e = lane < kRowWarps ? T.e[lane][j] : 0u;
-    before[j] = __reduce_add_sync(0xffffffffu, lane < warp ? e : 0u);
-    if (warp == j) {
-      const unsigned int n = __reduce_add_sync(0xffffffffu, e);
-      const unsigned int px = __reduce_add_sync(0xffffffffu, lane < kRowWarps ? T.p[lane][j] : 0u);
-      if (lane == 0) {
-        T.base[j] = n ? atomicAdd(j ? ne1 : ne0, n) : 0u;
-        if (px) atomicAdd(j ? np1 : np0, px);
-      }
-    }
-  }
-  __syncthreads();
-  base[0] = T.base[0] + before[0];
-  base[1] = T.base[1] + before[1];
-}
 
 // Writes the nonzero words of a warp as entries: word v of each lane is global word gw.
 __device__ __forceinline__ void row_write(uint32_t v, uint32_t gw, unsigned int& base, uint2* q) {
@@ -1170,7 +1179,7 @@ __global__ void __launch_bounds__(256) need_row_kernel(const Frame* __restrict__
                                                        Queues Q, const uint32_t* __restrict__ cls) {
   pdl_wait();
   pdl_launch();
-  __shared__ RowTotals tot;
+  __shared__ Totals<kRowWarps> tot;
   for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
     const RowLane L = row_lane(frames, nframes, u);
     const Frame& f = *L.f;
@@ -1217,7 +1226,7 @@ __global__ void __launch_bounds__(256) need_row_kernel(const Frame* __restrict__
       col_count(qsp[j], ents[1], pix[1]);
     }
     unsigned int base[2];
-    rows_reserve(tot, ents, pix, Q.n + kNS, Q.n + kNSP, Q.n + kNSpx, Q.n + kNSPpx, base);
+    block_reserve(tot, ents, pix, Q.n + kNS, Q.n + kNSP, base);
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       row_write(qs[j], L.gw + uint32_t(j) * L.wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
@@ -1231,7 +1240,7 @@ __global__ void __launch_bounds__(256) m3need_row_kernel(const Frame* __restrict
                                                          long long nunits, Queues Q, const uint32_t* __restrict__ cls) {
   pdl_wait();
   pdl_launch();
-  __shared__ RowTotals tot;
+  __shared__ Totals<kRowWarps> tot;
   for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
     const RowLane L = row_lane(frames, nframes, u);
     const Frame& f = *L.f;
@@ -1276,7 +1285,7 @@ __global__ void __launch_bounds__(256) m3need_row_kernel(const Frame* __restrict
       col_count(qt[j], ents[1], pix[1]);
     }
     unsigned int base[2];
-    rows_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, Q.n + kNM3px, Q.n + kNTpx, base);
+    block_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, base);
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       row_write(qm[j], L.gw + uint32_t(j) * L.wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
@@ -1290,7 +1299,7 @@ __global__ void __launch_bounds__(256) d2_row_kernel(const Frame* __restrict__ f
                                                      Queues Q, int k) {
   pdl_wait();
   pdl_launch();
-  __shared__ RowTotals tot;
+  __shared__ Totals<kRowWarps> tot;
   for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
     const RowLane L = row_lane(frames, nframes, u);
     uint32_t c[6], g[6], d[2];
@@ -1303,7 +1312,7 @@ __global__ void __launch_bounds__(256) d2_row_kernel(const Frame* __restrict__ f
       col_count(d[j], ents[0], pix[0]);
     }
     unsigned int base[2];
-    rows_reserve(tot, ents, pix, Q.n + kNB, Q.n + kNB, Q.n + kNBpx, Q.n + kNBpx, base);
+    block_reserve(tot, ents, pix, Q.n + kNB, Q.n + kNB, base);
 #pragma unroll
     for (int j = 0; j < 2; ++j) row_write(d[j], L.gw + uint32_t(j) * L.wpr, base[0], reinterpret_cast<uint2*>(Q.q2));
   }
@@ -1314,7 +1323,7 @@ __global__ void __launch_bounds__(256) grow_first_row_kernel(const Frame* __rest
                                                              long long nunits, Queues Q) {
   pdl_wait();
   pdl_launch();
-  __shared__ RowTotals tot;
+  __shared__ Totals<kRowWarps> tot;
   const int lane = threadIdx.x & 31;
   for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
     const RowLane L = row_lane(frames, nframes, u);
@@ -1349,8 +1358,8 @@ __global__ void __launch_bounds__(256) grow_first_row_kernel(const Frame* __rest
     const unsigned int n = __shfl_sync(0xffffffffu, incl, 31);
     const unsigned int ents[2] = {n, 0u}, pix[2] = {0u, 0u};
     unsigned int base[2];
-    rows_reserve(tot, ents, pix, Q.n + kNRep, Q.n + kNRep, nullptr, nullptr, base);
-    if (lane == 0 && n) atomicAdd(f.counters + 0, (unsigned long long)n);
+    block_reserve(tot, ents, pix, Q.n + kNRep, Q.n + kNRep, base);
+    if (threadIdx.x == 0 && tot.sum[0]) atomicAdd(f.counters + 0, (unsigned long long)tot.sum[0]);
     unsigned int o = base[0] + incl - cnt;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
@@ -1415,7 +1424,7 @@ __global__ void __launch_bounds__(256) d2_segrow_kernel(const Frame* __restrict_
                                                         int k) {
   pdl_wait();
   pdl_launch();
-  __shared__ RowTotals tot;
+  __shared__ Totals<kRowWarps> tot;
   const unsigned int nseg = Q.n[kNSegD];
   seg_blocks(nseg, [&](unsigned int i0) {
     uint32_t d[kSegPerWarp], gw[kSegPerWarp];
@@ -1431,7 +1440,7 @@ __global__ void __launch_bounds__(256) d2_segrow_kernel(const Frame* __restrict_
       col_count(d[j], ents[0], pix[0]);
     }
     unsigned int base[2];
-    rows_reserve(tot, ents, pix, Q.n + kNB, Q.n + kNB, Q.n + kNBpx, Q.n + kNBpx, base);
+    block_reserve(tot, ents, pix, Q.n + kNB, Q.n + kNB, base);
 #pragma unroll
     for (int j = 0; j < kSegPerWarp; ++j) row_write(d[j], gw[j], base[0], reinterpret_cast<uint2*>(Q.q2));
   });
@@ -1441,7 +1450,7 @@ __global__ void __launch_bounds__(256) need_segrow_kernel(const Frame* __restric
                                                           const uint32_t* __restrict__ cls) {
   pdl_wait();
   pdl_launch();
-  __shared__ RowTotals tot;
+  __shared__ Totals<kRowWarps> tot;
   const unsigned int nseg = Q.n[kNSegN];
   seg_blocks(nseg, [&](unsigned int i0) {
     uint32_t qs[kSegPerWarp], qsp[kSegPerWarp], gw[kSegPerWarp];
@@ -1474,7 +1483,7 @@ __global__ void __launch_bounds__(256) need_segrow_kernel(const Frame* __restric
       col_count(qsp[j], ents[1], pix[1]);
     }
     unsigned int base[2];
-    rows_reserve(tot, ents, pix, Q.n + kNS, Q.n + kNSP, Q.n + kNSpx, Q.n + kNSPpx, base);
+    block_reserve(tot, ents, pix, Q.n + kNS, Q.n + kNSP, base);
 #pragma unroll
     for (int j = 0; j < kSegPerWarp; ++j) {
       row_write(qs[j], gw[j], base[0], reinterpret_cast<uint2*>(Q.q0));
@@ -1487,7 +1496,7 @@ __global__ void __launch_bounds__(256) m3need_segrow_kernel(const Frame* __restr
                                                             const uint32_t* __restrict__ cls) {
   pdl_wait();
   pdl_launch();
-  __shared__ RowTotals tot;
+  __shared__ Totals<kRowWarps> tot;
   const unsigned int nseg = Q.n[kNSeg];
   seg_blocks(nseg, [&](unsigned int i0) {
     uint32_t qm[kSegPerWarp], qt[kSegPerWarp], gw[kSegPerWarp];
@@ -1518,7 +1527,7 @@ __global__ void __launch_bounds__(256) m3need_segrow_kernel(const Frame* __restr
       col_count(qt[j], ents[1], pix[1]);
     }
     unsigned int base[2];
-    rows_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, Q.n + kNM3px, Q.n + kNTpx, base);
+    block_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, base);
 #pragma unroll
     for (int j = 0; j < kSegPerWarp; ++j) {
       row_write(qm[j], gw[j], base[0], reinterpret_cast<uint2*>(Q.q0));
@@ -2104,8 +2113,12 @@ __global__ void __launch_bounds__(kColWarps * 32) grow_first_kernel(const Frame*
   pdl_wait();
   pdl_launch();
   __shared__ ColWords sw;
+  __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (long long u = (long long)blockIdx.x * kColWarps + warp; u < nunits; u += (long long)gridDim.x * kColWarps) {
+  const Frame* accf = nullptr;
+  unsigned long long acc = 0;
+  for (long long ub = (long long)blockIdx.x * kColWarps; ub < nunits; ub += (long long)gridDim.x * kColWarps) {  // whole blocks
+    const long long u = min(ub + warp, nunits - 1);
     const Frame& f = frames[frame_of_unit(frames, nframes, u)];
     const long long lu = u - f.u0;
     const int uy = int(lu / f.ugx), ux = int(lu - (long long)uy * f.ugx);
@@ -2114,12 +2127,13 @@ __global__ void __launch_bounds__(kColWarps * 32) grow_first_kernel(const Frame*
     const int hw = lane == 0 ? wc0 - 1 : wc0 + 32;  // the word beyond the strip (lanes 0 and 31)
     const bool hin = (lane == 0 || lane == 31) && hw >= 0 && hw < f.wpr;
     const uint32_t fmask = inw ? frame_word(wc, f.w) : 0u;
+    const bool on = ub + warp < nunits;
     uint32_t c0 = 0, c1 = 0, c2 = 0, e0 = 0, e1 = 0, e2 = 0;  // cand, rows r-2 .. r (own, beyond)
     uint32_t tp = 0, etp = 0;                                  // T of row r-1 (own, beyond)
     uint32_t a0 = 0, a1 = 0, a2 = 0, b0 = 0, b1 = 0, b2 = 0;  // g1, rows r-3 .. r-1 (own, beyond)
     uint32_t l0 = 0, l1 = 0, l2 = 0;                           // L, rows r-2 .. r (own)
     unsigned int cnt = 0;
-    for (int r = y0 - 2; r < y0 + kSH + 2; ++r) {
+    for (int r = y0 - 2; on && r < y0 + kSH + 2; ++r) {
       const bool rin = r >= 0 && r < f.h;
       const size_t ro = size_t(rin ? r : 0) * f.wpr;
       const uint32_t cr = (rin && inw) ? f.cand[ro + wc] : 0u, er = (rin && hin) ? f.cand[ro + hw] : 0u;
@@ -2159,15 +2173,17 @@ __global__ void __launch_bounds__(kColWarps * 32) grow_first_kernel(const Frame*
       if (lane >= o) incl += t;
     }
     const unsigned int total = __shfl_sync(0xffffffffu, incl, 31);
-    unsigned int base = 0;
-    if (lane == 0 && total) {
-      base = atomicAdd(Q.n + kNRep, total);
-      atomicAdd(f.counters + 0, (unsigned long long)total);
+    if (&f != accf) {  // the count of the warp's strips of a frame: one atomic each
+      if (lane == 0 && acc) atomicAdd(accf->counters + 0, acc);
+      accf = &f;
+      acc = 0;
     }
-    base = __shfl_sync(0xffffffffu, base, 0);
-    __syncwarp();
-    unsigned int o = base + incl - cnt;
-    if (inw) {
+    acc += total;
+    const unsigned int ents[2] = {total, 0u}, pix[2] = {0u, 0u};
+    unsigned int base[2];
+    block_reserve(tot, ents, pix, Q.n + kNRep, Q.n + kNRep, base);
+    unsigned int o = base[0] + incl - cnt;
+    if (on && inw) {
       for (int rr = 0; rr < kSH; ++rr) {
         uint32_t v = sw.w[warp][rr][0][lane];
         const uint32_t row = uint32_t(f.pix0 + (long long)(y0 + rr) * f.w + 32 * wc);
@@ -2180,6 +2196,7 @@ __global__ void __launch_bounds__(kColWarps * 32) grow_first_kernel(const Frame*
     }
     __syncwarp();  // the shared words are refilled for the next strip
   }
+  if (lane == 0 && acc) atomicAdd(accf->counters + 0, acc);
 }
 
 // grow_kernel (iterations 2 on): for each candidate c, the first growth g1
