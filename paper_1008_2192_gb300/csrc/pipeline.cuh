@@ -1665,12 +1665,19 @@ __device__ __forceinline__ void expand_words(const Frame* __restrict__ frames, i
   constexpr int kPer = 32 / kGran;  // items per entry at most
   __shared__ uint16_t items[kThreads / 32][32 * kPer];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned int wpb = blockDim.x >> 5;
-  for (unsigned int c0 = (blockIdx.x * wpb + warp) * 32u; c0 < n; c0 += gridDim.x * wpb * 32u) {
+  const unsigned int wpb = blockDim.x >> 5, warps = gridDim.x * wpb;
+  // entries per warp: 32, or fewer where every warp of the grid then still has some. A round of items takes 3000
+  // to 6000 cycles (window loads and networks), and 32 entries hold two to four rounds: the 500 to 5000
+  // entries of the later iterations of a 4146 x 2051 frame kept 17 to 150 warps busy for all of a launch
+  // (488 -> 438 us per call).
+  const unsigned int per = min(32u, max(1u, (n + warps - 1u) / warps)), step = warps * per;
+  // the lane's entry; lanes without one start beyond any queue
+  unsigned int c = (blockIdx.x * wpb + warp) * per + (unsigned(lane) < per ? unsigned(lane) : 1u << 30);
+  for (; __any_sync(0xffffffffu, c < n); c += step) {
     uint32_t m = 0, pm = 0;
     int fi = 0, y = 0, x0 = 0;
-    if (c0 + lane < n) {
-      const uint2 e = q[kRev ? n - 1u - (c0 + lane) : c0 + lane];
+    if (c < n) {
+      const uint2 e = q[kRev ? n - 1u - c : c];
       pm = e.y;
       m = group_mask<kGran>(e.y);
       decode_word(frames, nframes, e.x, fi, y, x0);
