@@ -290,14 +290,14 @@ int init_ctx(crb_ctx* c) {
     const void* fns[kQKernels] = {
         reinterpret_cast<const void*>(crb::bound_dense_kernel),      reinterpret_cast<const void*>(crb::need_kernel),
         reinterpret_cast<const void*>(crb::s_kernel),           reinterpret_cast<const void*>(crb::sp_kernel),
-        reinterpret_cast<const void*>(crb::m3need_kernel<false>), reinterpret_cast<const void*>(crb::m3_kernel),
+        reinterpret_cast<const void*>(crb::tests_kernel<false>), reinterpret_cast<const void*>(crb::clear_kernel),
         reinterpret_cast<const void*>(crb::cand_test_kernel),   reinterpret_cast<const void*>(crb::rep_compute_kernel),
         reinterpret_cast<const void*>(crb::bound_sparse_kernel),   reinterpret_cast<const void*>(crb::rq_kernel),
         reinterpret_cast<const void*>(crb::rep_write_kernel),   reinterpret_cast<const void*>(crb::d2_kernel),
         reinterpret_cast<const void*>(crb::cand_full_kernel),   reinterpret_cast<const void*>(crb::grow_kernel),
         reinterpret_cast<const void*>(crb::mask_kernel),        reinterpret_cast<const void*>(crb::seg_list_kernel),
         reinterpret_cast<const void*>(crb::d2_seg_kernel),      reinterpret_cast<const void*>(crb::need_seg_kernel),
-        reinterpret_cast<const void*>(crb::m3need_seg_kernel),  reinterpret_cast<const void*>(crb::m3need_kernel<true>),
+        reinterpret_cast<const void*>(crb::tests_seg_kernel),   reinterpret_cast<const void*>(crb::tests_kernel<true>),
         reinterpret_cast<const void*>(crb::grow_first_kernel)};
     for (int i = 0; i < kQKernels; ++i) {
       int o = 0;
@@ -523,8 +523,6 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
       uint32_t* cls = P.cells[k & 1];
       uint32_t* cls_next = (k < P.niter) ? P.cells[(k + 1) & 1] : nullptr;
       const uint32_t* kcls = (k == 1) ? nullptr : cls;
-      // the classes and changed pixels of iteration k+1 start at zero (those of iteration k-1 were read by then)
-      const bool clear = k >= 3 && cls_next;
       const long long ucol = (P.nunits + crb::kColWarps - 1) / crb::kColWarps;
       const int gcol = grid(kQNeed, ucol);
       const int gcolm = grid(kQM3need, ucol), gcol1m = grid(kQM3needAll, ucol);
@@ -585,35 +583,30 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
         tq(kQSp, [&] { go(crb::sp_kernel, gq * P.occ[kQSp], 256, c->d_frames, P.n, P.Q, c->p, k); });
       });
       timed(c, kPM3need, stream, [&] {
-        if (seg)
+        if (P.row_form)
+          tq(kQM3need, [&] { go(crb::tests_row_kernel, grow, 256, c->d_frames, P.n, P.nunits, P.Q, kcls); });
+        else if (seg)
           tq(kQM3needSeg, [&] {
-            if (P.row_form)
-              go(crb::m3need_segrow_kernel, gseg, 256, c->d_frames, P.n, P.Q, cls);
-            else
-              go(crb::m3need_seg_kernel, gq * P.occ[kQM3needSeg], tcol, c->d_frames, P.n, P.Q, cls);
+            go(crb::tests_seg_kernel, gq * P.occ[kQM3needSeg], tcol, c->d_frames, P.n, P.Q, cls);
           });
         else if (k == 1)
-          tq(kQM3needAll, [&] {
-            go(crb::m3need_kernel<true>, gcol1m, tcol, c->d_frames, P.n, P.nunits, P.Q, nullptr);
-          });
+          tq(kQM3needAll, [&] { go(crb::tests_kernel<true>, gcol1m, tcol, c->d_frames, P.n, P.nunits, P.Q, nullptr); });
         else
-          tq(kQM3need, [&] {
-            if (P.row_form)
-              go(crb::m3need_row_kernel, grow, 256, c->d_frames, P.n, P.nunits, P.Q, kcls);
-            else
-              go(crb::m3need_kernel<false>, gcolm, tcol, c->d_frames, P.n, P.nunits, P.Q, kcls);
-          });
+          tq(kQM3need, [&] { go(crb::tests_kernel<false>, gcolm, tcol, c->d_frames, P.n, P.nunits, P.Q, kcls); });
       });
-      timed(c, kPM3, stream, [&] {
-        tq(kQM3, [&] { go(crb::m3_kernel, gq * P.occ[kQM3], 256, c->d_frames, P.n, P.Q, k); });
+      timed(c, kPM3, stream, [&] {  // the classes and changed pixels of iteration k+1 start at zero
+        tq(kQM3, [&] {
+          go(crb::clear_kernel, cls_next ? gq * P.occ[kQM3] : 1, 256, reinterpret_cast<uint4*>(cls_next),
+             cls_next ? (cells_bytes + 15) / 16 : 0, reinterpret_cast<uint4*>(P.chg[(k + 1) & 1]),
+             cls_next ? P.chg_bytes / 16 : 0);
+        });
       });
       timed(c, kPCand, stream, [&] {
         tq(kQCand, [&] {
           go(crb::cand_test_kernel, gq * P.occ[kQCand], 256, c->d_frames, P.n, P.Q, c->p, k);
         });
         tq(kQCandFull, [&] {
-          go(crb::cand_full_kernel, gq * P.occ[kQCandFull], 256, c->d_frames, P.n, P.Q, c->p, k, reinterpret_cast<uint4*>(cls_next), clear ? (cells_bytes + 15) / 16 : 0,
-             reinterpret_cast<uint4*>(P.chg[(k + 1) & 1]), clear ? P.chg_bytes / 16 : 0);
+          go(crb::cand_full_kernel, gq * P.occ[kQCandFull], 256, c->d_frames, P.n, P.Q, c->p, k);
         });
       });
       timed(c, kPGrow, stream, [&] {
@@ -713,10 +706,10 @@ constexpr long long kPdlPixels = 1LL << 27;
 // level on 8192^2 (1462, 1460), slower above (4532 -> 4844 on 16384^2).
 constexpr long long kRowFormPixels = 1LL << 26;
 
-// Queue pipeline: workspace = [queue counters | per frame: bit planes M, rq, fb |
-// cell classes x 2 | changed-pixel planes x 2] (zeroed at the start of a call)
-// then [per frame: bit planes hot, act, nsp, test, sval, m3val, lpz; maps S, N, S',
-// M3] then [queues q0, q1, q2 (a pixel index per pixel or a word entry per
+// Queue pipeline: workspace = [queue counters | per frame: bit planes M, rq, fb, cand,
+// low] (zeroed at the start of a call) then [cell classes x 2 | changed-pixel planes
+// x 2] (clear_kernel) then [per frame: bit planes hot, act, nsp, test, sval, lpz; maps
+// S, N, S', M3] then [queues q0, q1, q2 (a pixel index per pixel or a word entry per
 // word), fresh, fbl (a pixel index per pixel)].
 int prepare_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Plan& P) {
   const int n = int(specs.size());
@@ -735,9 +728,10 @@ int prepare_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pl
     off_zero[size_t(i)] = total;
     total += 5 * align256(size_t(s.w + 31) / 32 * size_t(s.h) * 4);
   }
+  const size_t zero_bytes = total;
   const size_t off_cells = total;
   total += 2 * align256(size_t(ncells) * 4);
-  // changed-pixel planes, one region per parity (all frames), zeroed with one memset each
+  // changed-pixel planes, one region per parity (all frames)
   std::vector<size_t> off_chg(static_cast<size_t>(n));
   size_t chg_bytes = 0;
   for (int i = 0; i < n; ++i) {
@@ -746,11 +740,10 @@ int prepare_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pl
   }
   const size_t off_chg0 = total;
   total += 2 * chg_bytes;
-  const size_t zero_bytes = total;
   for (int i = 0; i < n; ++i) {
     const auto& s = specs[size_t(i)];
     off_bits[size_t(i)] = total;
-    total += 7 * align256(size_t(s.w + 31) / 32 * size_t(s.h) * 4);
+    total += 6 * align256(size_t(s.w + 31) / 32 * size_t(s.h) * 4);
     off_maps[size_t(i)] = total;
     total += 4 * align256(size_t(s.w) * size_t(s.h) * 4);
   }
@@ -759,9 +752,9 @@ int prepare_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pl
   const size_t fbytes = align256(size_t(npix) * 4);
   const size_t off_q = total;
   total += 3 * qbytes + 2 * fbytes;
-  const size_t off_seg = total;  // three segment lists, one entry per segment at most
+  const size_t off_seg = total;  // two segment lists, one entry per segment at most
   const size_t segbytes = align256(size_t(nsegs) * 4);
-  total += 3 * segbytes;
+  total += 2 * segbytes;
   const int nit = niter > 0 ? niter : 1;
   const int ncounters = (2 + crb::kWork) * nit * n;
   const size_t tab_n = size_t(npix >> crb::kTabShift) + 1;
@@ -795,8 +788,7 @@ int prepare_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pl
     f.nsp = reinterpret_cast<uint32_t*>(pb + 2 * plane);
     f.test = reinterpret_cast<uint32_t*>(pb + 3 * plane);
     f.sval = reinterpret_cast<uint32_t*>(pb + 4 * plane);
-    f.m3val = reinterpret_cast<uint32_t*>(pb + 5 * plane);
-    f.lpz = reinterpret_cast<uint32_t*>(pb + 6 * plane);
+    f.lpz = reinterpret_cast<uint32_t*>(pb + 5 * plane);
     f.mapS = reinterpret_cast<float*>(pm);
     f.mapN = reinterpret_cast<float*>(pm + fmap);
     f.mapSp = reinterpret_cast<float*>(pm + 2 * fmap);
@@ -865,7 +857,7 @@ int prepare_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pl
   P.Q.q2 = reinterpret_cast<uint32_t*>(ws + off_q + 2 * qbytes);
   P.Q.fresh = reinterpret_cast<uint32_t*>(ws + off_q + 3 * qbytes);
   P.Q.fbl = reinterpret_cast<uint32_t*>(ws + off_q + 3 * qbytes + fbytes);
-  for (int j = 0; j < 3; ++j) P.Q.seg[j] = reinterpret_cast<uint32_t*>(ws + off_seg + size_t(j) * segbytes);
+  for (int j = 0; j < 2; ++j) P.Q.seg[j] = reinterpret_cast<uint32_t*>(ws + off_seg + size_t(j) * segbytes);
   P.chg[0] = ws + off_chg0;
   P.chg[1] = ws + off_chg0 + chg_bytes;
   P.chg_bytes = chg_bytes;

@@ -69,7 +69,7 @@ struct Frame {
   int wps;
   // queue pipeline (pipeline.cuh): bit planes (flag-word layout) and float maps
   uint32_t *hot, *act, *nsp, *test;
-  uint32_t *sval, *m3val;  // positions whose mapS/mapN, mapM3 hold the current iteration's values
+  uint32_t* sval;  // positions whose mapS/mapN hold the current iteration's values
   uint32_t* lpz;           // L+ == 0 (then S == 0 exactly, and no median is needed)
   uint32_t *cand, *low;    // iteration 1: candidates; S' > sigfrac*sigclip (at the nsp pixels)
   float bkl, bkh;          // bound test thresholds over gain^2 (bound_thresholds)

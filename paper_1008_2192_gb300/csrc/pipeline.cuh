@@ -5,15 +5,15 @@
 //   bound          L+ and the upper bound S+ of every pixel -> bit planes hot
 //                  (S+ > sigclip), act (S+ > min(sigclip, sigfrac*sigclip))
 //                  and lpz (L+ = 0, where S = 0 exactly); in iteration 1 (the
-//                  dense pass) also med3 of every pixel -> map M3;
+//                  dense pass) also med3 of every pixel -> map M3; later (the
+//                  re-test within 2 px of a change) bits and med3 there, so
+//                  that the planes and M3 are always current;
 //   need           nsp = needS' = dilate5(hot) & act, needS = dilate5(nsp)
 //                  -> queues QS (S to compute) and QSP (S' to compute);
 //   s              at QS: m5, N, L+, S -> maps N, S;
 //   sp             at QSP: S' = S - med5(S) -> map S'; S' > sigclip -> bit
 //                  plane test;
-//   m3need         QT = the test bits to (re)test, needM3 = dilate3(QT) ->
-//                  queues QT and QM3 (iteration 1: QT only, M3 is whole);
-//   m3             at QM3: med3 -> map M3 (iterations >= 2);
+//   tests          QT = the test bits to (re)test -> queue QT;
 //   cand_test      at QT: the objlim test from bounds of med7(m3) (smallest
 //                  and largest column median), decided exactly where they
 //                  suffice -> candidates; otherwise -> open tests;
@@ -34,8 +34,8 @@
 // the replacement gave a new value: it sets their bits in a changed-pixel plane
 // and marks, per cell of one word x kCH rows, the smallest radius class (2, 4
 // or 6 px) that reaches into the cell. The bound pass re-tests exactly the
-// pixels within 2 px of a changed one (d2, bound_sparse). Validity planes sval
-// and m3val record where mapS/mapN and mapM3 hold current values; S' is
+// pixels within 2 px of a changed one (d2, bound_sparse). The validity plane sval
+// records where mapS/mapN hold current values; S' is
 // current on all of nsp (nsp and S' change only within 4 px). Iteration 1
 // treats every cell as changed; from iteration kSegFrom on, the bit-plane
 // kernels walk only the listed segments that hold work.
@@ -78,8 +78,8 @@ enum : int {
   kNSpx = 1,
   kNSP = 2,     // QSP
   kNSPpx = 3,
-  kNM3 = 4,     // QM3
-  kNM3px = 5,
+  kNFree = 4,   // (not used)
+  kNFree2 = 5,
   kNT = 6,      // QT
   kNTpx = 7,
   kNB = 8,      // pixels to re-test in the bound pass
@@ -90,25 +90,24 @@ enum : int {
   kNAmb = 13,   // tests the column-median bounds leave open
   kNFresh = 14, // new flags of this iteration
   kNFb = 15,    // pixels with a fully flagged window (kept over the iterations)
-  kNSeg = 16,   // segments (1 word x kSH rows) listed for m3need_seg_kernel,
-  kNSegN = 17,  // for need_seg_kernel,
-  kNSegD = 18,  // for d2_seg_kernel (the three in Queues::seg order)
-  kNCount = 19
+  kNSegN = 16,  // segments (1 word x kSH rows) listed for need_seg_kernel and tests_seg_kernel,
+  kNSegD = 17,  // for d2_seg_kernel (the two in Queues::seg order)
+  kNCount = 18
 };
 
-// QS, QSP, QM3 and QT hold word entries: (global word index, mask of the
+// QS, QSP and QT hold word entries: (global word index, mask of the
 // word's pixels), one per word with a set bit, so that the bit-plane kernels
 // write one entry per word; the kernels that use them expand the masks into
 // one pixel (or group of pixels) per thread (expand_words).
 struct Queues {
-  uint32_t* q0;     // QS, then QM3, then the candidates, then the replacement values (as float)
+  uint32_t* q0;     // QS, then the candidates, then the replacement values (as float)
   uint32_t* q1;     // QSP, then the open tests, then the replacement queue
   uint32_t* q2;     // the bound pass's pixels (iterations >= 2), then QT
   uint32_t* fresh;  // new flags
   uint32_t* fbl;    // fully flagged windows
   unsigned int* n;  // kNCount counters
   const uint32_t* ftab;  // frame of global pixel t << kTabShift
-  uint32_t* seg[3];      // segments listed for m3need, need, d2 (iterations >= kSegFrom): 32 * strip + word
+  uint32_t* seg[2];      // segments listed for need and tests, for d2 (iterations >= kSegFrom): 32 * strip + word
 };
 
 // the image J of iteration k (I0, then the in-place buffer)
@@ -430,7 +429,7 @@ __device__ __forceinline__ uint32_t cell_class(const uint32_t* __restrict__ cls,
   return cls ? cls[f.cell0 + (long long)(y / kCH) * f.wpr + wc] : 4u;
 }
 
-// The column kernels (need, m3need): one warp per strip of 32 words x kSH rows,
+// The column kernels (need, tests, d2): one warp per strip of 32 words x kSH rows,
 // lane = word. The lane walks down the strip keeping the last rows of its word
 // in registers, so a vertical dilation is an OR of registers and a horizontal
 // one an OR across lanes; lanes 0 and 31 also carry the words left and right of
@@ -468,8 +467,8 @@ __device__ __forceinline__ void col_write(const ColWords& sw, int warp, int j, u
 // Reserves the entries and positions of two queues (counter pairs at c0, c1) for
 // the block's NW warps: each warp's bases. One atomic per block and queue: the
 // queues' counters lie in one line, where an atomic takes about 1.7 ns: with two per
-// warp and queue, m3need in iteration 1 of 430 Mpix took 80 us (52,000 atomics) against
-// 44, d2 84 against 64, a whole 16384 x 16384 clean 4558 against 4468. Every thread of the
+// warp and queue, the test list of iteration 1 of 430 Mpix took 80 us (52,000 atomics)
+// against 44, d2 84 against 64, a whole 16384 x 16384 clean 4558 against 4468. Every thread of the
 // block calls it.
 template <int NW>
 struct Totals {
@@ -625,19 +624,15 @@ __global__ void __launch_bounds__(kColWarps * 32) need_kernel(const Frame* __res
   }
 }
 
-// m3need_kernel: QT = the test bits of cells of class >= 2, needM3 = dilate3(QT)
-// within the frame -> queue QT, and queue QM3 where M3 is not current (m3val;
-// cleared in cells of class 4); bit plane m3val. Column kernel: rows y0-3 ..
-// y0+kSH+2 feed the seven-row window of QT. kAll (iteration 1): every cell
-// counts as changed and cls is not read; the dense bound pass has written M3
-// on the whole frame, so QM3 is empty and m3val full.
+// tests_kernel: QT = the test words of cells of class >= 2 (kAll, iteration 1: of all cells, cls is not read)
+// -> queue q2. One warp per strip; M3 is current on the whole frame (bound_dense_kernel,
+// bound_sparse_kernel), so nothing else is needed for a test.
 template <bool kAll>
-__global__ void __launch_bounds__(kColWarps * 32) m3need_kernel(const Frame* __restrict__ frames, int nframes,
-                                                                long long nunits, Queues Q,
-                                                                const uint32_t* __restrict__ cls_in) {
+__global__ void __launch_bounds__(kColWarps * 32) tests_kernel(const Frame* __restrict__ frames, int nframes,
+                                                               long long nunits, Queues Q,
+                                                               const uint32_t* __restrict__ cls) {
   pdl_wait();
   pdl_launch();
-  const uint32_t* __restrict__ cls = kAll ? nullptr : cls_in;
   __shared__ ColWords sw;
   __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -646,84 +641,23 @@ __global__ void __launch_bounds__(kColWarps * 32) m3need_kernel(const Frame* __r
     const Frame& f = frames[frame_of_unit(frames, nframes, u)];
     const long long lu = u - f.u0;
     const int uy = int(lu / f.ugx), ux = int(lu - (long long)uy * f.ugx);
-    const int wc0 = ux * 32, y0 = uy * kSH, wc = wc0 + lane;
-    const bool inw = wc < f.wpr;
-    const int hw = lane == 0 ? wc0 - 1 : wc0 + 32;
-    const bool hin = (lane == 0 || lane == 31) && hw >= 0 && hw < f.wpr;
-    const uint32_t fmask = inw ? frame_word(wc, f.w) : 0u;
-    const bool on = ub + warp < nunits && !(cls && !__any_sync(0xffffffffu, strip_has_class2(cls, f, wc, inw, hw, hin, y0, 1)));
-    if constexpr (kAll) {
-      // iteration 1: the dense bound pass wrote M3 everywhere, so M3 is current on the whole frame and
-      // nothing is queued for m3; QT = the test words
-      unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
-      uint32_t tq[kSH];
-#pragma unroll
-      for (int t = 0; t < kSH; ++t) tq[t] = (on && inw && y0 + t < f.h) ? f.test[size_t(y0 + t) * f.wpr + wc] : 0u;
-#pragma unroll
-      for (int t = 0; t < kSH; ++t) {
-        if (on && inw && y0 + t < f.h) f.m3val[size_t(y0 + t) * f.wpr + wc] = fmask;
-        sw.w[warp][t][0][lane] = 0u;
-        sw.w[warp][t][1][lane] = tq[t];
-        col_count(tq[t], ents[1], pix[1]);
-      }
-      unsigned int base[2];
-      block_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, base);
-      __syncwarp();
-      if (on) col_write(sw, warp, 1, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[1],
-                reinterpret_cast<uint2*>(Q.q2));
-      __syncwarp();
-      continue;
-    }
-    uint32_t t0 = 0, t1 = 0, t2 = 0, t3 = 0, t4 = 0, t5 = 0, t6 = 0;  // own QT words, rows r-6 .. r
-    uint32_t s0 = 0, s1 = 0, s2 = 0, s3 = 0, s4 = 0, s5 = 0, s6 = 0;  // halo QT words
+    const int y0 = uy * kSH, wc = ux * 32 + lane;
+    const bool on = ub + warp < nunits && wc < f.wpr;
     unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
-    // rows y0-3 .. y0+kSH+2 in chunks of kColChunk (the last chunk runs past the end)
-    for (int rc = y0 - 3; on && rc < y0 + kSH + 3; rc += kColChunk) {
-      uint32_t Lq[kColChunk], Lg[kColChunk], Lm[kColChunk], Lc4[kColChunk];
+    uint32_t tq[kSH], cl[kSH / kCH];
 #pragma unroll
-      for (int i = 0; i < kColChunk; ++i) {
-        const int r = rc + i, yo = r - 3;
-        const bool rin = r >= 0 && r < f.h && r < y0 + kSH + 3;
-        const size_t ro = size_t(rin ? r : 0) * f.wpr;
-        Lq[i] = (rin && inw && cell_class(cls, f, wc, r) >= 2u) ? f.test[ro + wc] : 0u;
-        Lg[i] = (rin && hin && cell_class(cls, f, hw, r) >= 2u) ? f.test[ro + hw] : 0u;
-        const bool out = yo >= y0 && yo < y0 + kSH && yo < f.h && inw;
-        Lc4[i] = out ? uint32_t(cell_class(cls, f, wc, yo) >= 4u) : 0u;
-        Lm[i] = (out && !Lc4[i]) ? f.m3val[size_t(yo) * f.wpr + wc] : 0u;
-      }
+    for (int j = 0; j < kSH / kCH; ++j) cl[j] = (on && y0 + j * kCH < f.h) ? cell_class(kAll ? nullptr : cls, f, wc, y0 + j * kCH) : 0u;
 #pragma unroll
-      for (int i = 0; i < kColChunk; ++i) {
-        t0 = t1; t1 = t2; t2 = t3; t3 = t4; t4 = t5; t5 = t6; t6 = Lq[i];
-        s0 = s1; s1 = s2; s2 = s3; s3 = s4; s4 = s5; s5 = s6; s6 = Lg[i];
-        const int yo = rc + i - 3;
-        if (yo < y0 || yo >= y0 + kSH) continue;  // whole warp
-        const uint32_t v = t0 | t1 | t2 | t3 | t4 | t5 | t6, gv = s0 | s1 | s2 | s3 | s4 | s5 | s6;
-        uint32_t left = __shfl_up_sync(0xffffffffu, v, 1), right = __shfl_down_sync(0xffffffffu, v, 1);
-        const uint32_t gl = __shfl_sync(0xffffffffu, gv, 0), gr = __shfl_sync(0xffffffffu, gv, 31);
-        if (lane == 0) left = gl;
-        if (lane == 31) right = gr;
-        uint32_t qm = 0, qto = 0;
-        if (yo < f.h && inw) {
-          const uint32_t need = hdil<3>(left, v, right) & fmask;
-          const bool c4 = Lc4[i] != 0u;
-          if (need || c4) {
-            const uint32_t old = Lm[i];  // 0 in cells of class 4
-            qm = need & ~old;
-            if (c4 || qm) f.m3val[size_t(yo) * f.wpr + wc] = old | need;
-          }
-          qto = t3;  // QT word of row yo
-        }
-        sw.w[warp][yo - y0][0][lane] = qm;
-        sw.w[warp][yo - y0][1][lane] = qto;
-        col_count(qm, ents[0], pix[0]);
-        col_count(qto, ents[1], pix[1]);
-      }
+    for (int t = 0; t < kSH; ++t) tq[t] = (on && y0 + t < f.h && cl[t / kCH] >= 2u) ? f.test[size_t(y0 + t) * f.wpr + wc] : 0u;
+#pragma unroll
+    for (int t = 0; t < kSH; ++t) {
+      sw.w[warp][t][0][lane] = tq[t];
+      col_count(tq[t], ents[0], pix[0]);
     }
     unsigned int base[2];
-    block_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, base);
+    block_reserve(tot, ents, pix, Q.n + kNT, Q.n + kNT, base);
     __syncwarp();
-    if (on) col_write(sw, warp, 0, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
-    if (on) col_write(sw, warp, 1, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[1], reinterpret_cast<uint2*>(Q.q2));
+    if (ents[0]) col_write(sw, warp, 0, uint32_t(f.word0 + (long long)y0 * f.wpr + wc), f.wpr, base[0], reinterpret_cast<uint2*>(Q.q2));
     __syncwarp();
   }
 }
@@ -795,54 +729,38 @@ __global__ void __launch_bounds__(kColWarps * 32) d2_kernel(const Frame* __restr
 // one listed segment down its rows, loading the words left and right of it
 // themselves (the strip kernels above share them across lanes instead). The
 // outputs are those of the strip kernels: a segment left out of the list has
-// none, because every output of need, m3need and d2 lies within 3 px of a cell
-// of class >= 2.
+// none, because every output of need, tests and d2 lies in a cell of class >= 2.
 constexpr int kSegFrom = 3;
 
-// seg_list_kernel: lists the segments each segment kernel walks. d2: a cell
-// of class 4 among the segment's own cells (a pixel within 2 px of a change
-// lies in one); need: a cell of class >= 2 among them; m3need: a cell of class
-// >= 2 in the segment's word column or the ones left and right of it, among
-// the segment's cell rows widened by one each way (QT of those cells reaches 3
-// px into the segment). 8 strips per block (warp = strip, lane = word); one
-// atomic per block and list.
+// seg_list_kernel: lists the segments the segment kernels walk. need and tests: a
+// cell of class >= 2 among the segment's own; d2: a cell of class 4 (a pixel
+// within 2 px of a change lies in one). 8 strips per block (warp = strip, lane =
+// word); one atomic per block and list.
 __global__ void __launch_bounds__(kThreads) seg_list_kernel(const Frame* __restrict__ frames, int nframes,
                                                             long long nunits, Queues Q,
                                                             const uint32_t* __restrict__ cls) {
   pdl_wait();
   pdl_launch();
   __shared__ int ws[kThreads / 32 + 1];
-  __shared__ unsigned int sbase[3];
+  __shared__ unsigned int sbase[2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int kWarps = kThreads / 32, kCells = kSH / kCH;
   for (long long ub = (long long)blockIdx.x * kWarps; ub < nunits; ub += (long long)gridDim.x * kWarps) {
     const long long u = ub + warp;
-    bool put[3] = {false, false, false};
+    bool put[2] = {false, false};
     if (u < nunits) {  // whole warp
       const Frame& f = frames[frame_of_unit(frames, nframes, u)];
       const long long lu = u - f.u0;
       const int uy = int(lu / f.ugx), ux = int(lu - (long long)uy * f.ugx);
-      const int wc0 = ux * 32, wc = wc0 + lane;
-      const bool inw = wc < f.wpr;
-      const int hw = lane == 0 ? wc0 - 1 : wc0 + 32;
-      const bool hin = (lane == 0 || lane == 31) && hw >= 0 && hw < f.wpr;
-      bool own2 = false, own4 = false, near2 = false, halo2 = false;
-      for (int cy = max(uy * kCells - 1, 0); cy < min((uy + 1) * kCells + 1, f.ncy); ++cy) {
-        const uint32_t* row = cls + f.cell0 + (long long)cy * f.wpr;
-        const uint32_t c = inw ? row[wc] : 0u;
-        const bool mine = cy >= uy * kCells && cy < (uy + 1) * kCells;
-        near2 |= c >= 2u;
-        own2 |= mine && c >= 2u;
-        own4 |= mine && c >= 4u;
-        if (hin && row[hw] >= 2u) halo2 = true;
+      const int wc = ux * 32 + lane;
+      for (int cy = uy * kCells; cy < min((uy + 1) * kCells, f.ncy); ++cy) {
+        const uint32_t c = wc < f.wpr ? cls[f.cell0 + (long long)cy * f.wpr + wc] : 0u;
+        put[0] |= c >= 2u;
+        put[1] |= c >= 4u;
       }
-      const bool l = __shfl_up_sync(0xffffffffu, near2, 1), r = __shfl_down_sync(0xffffffffu, near2, 1);
-      put[0] = inw && (near2 || (lane == 0 ? halo2 : l) || (lane == 31 ? halo2 : r));
-      put[1] = own2;
-      put[2] = own4;
     }
-    uint32_t* const qq[3] = {Q.seg[0], Q.seg[1], Q.seg[2]};
-    block_append<3>(put, uint32_t(u * 32 + lane), qq, Q.n + kNSeg, ws, sbase);
+    uint32_t* const qq[2] = {Q.seg[0], Q.seg[1]};
+    block_append<2>(put, uint32_t(u * 32 + lane), qq, Q.n + kNSegN, ws, sbase);
   }
 }
 
@@ -890,7 +808,7 @@ __global__ void __launch_bounds__(kColWarps * 32) d2_seg_kernel(const Frame* __r
   for (unsigned int bb = blockIdx.x * kColWarps * 32u; bb < nseg; bb += gridDim.x * kColWarps * 32u) {  // whole blocks
     const bool on = bb + warp * 32u < nseg;
     const unsigned int b = on ? bb + warp * 32u : bb;
-    const SegLane S = seg_lane(frames, nframes, Q.seg[2], b, nseg);
+    const SegLane S = seg_lane(frames, nframes, Q.seg[1], b, nseg);
     const Frame& f = *S.f;
     const int wc = S.wc, y0 = S.y0, wpr = S.wpr, h = S.h;
     const bool ok = S.ok, inl = S.inl, inr = S.inr;
@@ -943,7 +861,7 @@ __global__ void __launch_bounds__(kColWarps * 32) need_seg_kernel(const Frame* _
   for (unsigned int bb = blockIdx.x * kColWarps * 32u; bb < nseg; bb += gridDim.x * kColWarps * 32u) {  // whole blocks
     const bool on = bb + warp * 32u < nseg;
     const unsigned int b = on ? bb + warp * 32u : bb;
-    const SegLane S = seg_lane(frames, nframes, Q.seg[1], b, nseg);
+    const SegLane S = seg_lane(frames, nframes, Q.seg[0], b, nseg);
     const Frame& f = *S.f;
     const int wc = S.wc, y0 = S.y0, wpr = S.wpr, h = S.h;
     const bool ok = S.ok, inl = S.inl, inr = S.inr;
@@ -1026,74 +944,33 @@ __global__ void __launch_bounds__(kColWarps * 32) need_seg_kernel(const Frame* _
   }
 }
 
-// m3need_seg_kernel: m3need_kernel over the listed segments.
-__global__ void __launch_bounds__(kColWarps * 32) m3need_seg_kernel(const Frame* __restrict__ frames, int nframes,
-                                                                    Queues Q, const uint32_t* __restrict__ cls) {
+// tests_seg_kernel: tests_kernel over the segments listed for need_seg_kernel (those with a cell of class >= 2).
+__global__ void __launch_bounds__(kColWarps * 32) tests_seg_kernel(const Frame* __restrict__ frames, int nframes,
+                                                                   Queues Q, const uint32_t* __restrict__ cls) {
   pdl_wait();
   pdl_launch();
   __shared__ ColWords sw;
   __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned int nseg = Q.n[kNSeg];
+  const unsigned int nseg = Q.n[kNSegN];
   for (unsigned int bb = blockIdx.x * kColWarps * 32u; bb < nseg; bb += gridDim.x * kColWarps * 32u) {  // whole blocks
     const bool on = bb + warp * 32u < nseg;
-    const unsigned int b = on ? bb + warp * 32u : bb;
-    const SegLane S = seg_lane(frames, nframes, Q.seg[0], b, nseg);
+    const SegLane S = seg_lane(frames, nframes, Q.seg[0], on ? bb + warp * 32u : bb, nseg);
     const Frame& f = *S.f;
-    const int wc = S.wc, y0 = S.y0, wpr = S.wpr, h = S.h;
-    const bool ok = S.ok, inl = S.inl, inr = S.inr;
-    const uint32_t* __restrict__ test = f.test;
-    const long long cb = f.cell0 + wc;
-    uint32_t ql[7] = {}, qc[7] = {}, qr[7] = {};  // QT, rows r-6 .. r: left, own, right words
     unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
-    for (int tc = -3; on && tc < kSH + 3; tc += 8) {  // rows y0-3 .. y0+kSH+2 (the last chunk runs past them)
-      uint32_t Ql[8], Qc[8], Qr[8], Lm[8], Lc4[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int r = y0 + tc + i, t = tc + i - 3;
-        const bool rin = ok && r >= 0 && r < h && tc + i < kSH + 3;
-        const size_t ro = size_t(rin ? r : 0) * wpr + wc;
-        const long long cr = cb + (long long)((rin ? r : 0) / kCH) * wpr;
-        // the loads do not wait for the classes: test is masked by them afterwards
-        Qc[i] = rin ? test[ro] & (cls[cr] >= 2u ? ~0u : 0u) : 0u;
-        Ql[i] = (rin && inl) ? test[ro - 1] & (cls[cr - 1] >= 2u ? ~0u : 0u) : 0u;
-        Qr[i] = (rin && inr) ? test[ro + 1] & (cls[cr + 1] >= 2u ? ~0u : 0u) : 0u;
-        const bool out = ok && t >= 0 && t < kSH && y0 + t < h;
-        Lc4[i] = out ? uint32_t(cls[cb + (long long)((y0 + t) / kCH) * wpr] >= 4u) : 0u;
-        Lm[i] = out ? f.m3val[size_t(y0 + t) * wpr + wc] : 0u;
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-#pragma unroll
-        for (int j = 0; j < 6; ++j) { ql[j] = ql[j + 1]; qc[j] = qc[j + 1]; qr[j] = qr[j + 1]; }
-        ql[6] = Ql[i]; qc[6] = Qc[i]; qr[6] = Qr[i];
-        const int t = tc + i - 3;
-        if (t < 0 || t >= kSH) continue;  // whole warp
-        uint32_t qm = 0, qto = 0;
-        if (ok && y0 + t < h) {
-          const uint32_t need = hdil<3>(ql[0] | ql[1] | ql[2] | ql[3] | ql[4] | ql[5] | ql[6],
-                                        qc[0] | qc[1] | qc[2] | qc[3] | qc[4] | qc[5] | qc[6],
-                                        qr[0] | qr[1] | qr[2] | qr[3] | qr[4] | qr[5] | qr[6]) &
-                                S.fmask;
-          const bool c4 = Lc4[i] != 0u;
-          if (need || c4) {
-            const uint32_t old = c4 ? 0u : Lm[i];  // M3 is not current anywhere in cells of class 4
-            qm = need & ~old;
-            if (c4 || qm) f.m3val[size_t(y0 + t) * wpr + wc] = old | need;
-          }
-          qto = qc[3];  // QT word of row y0+t
-        }
-        sw.w[warp][t][0][lane] = qm;
-        sw.w[warp][t][1][lane] = qto;
-        col_count(qm, ents[0], pix[0]);
-        col_count(qto, ents[1], pix[1]);
-      }
+    for (int t = 0; t < kSH; ++t) {
+      const int y = S.y0 + t;
+      const bool in = on && S.ok && y < S.h;
+      const uint32_t c = in ? cls[f.cell0 + (long long)(y / kCH) * S.wpr + S.wc] : 0u;
+      const uint32_t v = (in ? f.test[size_t(y) * S.wpr + S.wc] : 0u) & (c >= 2u ? ~0u : 0u);
+      sw.w[warp][t][0][lane] = v;
+      col_count(v, ents[0], pix[0]);
     }
     unsigned int base[2];
-    block_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, base);
+    block_reserve(tot, ents, pix, Q.n + kNT, Q.n + kNT, base);
     __syncwarp();
-    if (on) col_write(sw, warp, 0, S.gw0, wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
-    if (on) col_write(sw, warp, 1, S.gw0, wpr, base[1], reinterpret_cast<uint2*>(Q.q2));
+    if (ents[0]) col_write(sw, warp, 0, S.gw0, S.wpr, base[0], reinterpret_cast<uint2*>(Q.q2));
     __syncwarp();
   }
 }
@@ -1235,62 +1112,29 @@ __global__ void __launch_bounds__(256) need_row_kernel(const Frame* __restrict__
   }
 }
 
-// m3need_kernel<false>, row form.
-__global__ void __launch_bounds__(256) m3need_row_kernel(const Frame* __restrict__ frames, int nframes,
-                                                         long long nunits, Queues Q, const uint32_t* __restrict__ cls) {
+// tests_kernel, row form (cls: nullptr in iteration 1).
+__global__ void __launch_bounds__(256) tests_row_kernel(const Frame* __restrict__ frames, int nframes, long long nunits,
+                                                        Queues Q, const uint32_t* __restrict__ cls) {
   pdl_wait();
   pdl_launch();
   __shared__ Totals<kRowWarps> tot;
   for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
     const RowLane L = row_lane(frames, nframes, u);
     const Frame& f = *L.f;
-    uint32_t q[8], g[8], m[2];
-    row_load<8>(f.test, L, -3, q, g);
-    // rows ya-3 .. ya+4 lie in two cell rows at most
-    const int clo = max(L.ya - 3, 0) / kCH, chi = min(L.ya + 4, L.h - 1) / kCH;
-    const uint32_t* cr = cls + f.cell0;
-    const bool any = L.ya < L.h;
-    const uint32_t c0 = (any && L.inw) ? cr[(long long)clo * L.wpr + L.wc] : 0u;
-    const uint32_t c1 = (any && L.inw) ? cr[(long long)chi * L.wpr + L.wc] : 0u;
-    const uint32_t g0 = (any && L.hin) ? cr[(long long)clo * L.wpr + L.hw] : 0u;
-    const uint32_t g1 = (any && L.hin) ? cr[(long long)chi * L.wpr + L.hw] : 0u;
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-      m[j] = (L.inw && L.ya + j < L.h) ? f.m3val[size_t(L.ya + j) * L.wpr + L.wc] : 0u;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const bool lo = max(L.ya - 3 + i, 0) / kCH == clo;
-      if ((lo ? c0 : c1) < 2u) q[i] = 0u;
-      if ((lo ? g0 : g1) < 2u) g[i] = 0u;
-    }
-    const bool c4 = (L.ya / kCH == clo ? c0 : c1) >= 4u;
-    uint32_t qm[2], qt[2];
+    const bool in = L.inw && L.ya < L.h;
+    const uint32_t cl = in ? cell_class(cls, f, L.wc, L.ya) : 0u;  // both rows lie in one cell
+    uint32_t q[2];
     unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      uint32_t v = 0, gv = 0;
-#pragma unroll
-      for (int i = 0; i < 7; ++i) v |= q[j + i], gv |= g[j + i];
-      const uint32_t need = row_dil<3>(v, gv) & L.fmask;
-      qm[j] = qt[j] = 0u;
-      if (L.ya + j < L.h && L.inw) {
-        if (need || c4) {
-          const uint32_t old = c4 ? 0u : m[j];
-          qm[j] = need & ~old;
-          if (c4 || qm[j]) f.m3val[size_t(L.ya + j) * L.wpr + L.wc] = old | need;
-        }
-        qt[j] = q[j + 3];
-      }
-      col_count(qm[j], ents[0], pix[0]);
-      col_count(qt[j], ents[1], pix[1]);
+      // the load does not wait for the class
+      q[j] = ((in && L.ya + j < L.h) ? f.test[size_t(L.ya + j) * L.wpr + L.wc] : 0u) & (cl >= 2u ? ~0u : 0u);
+      col_count(q[j], ents[0], pix[0]);
     }
     unsigned int base[2];
-    block_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, base);
+    block_reserve(tot, ents, pix, Q.n + kNT, Q.n + kNT, base);
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      row_write(qm[j], L.gw + uint32_t(j) * L.wpr, base[0], reinterpret_cast<uint2*>(Q.q0));
-      row_write(qt[j], L.gw + uint32_t(j) * L.wpr, base[1], reinterpret_cast<uint2*>(Q.q2));
-    }
+    for (int j = 0; j < 2; ++j) row_write(q[j], L.gw + uint32_t(j) * L.wpr, base[0], reinterpret_cast<uint2*>(Q.q2));
   }
 }
 
@@ -1431,7 +1275,7 @@ __global__ void __launch_bounds__(256) d2_segrow_kernel(const Frame* __restrict_
     unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
 #pragma unroll
     for (int j = 0; j < kSegPerWarp; ++j) {
-      const SegRow S = seg_row(frames, nframes, Q.seg[2], i0 + j, nseg);
+      const SegRow S = seg_row(frames, nframes, Q.seg[1], i0 + j, nseg);
       const uint32_t* chg = S.f->chg[k & 1];
       const uint32_t c = S.rin ? chg[S.ro] : 0u, l = S.inl ? chg[S.ro - 1] : 0u, r = S.inr ? chg[S.ro + 1] : 0u;
       d[j] = hdil<2>(vor<2>(l), vor<2>(c), vor<2>(r)) & S.fmask;
@@ -1457,7 +1301,7 @@ __global__ void __launch_bounds__(256) need_segrow_kernel(const Frame* __restric
     unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
 #pragma unroll
     for (int j = 0; j < kSegPerWarp; ++j) {
-      const SegRow S = seg_row(frames, nframes, Q.seg[1], i0 + j, nseg);
+      const SegRow S = seg_row(frames, nframes, Q.seg[0], i0 + j, nseg);
       const Frame& f = *S.f;
       const uint32_t hc = S.rin ? f.hot[S.ro] : 0u, hl = S.inl ? f.hot[S.ro - 1] : 0u, hr = S.inr ? f.hot[S.ro + 1] : 0u;
       const uint32_t ac = S.rin ? f.act[S.ro] : 0u, al = S.inl ? f.act[S.ro - 1] : 0u, ar = S.inr ? f.act[S.ro + 1] : 0u;
@@ -1488,50 +1332,6 @@ __global__ void __launch_bounds__(256) need_segrow_kernel(const Frame* __restric
     for (int j = 0; j < kSegPerWarp; ++j) {
       row_write(qs[j], gw[j], base[0], reinterpret_cast<uint2*>(Q.q0));
       row_write(qsp[j], gw[j], base[1], reinterpret_cast<uint2*>(Q.q1));
-    }
-  });
-}
-
-__global__ void __launch_bounds__(256) m3need_segrow_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
-                                                            const uint32_t* __restrict__ cls) {
-  pdl_wait();
-  pdl_launch();
-  __shared__ Totals<kRowWarps> tot;
-  const unsigned int nseg = Q.n[kNSeg];
-  seg_blocks(nseg, [&](unsigned int i0) {
-    uint32_t qm[kSegPerWarp], qt[kSegPerWarp], gw[kSegPerWarp];
-    unsigned int ents[2] = {0u, 0u}, pix[2] = {0u, 0u};
-#pragma unroll
-    for (int j = 0; j < kSegPerWarp; ++j) {
-      const SegRow S = seg_row(frames, nframes, Q.seg[0], i0 + j, nseg);
-      const Frame& f = *S.f;
-      const uint32_t* cr = cls + f.cell0 + (long long)((S.rin ? S.y : 0) / kCH) * f.wpr + S.wc;
-      const uint32_t cl = S.rin ? cr[0] : 0u;
-      const uint32_t c = (S.rin ? f.test[S.ro] : 0u) & (cl >= 2u ? ~0u : 0u);
-      const uint32_t l = S.inl ? f.test[S.ro - 1] & (cr[-1] >= 2u ? ~0u : 0u) : 0u;
-      const uint32_t r = S.inr ? f.test[S.ro + 1] & (cr[1] >= 2u ? ~0u : 0u) : 0u;
-      const uint32_t m = S.out ? f.m3val[S.ro] : 0u;
-      const uint32_t need = hdil<3>(vor<3>(l), vor<3>(c), vor<3>(r)) & S.fmask;
-      qm[j] = qt[j] = 0u;
-      gw[j] = S.gw;
-      if (S.out) {
-        const bool c4 = cl >= 4u;
-        if (need || c4) {
-          const uint32_t old = c4 ? 0u : m;  // M3 is not current anywhere in cells of class 4
-          qm[j] = need & ~old;
-          if (c4 || qm[j]) f.m3val[S.ro] = old | need;
-        }
-        qt[j] = c;
-      }
-      col_count(qm[j], ents[0], pix[0]);
-      col_count(qt[j], ents[1], pix[1]);
-    }
-    unsigned int base[2];
-    block_reserve(tot, ents, pix, Q.n + kNM3, Q.n + kNT, base);
-#pragma unroll
-    for (int j = 0; j < kSegPerWarp; ++j) {
-      row_write(qm[j], gw[j], base[0], reinterpret_cast<uint2*>(Q.q0));
-      row_write(qt[j], gw[j], base[1], reinterpret_cast<uint2*>(Q.q2));
     }
   });
 }
@@ -1878,43 +1678,19 @@ __global__ void __launch_bounds__(256, 3) sp_kernel(const Frame* __restrict__ fr
                   });
 }
 
-// m3_kernel: at QM3, med3 of J, by groups of four pixels x0 .. x0+3 that hold
-// a listed one. The six columns x0-1 .. x0+4 of the rows y-1 .. y+1 are sorted
-// once; the median of a 3x3 window is then the median of three values: the
-// largest of its column minima, the median of its column medians and the
-// smallest of its column maxima (an exact selection of the fifth of nine).
-__global__ void __launch_bounds__(256) m3_kernel(const Frame* __restrict__ frames, int nframes, Queues Q, int k) {
+// clear_kernel (each iteration): the cell classes and changed pixels that this
+// iteration's replacement will mark for the next start at zero (n0 and n1 16-byte
+// vectors at z0 and z1; last read in the previous iteration; none in the last).
+__global__ void __launch_bounds__(256) clear_kernel(uint4* z0, size_t n0, uint4* z1, size_t n1) {
   pdl_wait();
   pdl_launch();
-  expand_words<4, true>(frames, nframes, reinterpret_cast<const uint2*>(Q.q0), Q.n[kNM3],
-                  [&](bool valid, int fi, int x0, int y, uint32_t bits) {
-                    if (!valid) return;
-                    const Frame& f = frames[fi];
-                    float v[3][6];
-                    load_span<1>(qsrc(f, k), x0, y, f.w, f.h, v);
-                    float lo[6], mi[6], hi[6];
-#pragma unroll
-                    for (int c = 0; c < 6; ++c) {  // sort the column: lo <= mi <= hi
-                      const float s0 = fminf(v[0][c], v[1][c]), s1 = fmaxf(v[0][c], v[1][c]);
-                      hi[c] = fmaxf(s1, v[2][c]);
-                      const float t = fminf(s1, v[2][c]);
-                      lo[c] = fminf(s0, t);
-                      mi[c] = fmaxf(s0, t);
-                    }
-                    float* __restrict__ out = f.mapM3 + size_t(y) * f.w + x0;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                      if (!((bits >> i) & 1u)) continue;
-                      const float a = max3f(lo[i], lo[i + 1], lo[i + 2]);
-                      const float b = fmaxf(fminf(mi[i], mi[i + 1]), fminf(fmaxf(mi[i], mi[i + 1]), mi[i + 2]));
-                      const float c = min3f(hi[i], hi[i + 1], hi[i + 2]);
-                      out[i] = fmaxf(fminf(a, b), fminf(fmaxf(a, b), c));
-                    }
-                  });
+  const size_t t = size_t(blockIdx.x) * blockDim.x + threadIdx.x, step = size_t(gridDim.x) * blockDim.x;
+  for (size_t i = t; i < n0; i += step) z0[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (size_t i = t; i < n1; i += step) z1[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// bound_sparse_kernel (iteration >= 2): the bound test of the pixels listed in
-// q2 (within 2 px of a change), by groups of four pixels x .. x+3 that hold a
+// bound_sparse_kernel (iteration >= 2): the bound test and med3 of the pixels listed
+// in q2 (within 2 px of a change; med3 changes within 1 px), by groups of four pixels x .. x+3 that hold a
 // listed one: one thread forms the column medians of the eight columns x-2 ..
 // x+5 (rows and columns clamped at the frame's edges, as in the dense pass),
 // then per pixel the minimum of five of them and L+: the dense pass's
@@ -1923,7 +1699,11 @@ __global__ void __launch_bounds__(256) m3_kernel(const Frame* __restrict__ frame
 // the kernel, so the thread reads the plane words and XORs in only the bits
 // that changed, with no atomic where none did (most re-tests change nothing);
 // XORs of disjoint bits by other groups of the word commute with it.
-__global__ void __launch_bounds__(256, 4) bound_sparse_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
+// med3 was a pass of its own over the 7x7 neighbourhoods of the tests (listed
+// by dilating them, with a plane of where it was current): listing and pass took
+// 0.57 ms of a 430 Mpix batch, against 0.2 ms more here and 0.14 for the list of
+// tests. Three blocks per SM: at four it spills (batch 6657 us, at three 6527).
+__global__ void __launch_bounds__(256, 3) bound_sparse_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
                                                            Params p) {
   pdl_wait();
   pdl_launch();
@@ -1934,6 +1714,24 @@ __global__ void __launch_bounds__(256, 4) bound_sparse_kernel(const Frame* __res
                     const int w = f.w, h = f.h;
                     float v[5][8];  // rows y-2 .. y+2, columns x0-2 .. x0+5
                     load_span<2>(f.out_clean, x0, y, w, h, v);
+                    {  // med3 of the group, from the sorted columns x0-1 .. x0+4
+                      float lo[6], mi[6], hi[6];
+#pragma unroll
+                      for (int c = 0; c < 6; ++c) sort3(v[1][c + 1], v[2][c + 1], v[3][c + 1], lo[c], mi[c], hi[c]);
+                      float m3[4];
+#pragma unroll
+                      for (int i = 0; i < 4; ++i)
+                        m3[i] = med3f(max3f(lo[i], lo[i + 1], lo[i + 2]), med3f(mi[i], mi[i + 1], mi[i + 2]),
+                                      min3f(hi[i], hi[i + 1], hi[i + 2]));
+                      float* __restrict__ out = f.mapM3 + size_t(y) * w + x0;
+                      if ((w & 3) == 0) {  // the map starts on a 256-byte boundary, x0 is a multiple of 4
+                        *reinterpret_cast<float4*>(out) = make_float4(m3[0], m3[1], m3[2], m3[3]);
+                      } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                          if (x0 + i < w) out[i] = m3[i];
+                      }
+                    }
                     float cm[8];
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
@@ -2068,16 +1866,11 @@ __global__ void __launch_bounds__(256, 3) cand_test_kernel(const Frame* __restri
 }
 
 // cand_full_kernel: at the open tests, the exact F = m3 - med7(m3) and the
-// objlim test -> candidates. It also clears the cell classes and changed pixels
-// the replacement will mark (n0 and n1 16-byte vectors at z0 and z1), last read
-// in the previous iteration.
+// objlim test -> candidates.
 __global__ void __launch_bounds__(256) cand_full_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
-                                                        Params p, int k, uint4* z0, size_t n0, uint4* z1, size_t n1) {
+                                                        Params p, int k) {
   pdl_wait();
   pdl_launch();
-  const size_t zt = size_t(blockIdx.x) * blockDim.x + threadIdx.x, zs = size_t(gridDim.x) * blockDim.x;
-  for (size_t i = zt; i < n0; i += zs) z0[i] = make_uint4(0u, 0u, 0u, 0u);
-  for (size_t i = zt; i < n1; i += zs) z1[i] = make_uint4(0u, 0u, 0u, 0u);
   __shared__ WarpLists<1, 128> wl;
   wl.init();
   uint32_t* const lists[1] = {Q.q0};
@@ -2586,7 +2379,7 @@ __global__ void queue_work_kernel(const Frame* __restrict__ frames, Queues Q, in
     unsigned long long* wk = frames[0].work + kWork * (k - 1);
     wk[0] += Q.n[kNSpx];
     wk[1] += Q.n[kNSPpx];
-    wk[2] += Q.n[kNM3px];
+    wk[2] += (k == 1) ? 0ull : (unsigned long long)Q.n[kNBpx];  // med3 goes with the re-test (iteration 1: with the dense pass)
     wk[3] += Q.n[kNTpx];
     wk[4] += Q.n[kNAmb];
     wk[5] += (k == 1) ? (unsigned long long)dense : (unsigned long long)Q.n[kNBpx];

@@ -90,9 +90,10 @@ namespace {
 size_t frame_bytes(int w, int h) {
   // the caller's input, cleaned output and mask (resident while queued), and the
   // workspace of the queue pipeline: 4 float maps, 5 queue entries per pixel,
-  // 14 bit planes (2 of them changed-pixel planes), 2 words per cell of one
-  // word x 8 rows (the class arrays) and 3 words per segment of one word x 16
-  // rows (the segment lists)
+  // 13 bit planes (2 of them changed-pixel planes), 2 words per cell of one
+  // word x 8 rows (the class arrays) and 2 words per segment of one word x 16
+  // rows (the segment lists); the admission rule counts one plane and one word
+  // per segment more
   const size_t n = size_t(w) * size_t(h);
   const size_t wpr = size_t(w + 31) / 32;
   const size_t plane = wpr * size_t(h) * 4;
