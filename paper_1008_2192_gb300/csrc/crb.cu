@@ -302,7 +302,7 @@ int init_ctx(crb_ctx* c) {
     for (int i = 0; i < kQKernels; ++i) {
       int o = 0;
       const bool col = i == kQNeed || i == kQM3need || i == kQD2 || i == kQD2Seg || i == kQNeedSeg ||
-                       i == kQM3needSeg || i == kQM3needAll || i == kQGrowFirst;
+                       i == kQM3needSeg || i == kQM3needAll;
       const int threads = i == kQBound ? crb::kBoundThreads : col ? crb::kColWarps * 32 : 256;
       CRB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fns[i], threads, 0));
       c->occ_q[i] = o > 0 ? o : 1;
@@ -583,7 +583,7 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
         tq(kQSp, [&] { go(crb::sp_kernel, gq * P.occ[kQSp], 256, c->d_frames, P.n, P.Q, c->p, k); });
       });
       timed(c, kPM3need, stream, [&] {
-        if (P.row_form)
+        if (P.row_form || P.pdl)  // launched early, the strip form holds the others back (11000^2: 2492 us, rows 2137)
           tq(kQM3need, [&] { go(crb::tests_row_kernel, grow, 256, c->d_frames, P.n, P.nunits, P.Q, kcls); });
         else if (seg)
           tq(kQM3needSeg, [&] {
@@ -612,10 +612,7 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
       timed(c, kPGrow, stream, [&] {
         if (k == 1)  // both growths from the bit planes; flags counted and queued for the replacement
           tq(kQGrowFirst, [&] {
-            if (P.row_form)
-              go(crb::grow_first_row_kernel, grow, 256, c->d_frames, P.n, P.nunits, P.Q);
-            else
-              go(crb::grow_first_kernel, grid(kQGrowFirst, ucol), tcol, c->d_frames, P.n, P.nunits, P.Q);
+            go(crb::grow_first_kernel, grow, 256, c->d_frames, P.n, P.nunits, P.Q);
           });
         else
           tq(kQGrow, [&] {

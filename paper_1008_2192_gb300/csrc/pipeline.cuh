@@ -1162,8 +1162,17 @@ __global__ void __launch_bounds__(256) d2_row_kernel(const Frame* __restrict__ f
   }
 }
 
-// grow_first_kernel, row form.
-__global__ void __launch_bounds__(256) grow_first_row_kernel(const Frame* __restrict__ frames, int nframes,
+// grow_first_kernel (iteration 1): both growths as bit-plane algebra,
+// M_1 = dilate3(dilate3(cand) & T) & L, where T (the test plane) holds
+// S' > sigclip and L (low) S' > sigfrac*sigclip, both set by sp_kernel at the
+// nsp pixels (the only pixels whose S' can pass either threshold), and cand
+// the candidates. This is the union of every candidate's growth (the 3x3 of
+// T around it, then the 3x3 of L around those). A warp forms two rows of a strip,
+// at every size (walking a strip's 20 rows took 148 us on 430 Mpix, this about 120; 27
+// and 8 us on 8.5 Mpix). Writes M_1 (no flag exists before: the queue
+// pipeline takes no explicit previous mask), counts it per frame, and queues its
+// pixels for the replacement, all of them being new.
+__global__ void __launch_bounds__(256) grow_first_kernel(const Frame* __restrict__ frames, int nframes,
                                                              long long nunits, Queues Q) {
   pdl_wait();
   pdl_launch();
@@ -1896,107 +1905,6 @@ __global__ void __launch_bounds__(256) cand_full_kernel(const Frame* __restrict_
     wl.put(put, g, lists, Q.n + kNPass);
   }
   wl.flush(lists, Q.n + kNPass);
-}
-
-// grow_first_kernel (iteration 1): both growths as bit-plane algebra,
-// M_1 = dilate3(dilate3(cand) & T) & L, where T (the test plane) holds
-// S' > sigclip and L (low) S' > sigfrac*sigclip, both set by sp_kernel at the
-// nsp pixels (the only pixels whose S' can pass either threshold), and cand
-// the candidates. This is the union of every candidate's growth (the 3x3 of
-// T around it, then the 3x3 of L around those). One warp per strip (lane =
-// word) walks rows y0-2 .. y0+kSH+1; lanes 0 and 31 also form the words beyond
-// the strip. Writes M_1 (no flag exists before: the queue pipeline takes no
-// explicit previous mask), counts it per frame, and queues its pixels for the
-// replacement, all of them being new.
-__global__ void __launch_bounds__(kColWarps * 32) grow_first_kernel(const Frame* __restrict__ frames, int nframes,
-                                                                    long long nunits, Queues Q) {
-  pdl_wait();
-  pdl_launch();
-  __shared__ ColWords sw;
-  __shared__ Totals<kColWarps> tot;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const Frame* accf = nullptr;
-  unsigned long long acc = 0;
-  for (long long ub = (long long)blockIdx.x * kColWarps; ub < nunits; ub += (long long)gridDim.x * kColWarps) {  // whole blocks
-    const long long u = min(ub + warp, nunits - 1);
-    const Frame& f = frames[frame_of_unit(frames, nframes, u)];
-    const long long lu = u - f.u0;
-    const int uy = int(lu / f.ugx), ux = int(lu - (long long)uy * f.ugx);
-    const int wc0 = ux * 32, y0 = uy * kSH, wc = wc0 + lane;
-    const bool inw = wc < f.wpr;
-    const int hw = lane == 0 ? wc0 - 1 : wc0 + 32;  // the word beyond the strip (lanes 0 and 31)
-    const bool hin = (lane == 0 || lane == 31) && hw >= 0 && hw < f.wpr;
-    const uint32_t fmask = inw ? frame_word(wc, f.w) : 0u;
-    const bool on = ub + warp < nunits;
-    uint32_t c0 = 0, c1 = 0, c2 = 0, e0 = 0, e1 = 0, e2 = 0;  // cand, rows r-2 .. r (own, beyond)
-    uint32_t tp = 0, etp = 0;                                  // T of row r-1 (own, beyond)
-    uint32_t a0 = 0, a1 = 0, a2 = 0, b0 = 0, b1 = 0, b2 = 0;  // g1, rows r-3 .. r-1 (own, beyond)
-    uint32_t l0 = 0, l1 = 0, l2 = 0;                           // L, rows r-2 .. r (own)
-    unsigned int cnt = 0;
-    for (int r = y0 - 2; on && r < y0 + kSH + 2; ++r) {
-      const bool rin = r >= 0 && r < f.h;
-      const size_t ro = size_t(rin ? r : 0) * f.wpr;
-      const uint32_t cr = (rin && inw) ? f.cand[ro + wc] : 0u, er = (rin && hin) ? f.cand[ro + hw] : 0u;
-      const uint32_t tr = (rin && inw) ? f.test[ro + wc] : 0u, etr = (rin && hin) ? f.test[ro + hw] : 0u;
-      const uint32_t lr = (rin && inw) ? f.low[ro + wc] : 0u;
-      c0 = c1; c1 = c2; c2 = cr;
-      e0 = e1; e1 = e2; e2 = er;
-      l0 = l1; l1 = l2; l2 = lr;
-      // g1 of row r-1
-      const uint32_t vc = c0 | c1 | c2, evc = e0 | e1 | e2;
-      uint32_t left = __shfl_up_sync(0xffffffffu, vc, 1), right = __shfl_down_sync(0xffffffffu, vc, 1);
-      if (lane == 0) left = evc;
-      if (lane == 31) right = evc;
-      const uint32_t g1 = hdil<1>(left, vc, right) & tp;
-      const uint32_t eg1 = (lane == 0 ? hdil<1>(0u, evc, vc) : hdil<1>(vc, evc, 0u)) & etp;
-      tp = tr;
-      etp = etr;
-      a0 = a1; a1 = a2; a2 = g1;
-      b0 = b1; b1 = b2; b2 = eg1;
-      // M_1 of row r-2
-      const int yo = r - 2;
-      if (yo < y0) continue;  // whole warp
-      const uint32_t vg = a0 | a1 | a2, evg = b0 | b1 | b2;
-      uint32_t gl = __shfl_up_sync(0xffffffffu, vg, 1), gr = __shfl_down_sync(0xffffffffu, vg, 1);
-      if (lane == 0) gl = evg;
-      if (lane == 31) gr = evg;
-      const uint32_t m = (yo < f.h) ? (hdil<1>(gl, vg, gr) & l0 & fmask) : 0u;
-      if (yo < f.h && inw) f.bits_a[size_t(yo) * f.wpr + wc] = m;
-      sw.w[warp][yo - y0][0][lane] = m;
-      cnt += unsigned(__popc(m));
-    }
-    // the strip's flags: one count per frame, then the replacement queue, one atomic per warp
-    unsigned int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned int t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    const unsigned int total = __shfl_sync(0xffffffffu, incl, 31);
-    if (&f != accf) {  // the count of the warp's strips of a frame: one atomic each
-      if (lane == 0 && acc) atomicAdd(accf->counters + 0, acc);
-      accf = &f;
-      acc = 0;
-    }
-    acc += total;
-    const unsigned int ents[2] = {total, 0u}, pix[2] = {0u, 0u};
-    unsigned int base[2];
-    block_reserve(tot, ents, pix, Q.n + kNRep, Q.n + kNRep, base);
-    unsigned int o = base[0] + incl - cnt;
-    if (on && inw) {
-      for (int rr = 0; rr < kSH; ++rr) {
-        uint32_t v = sw.w[warp][rr][0][lane];
-        const uint32_t row = uint32_t(f.pix0 + (long long)(y0 + rr) * f.w + 32 * wc);
-        while (v) {
-          const int bb = __ffs(v) - 1;
-          v &= v - 1u;
-          Q.q1[o++] = row + bb;
-        }
-      }
-    }
-    __syncwarp();  // the shared words are refilled for the next strip
-  }
-  if (lane == 0 && acc) atomicAdd(accf->counters + 0, acc);
 }
 
 // grow_kernel (iterations 2 on): for each candidate c, the first growth g1
