@@ -444,6 +444,23 @@ def test_row_tiles_edges(w, h, pset):
         assert c.last_counts() == list(zip(r32.n_new, r32.n_none_left)), niter
 
 
+@pytest.mark.parametrize("w,h", [(528, 330), (500, 331), (529, 271), (1152, 780), (1601, 601)])
+@pytest.mark.parametrize("pset", [dict(), dict(sigclip=1.2, sigfrac=0.3, objlim=0.05), dict(sigclip=5.0, objlim=500.0)],
+                         ids=["default", "dense-flags", "floored-objlim"])
+def test_row_tiles_of_30_rows(w, h, pset):
+    """The row kernels' 30-row tiles, which frames of more than one 14-row tile per SM take: whole tiles and
+    remainders of 1 px either way, in one round of tiles (the first three) and in more (from 609 tiles on, the
+    kernels with more blocks per SM). Masks, images and counters equal the FP32 oracle's."""
+    img = scene(w, h, seed=5 * w + h)
+    img[h // 2, :] += np.float32(4000.0)
+    img[:, w // 2] += np.float32(1500.0)
+    c = Cleaner(niter=3, pipeline="tile", **pset)
+    out, mask = gpu_clean(c, img)
+    r32 = oracle.clean(img, params_of(pset), 3, precision="f32")
+    assert np.array_equal(mask, r32.mask) and np.array_equal(out, r32.clean)
+    assert c.last_counts() == list(zip(r32.n_new, r32.n_none_left))
+
+
 @pytest.mark.parametrize("w,h", [(32, 40), (33, 40), (47, 33), (50, 17), (1040, 37), (1025, 18)])
 def test_queue_masks_off_alignment(w, h):
     """The u8 mask of rows off the 16-byte boundaries, at every offset of the mask's first byte: 16-byte vectors
