@@ -140,8 +140,8 @@ struct GraphKey {
   void* frames;
   void* tab;
   bool operator==(const GraphKey& o) const {
-    return n == o.n && niter == o.niter && shape == o.shape && rows == o.rows && fuse == o.fuse && fuse2 == o.fuse2 && queue == o.queue && pdl == o.pdl && row_form == o.row_form &&
-           seg_from == o.seg_from && occ_sig == o.occ_sig &&
+    return n == o.n && niter == o.niter && shape == o.shape && rows == o.rows && fuse == o.fuse && fuse2 == o.fuse2 &&
+           queue == o.queue && pdl == o.pdl && row_form == o.row_form && seg_from == o.seg_from && occ_sig == o.occ_sig &&
            tiles == o.tiles && nblocks == o.nblocks && ncells == o.ncells && npix == o.npix &&
            rtiles == o.rtiles && bits_total == o.bits_total && ncounters == o.ncounters && dgrid == o.dgrid &&
            fgrid == o.fgrid && rgrid == o.rgrid && ws == o.ws && counters == o.counters && frames == o.frames &&
@@ -511,7 +511,10 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
       cudaEventRecord(b, stream);
       c->tune_ev.push_back({kernel, {a, b}});
     };
-    // Below kPdlPixels every kernel may start while the one ahead of it ends.
+    // Outside a graph every kernel is launched while the one ahead of it runs, and starts once all that one's
+    // blocks have ended, before its writes are whole (pdl_wait): 639 -> 505 us on 4096^2, 522 -> 389 on
+    // 4146 x 2051, 4240 -> 4110 on 16384^2. None lets the next one start earlier (pdl_launch): blocks that
+    // wait beside the ones that work cost more than they gain (548 us, 415).
     auto go = [&](auto fn, auto grid, int block, auto... args) {
       if (P.pdl)
         launch_pdl(fn, unsigned(grid), unsigned(block), 0, stream, args...);
@@ -532,14 +535,14 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
       timed(c, kPBound, stream, [&] {
         if (k == 1) {
           tq(kQBound, [&] {
-            go(crb::bound_dense_kernel, grid(kQBound, P.nblocks), crb::kBoundThreads, c->d_frames, P.n,
-                                                                                         P.nblocks, c->p);
+            go(crb::bound_dense_kernel, grid(kQBound, P.nblocks), crb::kBoundThreads, c->d_frames, P.n, P.nblocks,
+               c->p);
           });
         } else {  // the pixels within 2 px of a change, re-tested one by one
           if (seg) {
             tq(kQSegList, [&] {
-              go(crb::seg_list_kernel, grid(kQSegList, (P.nunits + 7) / 8), crb::kThreads, 
-                  c->d_frames, P.n, P.nunits, P.Q, cls);
+              go(crb::seg_list_kernel, grid(kQSegList, (P.nunits + 7) / 8), crb::kThreads, c->d_frames, P.n,
+                 P.nunits, P.Q, cls);
             });
             tq(kQD2Seg, [&] {
               if (P.row_form)
@@ -583,7 +586,7 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
         tq(kQSp, [&] { go(crb::sp_kernel, gq * P.occ[kQSp], 256, c->d_frames, P.n, P.Q, c->p, k); });
       });
       timed(c, kPM3need, stream, [&] {
-        if (P.row_form || P.pdl)  // launched early, the strip form holds the others back (11000^2: 2492 us, rows 2137)
+        if (P.row_form)
           tq(kQM3need, [&] { go(crb::tests_row_kernel, grow, 256, c->d_frames, P.n, P.nunits, P.Q, kcls); });
         else if (seg)
           tq(kQM3needSeg, [&] {
@@ -623,13 +626,11 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
         if (k >= 2)
           tq(kQRq, [&] { go(crb::rq_kernel, gq * P.occ[kQRq], 256, c->d_frames, P.n, P.Q); });
         tq(kQRepCompute, [&] {
-          go(crb::rep_compute_kernel, gq * P.occ[kQRepCompute], 256, c->d_frames, P.n, P.Q, k,
-                                                                                cls_next);
+          go(crb::rep_compute_kernel, gq * P.occ[kQRepCompute], 256, c->d_frames, P.n, P.Q, k, cls_next);
         });
         if (k >= 2)
           tq(kQRepWrite, [&] {
-            go(crb::rep_write_kernel, gq * P.occ[kQRepWrite], 256, c->d_frames, P.n, P.Q, cls_next,
-                                                                              k + 1, 1);
+            go(crb::rep_write_kernel, gq * P.occ[kQRepWrite], 256, c->d_frames, P.n, P.Q, cls_next, k + 1, 1);
           });
       });
       if (k == P.niter)
@@ -646,8 +647,8 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
     for (int k = 1; k <= P.niter + 1; ++k) {
       const int mode = k == 1 ? 0 : k <= P.niter ? 1 : 2;
       timed(c, mode == 2 ? kPTileReplace : kPTileDetect, stream, [&] {
-        launch_pdl(t.fn[mode], unsigned(P.tiles), 256, t.smem[mode], stream, c->d_frames, k == 1 && P.one ? 0 : P.n, c->p, k, P.niter,
-                   c->h_frames[0]);
+        launch_pdl(t.fn[mode], unsigned(P.tiles), 256, t.smem[mode], stream, c->d_frames,
+                   k == 1 && P.one ? 0 : P.n, c->p, k, P.niter, c->h_frames[0]);
       });
     }
     CRB_CUDA(cudaGetLastError());
@@ -692,15 +693,9 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
   return CRB_OK;
 }
 
-// Calls below this many pixels, not replayed from a graph, launch the queue kernels so that each may start
-// while the one ahead ends (about 2 us of each of the 57 launches): 721 -> 615 us on 4146 x 2051, 782 -> 682
-// on 4096^2, 1517 -> 1466 on 8192^2, no gain on 16384^2. In a graph the same edges are slower than plain ones
-// (650 -> 677 us on 4096^2).
-constexpr long long kPdlPixels = 1LL << 27;
-
 // Calls below this many pixels take the row forms of the bit-plane kernels (pipeline.cuh): 522 -> 447 us on
-// 2048 x 3100, 573 -> 484 on 4146 x 2051, 685 -> 622 on 4096^2 (643 -> 581 in a graph), 986 -> 920 on 6000^2;
-// level on 8192^2 (1462, 1460), slower above (4532 -> 4844 on 16384^2).
+// 2048 x 3100, 547 -> 506 on 4096^2, 813 -> 790 on 6000^2, 1221 -> 1214 on 8000^2; slower on 8192^2 (1241 ->
+// 1271) and above (4532 -> 4844 on 16384^2).
 constexpr long long kRowFormPixels = 1LL << 26;
 
 // Queue pipeline: workspace = [queue counters | per frame: bit planes M, rq, fb, cand,
@@ -832,9 +827,9 @@ int prepare_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pl
   P.maps = false;
   P.fuse = false;
   P.queue = true;
-  P.zeroed = npix < kPdlPixels;
+  P.zeroed = true;
   P.row_form = npix < kRowFormPixels;
-  P.pdl = npix < kPdlPixels && !c->opt.use_graphs;
+  P.pdl = !c->opt.use_graphs;
   P.rtiles = rtiles;
   P.bits_total = zero_bytes;
   P.ncounters = ncounters;
@@ -1171,9 +1166,10 @@ int upload(crb_ctx* c, const Plan& P, cudaStream_t stream) {
 int launch_graph(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs, cudaStream_t stream) {
   long long occ_sig = 0;
   for (int i = 0; i < kQKernels; ++i) occ_sig = occ_sig * 31 + P.occ[i];
-  GraphKey key{P.n,      P.niter,      P.shape,      P.rows,  P.fuse,  P.fuse2, P.queue, P.pdl, P.row_form, P.seg_from,  occ_sig,      P.tiles,
-               P.rtiles, P.nblocks,    P.ncells,     P.npix,  P.bits_total, P.ncounters, P.dgrid, P.fgrid,
-               P.rgrid,  c->ws,        c->d_counters, c->d_frames, P.queue ? c->d_tab : nullptr};
+  GraphKey key{P.n,       P.niter,  P.shape, P.rows,  P.fuse,  P.fuse2,  P.queue,      P.pdl,
+               P.row_form, P.seg_from, occ_sig, P.tiles, P.rtiles, P.nblocks,   P.ncells,
+               P.npix,    P.bits_total, P.ncounters, P.dgrid, P.fgrid, P.rgrid, c->ws,
+               c->d_counters, c->d_frames, P.queue ? c->d_tab : nullptr};
   for (auto& g : c->graphs)
     if (g.first == key) {
       CRB_CUDA(cudaGraphLaunch(g.second, stream));

@@ -366,7 +366,6 @@ constexpr int kBoundThreads = 32 * kBW / kBoundNP;
 __global__ void __launch_bounds__(kBoundThreads, kBoundNP == 4 ? 12 : 16)
     bound_dense_kernel(const Frame* __restrict__ frames, int nframes, long long nblocks, Params p) {
   pdl_wait();
-  pdl_launch();
   const int warp = threadIdx.x >> 5;
   for (long long b = blockIdx.x; b < nblocks; b += gridDim.x) {
     const int fi = frame_of_block(frames, nframes, b);
@@ -530,7 +529,6 @@ __global__ void __launch_bounds__(kColWarps * 32) need_kernel(const Frame* __res
                                                               long long nunits, Queues Q,
                                                               const uint32_t* __restrict__ cls) {
   pdl_wait();
-  pdl_launch();
   __shared__ ColWords sw;
   __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -632,7 +630,6 @@ __global__ void __launch_bounds__(kColWarps * 32) tests_kernel(const Frame* __re
                                                                long long nunits, Queues Q,
                                                                const uint32_t* __restrict__ cls) {
   pdl_wait();
-  pdl_launch();
   __shared__ ColWords sw;
   __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -669,7 +666,6 @@ __global__ void __launch_bounds__(kColWarps * 32) tests_kernel(const Frame* __re
 __global__ void __launch_bounds__(kColWarps * 32) d2_kernel(const Frame* __restrict__ frames, int nframes,
                                                             long long nunits, Queues Q, int k) {
   pdl_wait();
-  pdl_launch();
   __shared__ ColWords sw;
   __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -740,7 +736,6 @@ __global__ void __launch_bounds__(kThreads) seg_list_kernel(const Frame* __restr
                                                             long long nunits, Queues Q,
                                                             const uint32_t* __restrict__ cls) {
   pdl_wait();
-  pdl_launch();
   __shared__ int ws[kThreads / 32 + 1];
   __shared__ unsigned int sbase[2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -800,7 +795,6 @@ __device__ __forceinline__ SegLane seg_lane(const Frame* __restrict__ frames, in
 __global__ void __launch_bounds__(kColWarps * 32) d2_seg_kernel(const Frame* __restrict__ frames, int nframes,
                                                                 Queues Q, int k) {
   pdl_wait();
-  pdl_launch();
   __shared__ ColWords sw;
   __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -853,7 +847,6 @@ __global__ void __launch_bounds__(kColWarps * 32) d2_seg_kernel(const Frame* __r
 __global__ void __launch_bounds__(kColWarps * 32) need_seg_kernel(const Frame* __restrict__ frames, int nframes,
                                                                   Queues Q, const uint32_t* __restrict__ cls) {
   pdl_wait();
-  pdl_launch();
   __shared__ ColWords sw;
   __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -948,7 +941,6 @@ __global__ void __launch_bounds__(kColWarps * 32) need_seg_kernel(const Frame* _
 __global__ void __launch_bounds__(kColWarps * 32) tests_seg_kernel(const Frame* __restrict__ frames, int nframes,
                                                                    Queues Q, const uint32_t* __restrict__ cls) {
   pdl_wait();
-  pdl_launch();
   __shared__ ColWords sw;
   __shared__ Totals<kColWarps> tot;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1055,7 +1047,6 @@ __device__ __forceinline__ uint32_t row_dil_halo(uint32_t v, uint32_t g) {
 __global__ void __launch_bounds__(256) need_row_kernel(const Frame* __restrict__ frames, int nframes, long long nunits,
                                                        Queues Q, const uint32_t* __restrict__ cls) {
   pdl_wait();
-  pdl_launch();
   __shared__ Totals<kRowWarps> tot;
   for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
     const RowLane L = row_lane(frames, nframes, u);
@@ -1116,7 +1107,6 @@ __global__ void __launch_bounds__(256) need_row_kernel(const Frame* __restrict__
 __global__ void __launch_bounds__(256) tests_row_kernel(const Frame* __restrict__ frames, int nframes, long long nunits,
                                                         Queues Q, const uint32_t* __restrict__ cls) {
   pdl_wait();
-  pdl_launch();
   __shared__ Totals<kRowWarps> tot;
   for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
     const RowLane L = row_lane(frames, nframes, u);
@@ -1142,7 +1132,6 @@ __global__ void __launch_bounds__(256) tests_row_kernel(const Frame* __restrict_
 __global__ void __launch_bounds__(256) d2_row_kernel(const Frame* __restrict__ frames, int nframes, long long nunits,
                                                      Queues Q, int k) {
   pdl_wait();
-  pdl_launch();
   __shared__ Totals<kRowWarps> tot;
   for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
     const RowLane L = row_lane(frames, nframes, u);
@@ -1175,7 +1164,6 @@ __global__ void __launch_bounds__(256) d2_row_kernel(const Frame* __restrict__ f
 __global__ void __launch_bounds__(256) grow_first_kernel(const Frame* __restrict__ frames, int nframes,
                                                              long long nunits, Queues Q) {
   pdl_wait();
-  pdl_launch();
   __shared__ Totals<kRowWarps> tot;
   const int lane = threadIdx.x & 31;
   for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
@@ -1276,7 +1264,6 @@ __device__ __forceinline__ void seg_blocks(unsigned int nseg, F&& body) {
 __global__ void __launch_bounds__(256) d2_segrow_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
                                                         int k) {
   pdl_wait();
-  pdl_launch();
   __shared__ Totals<kRowWarps> tot;
   const unsigned int nseg = Q.n[kNSegD];
   seg_blocks(nseg, [&](unsigned int i0) {
@@ -1302,7 +1289,6 @@ __global__ void __launch_bounds__(256) d2_segrow_kernel(const Frame* __restrict_
 __global__ void __launch_bounds__(256) need_segrow_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
                                                           const uint32_t* __restrict__ cls) {
   pdl_wait();
-  pdl_launch();
   __shared__ Totals<kRowWarps> tot;
   const unsigned int nseg = Q.n[kNSegN];
   seg_blocks(nseg, [&](unsigned int i0) {
@@ -1605,7 +1591,6 @@ __device__ __forceinline__ void load_pair_span(const float* __restrict__ a, int 
 // than single medians; a run of five listed pixels fills three pairs.)
 __global__ void __launch_bounds__(256, 4) s_kernel(const Frame* __restrict__ frames, int nframes, Queues Q, int k) {
   pdl_wait();
-  pdl_launch();
   expand_words<2, true>(frames, nframes, reinterpret_cast<const uint2*>(Q.q0), Q.n[kNS],
                   [&](bool valid, int fi, int x0, int y, uint32_t bits) {
                     if (!valid) return;
@@ -1644,7 +1629,6 @@ __device__ __forceinline__ uint32_t plane_bits8(const uint32_t* __restrict__ pla
 __global__ void __launch_bounds__(256, 3) sp_kernel(const Frame* __restrict__ frames, int nframes, Queues Q, Params p,
                                                     int k) {
   pdl_wait();
-  pdl_launch();
   const float siglow = __fmul_rn(p.sigfrac, p.sigclip);
   expand_words<2, true>(frames, nframes, reinterpret_cast<const uint2*>(Q.q1), Q.n[kNSP],
                   [&](bool valid, int fi, int x0, int y, uint32_t bits) {
@@ -1692,7 +1676,6 @@ __global__ void __launch_bounds__(256, 3) sp_kernel(const Frame* __restrict__ fr
 // vectors at z0 and z1; last read in the previous iteration; none in the last).
 __global__ void __launch_bounds__(256) clear_kernel(uint4* z0, size_t n0, uint4* z1, size_t n1) {
   pdl_wait();
-  pdl_launch();
   const size_t t = size_t(blockIdx.x) * blockDim.x + threadIdx.x, step = size_t(gridDim.x) * blockDim.x;
   for (size_t i = t; i < n0; i += step) z0[i] = make_uint4(0u, 0u, 0u, 0u);
   for (size_t i = t; i < n1; i += step) z1[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -1715,7 +1698,6 @@ __global__ void __launch_bounds__(256) clear_kernel(uint4* z0, size_t n0, uint4*
 __global__ void __launch_bounds__(256, 3) bound_sparse_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
                                                            Params p) {
   pdl_wait();
-  pdl_launch();
   expand_words<4, true>(frames, nframes, reinterpret_cast<const uint2*>(Q.q2), Q.n[kNB],
                   [&](bool valid, int fi, int x0, int y, uint32_t) {
                     if (!valid) return;
@@ -1815,7 +1797,6 @@ __device__ __forceinline__ void load_pair_span7(const float* __restrict__ a, int
 __global__ void __launch_bounds__(256, 3) cand_test_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
                                                            Params p, int k) {
   pdl_wait();
-  pdl_launch();
   __shared__ WarpLists<2, 128> wl;
   wl.init();
   uint32_t* const lists[2] = {Q.q0, Q.q1};
@@ -1879,7 +1860,6 @@ __global__ void __launch_bounds__(256, 3) cand_test_kernel(const Frame* __restri
 __global__ void __launch_bounds__(256) cand_full_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
                                                         Params p, int k) {
   pdl_wait();
-  pdl_launch();
   __shared__ WarpLists<1, 128> wl;
   wl.init();
   uint32_t* const lists[1] = {Q.q0};
@@ -1916,7 +1896,6 @@ __global__ void __launch_bounds__(256) cand_full_kernel(const Frame* __restrict_
 __global__ void __launch_bounds__(256, 4) grow_kernel(const Frame* __restrict__ frames, int nframes, Queues Q, Params p,
                                                    int k) {
   pdl_wait();
-  pdl_launch();
   const unsigned int n = Q.n[kNPass];
   const float sigclip = p.sigclip, siglow = __fmul_rn(p.sigfrac, p.sigclip);
   const unsigned int stride = gridDim.x * blockDim.x;
@@ -2066,7 +2045,6 @@ __device__ __forceinline__ uint32_t or_window(uint32_t* plane, int wpr, int h, i
 // one append atomic per block).
 __global__ void __launch_bounds__(256) rq_kernel(const Frame* __restrict__ frames, int nframes, Queues Q) {
   pdl_wait();
-  pdl_launch();
   __shared__ int ws[kThreads / 32 + 1];
   __shared__ unsigned int sbase;
   const unsigned int nf = Q.n[kNFresh], n = nf + Q.n[kNFb];
@@ -2135,7 +2113,6 @@ __device__ __forceinline__ void mark_change(const Frame& f, int x, int y, uint32
 __global__ void __launch_bounds__(256) rep_compute_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
                                                           int k, uint32_t* cls_next) {
   pdl_wait();
-  pdl_launch();
   const unsigned int n = Q.n[kNRep];
   float* __restrict__ vals = reinterpret_cast<float*>(Q.q0);
   for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -2196,7 +2173,6 @@ __global__ void __launch_bounds__(256) rep_compute_kernel(const Frame* __restric
 __global__ void __launch_bounds__(256) rep_write_kernel(const Frame* __restrict__ frames, int nframes, Queues Q,
                                                         uint32_t* cls_next, int knext, int clear_rq) {
   pdl_wait();
-  pdl_launch();
   const unsigned int n = Q.n[kNRep];
   const float* __restrict__ vals = reinterpret_cast<const float*>(Q.q0);
   for (unsigned int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -2225,7 +2201,6 @@ __device__ __forceinline__ uint4 mask16(uint32_t v) {
 
 __global__ void __launch_bounds__(256) mask_kernel(const Frame* __restrict__ frames, int nframes, long long nblocks) {
   pdl_wait();
-  pdl_launch();
   const int t = threadIdx.x;
   for (long long b = blockIdx.x; b < nblocks; b += gridDim.x) {
     const int fi = frame_of_block(frames, nframes, b);
