@@ -142,12 +142,14 @@ __device__ __forceinline__ float uniform_approx(uint64_t z) {
 // longest draw (22.5 of 32 active). The form that multiplied in double was bound
 // by the FP64 pipe (2 lanes per clock and SM, 81 % active): 94.2 us on a 750x750
 // image of mean 24.3, against 31.1 us (with an integer-to-float conversion
-// instruction, which runs on the FP64 pipe too, 47.8 us). Two draws per step with
+// instruction, which runs on the FP64 pipe too, 47.8 us), and 29.7 launched ahead of time. Two draws per step with
 // one comparison: the products fall monotonically, so the second one alone
 // tells whether to go on.
 // mu > 60, where e^-mu leaves float's range: the product is scaled up by 2^64
 // each time it falls below 2^-64, until the rest of e^-mu lies above 2^-90.
+// Launched while the kernel ahead of it on the stream runs; it waits for that one's results first.
 __global__ void __launch_bounds__(kPThreads) poisson_kernel(const __grid_constant__ PLaunch P) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < P.total;
        t += (long long)gridDim.x * blockDim.x) {
     int lo = 0, hi = P.n - 1;  // frame of pixel t
@@ -234,7 +236,16 @@ void fill_constants(PLaunch& P) {
 int launch(PLaunch& P, cudaStream_t stream) {
   // a pixel per thread: blocks that draw long are balanced by the blocks still to start
   const long long blocks = std::min<long long>((P.total + kPThreads - 1) / kPThreads, 1 << 22);
-  poisson_kernel<<<int(std::max<long long>(blocks, 1)), kPThreads, 0, stream>>>(P);
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(std::max<long long>(blocks, 1)));
+  cfg.blockDim = dim3(kPThreads);
+  cfg.stream = stream;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, poisson_kernel, P);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(CRB_ECUDA, std::string("crb_poisson launch: ") + cudaGetErrorString(e));
   return CRB_OK;
