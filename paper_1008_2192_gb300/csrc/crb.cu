@@ -128,7 +128,7 @@ enum QK {
 };
 
 struct GraphKey {
-  int n, niter, shape, rows;
+  int n, niter, shape;
   bool fuse, fuse2, queue, pdl, row_form;
   int seg_from;
   long long occ_sig;  // the queue kernels' blocks per SM, packed
@@ -140,7 +140,7 @@ struct GraphKey {
   void* frames;
   void* tab;
   bool operator==(const GraphKey& o) const {
-    return n == o.n && niter == o.niter && shape == o.shape && rows == o.rows && fuse == o.fuse && fuse2 == o.fuse2 &&
+    return n == o.n && niter == o.niter && shape == o.shape && fuse == o.fuse && fuse2 == o.fuse2 &&
            queue == o.queue && pdl == o.pdl && row_form == o.row_form && seg_from == o.seg_from && occ_sig == o.occ_sig &&
            tiles == o.tiles && nblocks == o.nblocks && ncells == o.ncells && npix == o.npix &&
            rtiles == o.rtiles && bits_total == o.bits_total && ncounters == o.ncounters && dgrid == o.dgrid &&
@@ -437,7 +437,6 @@ struct Plan {
   bool row_form = false;  // the row forms of the bit-plane kernels
   bool zeroed = false;  // the upload zeroes the planes and counters (else two memsets do)
   bool fuse2 = false;  // tile pipeline: iterations 2 and 3 in one launch
-  bool one = false;    // row kernels: one frame, whose descriptor iteration 1 takes with its launch (not in a graph)
   int rows = -1;       // tile pipeline: the row kernels' variant (kTileKernels), or -1 for the detect kernels
   long long tiles = 0, rtiles = 0;
   size_t bits_total = 0;  // bytes from the start of the workspace that start at zero
@@ -647,8 +646,9 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
     for (int k = 1; k <= P.niter + 1; ++k) {
       const int mode = k == 1 ? 0 : k <= P.niter ? 1 : 2;
       timed(c, mode == 2 ? kPTileReplace : kPTileDetect, stream, [&] {
+        // of one frame, iteration 1 takes the descriptor with its launch, and runs beside the upload
         launch_pdl(t.fn[mode], unsigned(P.tiles), 256, t.smem[mode], stream, c->d_frames,
-                   k == 1 && P.one ? 0 : P.n, c->p, k, P.niter, c->h_frames[0]);
+                   k == 1 && P.n == 1 ? 0 : P.n, c->p, k, P.niter, c->h_frames[0]);
       });
     }
     CRB_CUDA(cudaGetLastError());
@@ -965,7 +965,6 @@ int prepare_tile(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pla
   P.niter = niter;
   P.fuse = true;
   P.rows = v;
-  P.one = n == 1 && !c->opt.use_graphs;
   P.zeroed = true;
   P.tiles = tiles;
   P.bits_total = bits;
@@ -1169,7 +1168,7 @@ int upload(crb_ctx* c, const Plan& P, cudaStream_t stream) {
 int launch_graph(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs, cudaStream_t stream) {
   long long occ_sig = 0;
   for (int i = 0; i < kQKernels; ++i) occ_sig = occ_sig * 31 + P.occ[i];
-  GraphKey key{P.n,       P.niter,  P.shape, P.rows,  P.fuse,  P.fuse2,  P.queue,      P.pdl,
+  GraphKey key{P.n,       P.niter,  P.shape,   P.fuse,  P.fuse2,  P.queue,      P.pdl,
                P.row_form, P.seg_from, occ_sig, P.tiles, P.rtiles, P.nblocks,   P.ncells,
                P.npix,    P.bits_total, P.ncounters, P.dgrid, P.fgrid, P.rgrid, c->ws,
                c->d_counters, c->d_frames, P.queue ? c->d_tab : nullptr};
@@ -1439,8 +1438,10 @@ int run(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool maps, c
   c->mprev_frames = int(std::count_if(specs.begin(), specs.end(), [](const FrameSpec& s) { return s.mprev; }));
   rc = upload(c, P, stream);
   if (rc) return rc;
-  // graphs replay only work whose pointers all come from the descriptors
-  const bool graphable = niter > 0 && !maps && !c->opt.profile &&
+  // graphs replay only work whose pointers all come from the descriptors; the row kernels' few launches are
+  // quicker one by one, since a graph starts after the whole upload and its first kernel takes no frame
+  // (800 x 800: 75 us replayed, 53 launched)
+  const bool graphable = niter > 0 && !maps && P.rows < 0 && !c->opt.profile &&
                          std::all_of(specs.begin(), specs.end(), [](const FrameSpec& s) { return !s.mprev; });
   if (c->opt.use_graphs && graphable)
     rc = launch_graph(c, P, specs, stream);
