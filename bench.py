@@ -58,21 +58,20 @@ ALG_BYTES_PER_PIX_ITER = 8.25
 # sums, 4 clips taken as t+|t|, 3 sums, 1 scale = 16) and the two threshold
 # tests (gain*m, +rn^2, L+^2, *gain^2, two scaled thresholds, two compares = 8).
 BOUND_TEST_MINMAX = 6 + 4 + 1
-# Per pixel of iteration 1 the dense bound pass also takes med3 (the 3x3 median) from sorted columns:
+# Per tested pixel the bound pass also takes med3 (the 3x3 median) from sorted columns:
 # its column's three rows sorted (6), then the largest of three column minima (2), the median of three
 # column medians (4), the smallest of three column maxima (2) and the median of those three (4).
-M3_DENSE_MINMAX = 6 + 2 + 4 + 2 + 4
+M3_MINMAX = 6 + 2 + 4 + 2 + 4
 # DRAM bytes (read + write) per step and per input pixel of each kernel kind's
 # launches, from an ncu capture of one step on three 4096x4096 frames of the
 # batch mix (the summaries are kept with the profiles), applied to the
 # workload's pixels; a kind whose kernels changed since their capture has none.
-TRAFFIC_PER_PIXEL = {"bound": 858694144 / 50331648}
+TRAFFIC_PER_PIXEL = {"bound": 904751872 / 50331648}
 # Algorithmic FP32 operations per unit of each kernel kind: (min/max, other).
 KIND_OPS = {
-    "bound": (BOUND_TEST_MINMAX, 24),
+    "bound": (BOUND_TEST_MINMAX + M3_MINMAX, 24),
     "s": (192, 22),       # med25; L+ 16, N: mul, add, sqrt, div; S: mul, div
     "sprime": (192, 1),   # med25 of S; the difference
-    "m3": (33, 0),        # med9
 }
 
 
@@ -449,14 +448,11 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
-# FP64 arithmetic of the POISSON work function: one multiply per uniform drawn (the product; the
-# uniform's exact scaling by 2^-53 is built from its bits and the comparison with e^-mu is made on
-# the bit patterns), and per pixel 32 for e^-mu: the reduction (3 multiplies, 1 rounding, 2
-# subtractions) and the degree-13 Horner polynomial (13 multiplies, 13 additions).
-POISSON_FP64_EXP = 32
-# Nominal dense FP64 rate of a GB300 (no measured figure): 1.25 TFLOP/s counting a multiply-add as two
-# operations, i.e. 0.625 T single FP64 operations per second.
-POISSON_FP64_PEAK = 0.625e12
+# 32-bit operations of the POISSON work function per uniform drawn, as its definition asks for them: the
+# counter's 64-bit addition 2; mix13's two 64-bit products 6 (three multiply-adds each) and its first two
+# shift-and-XOR steps 8 (two shifts, two XORs each); the top word as a float in [0, 1) 3, its product 1
+# and the comparison 1. e^-mu, once per pixel (one draw in 25 at this mean), is not counted.
+POISSON_DRAW_OPS = 2 + 6 + 8 + 3 + 1 + 1
 
 
 def run_poisson(args):
@@ -465,6 +461,7 @@ def run_poisson(args):
     import torch
     import oracle
     from paper_1008_2192_gb300 import poisson_batch_into
+    from paper_1008_2192_gb300.api import fadd_peak
     torch.cuda.set_device(int(os.environ.get("LOCAL_RANK", "0")))
     mu = 24.3
     if args.workload == "poisson750":
@@ -496,7 +493,7 @@ def run_poisson(args):
     ms = e0.elapsed_time(e1) / args.steps
     clk = clocks.stop()
     draws = sum(float(o.double().sum().item()) + o.numel() for o in outs)  # k + 1 uniforms per pixel
-    fp64 = draws + POISSON_FP64_EXP * npix
+    ops, peak = draws * POISSON_DRAW_OPS, fadd_peak()
     # end to end: pinned host input, copies in and out inside the timed region
     h_in = [a.cpu().pin_memory() for a in imgs]
     h_out = [torch.empty(a.shape, dtype=torch.float32).pin_memory() for a in imgs]
@@ -529,7 +526,7 @@ def run_poisson(args):
         oracle.poisson(h0, reps)
         reps += 1
     cpu = reps * h0.size / (time.perf_counter() - t0) / 1e6
-    achieved = fp64 / (ms * 1e-3)
+    achieved = ops / (ms * 1e-3)
     line = {"metric": "Mpix/s of the POISSON work function (mean 24.3, 1 GB300)", "value": npix / (ms * 1e-3) / 1e6,
             "unit": "Mpix/s", "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
@@ -537,11 +534,12 @@ def run_poisson(args):
                        "l2": "inputs below L2" if npix * 8 < 120e6 else "inputs above L2, no flush"},
             "gpu_launches": args.steps * ((len(sizes) + 255) // 256), "clocks": clk,
             "roofline": {"bound": "alu", "kernel": "poisson_kernel", "achieved": achieved / 1e12,
-                         "peak": POISSON_FP64_PEAK / 1e12, "unit": "T FP64 ops/s",
-                         "frac": achieved / POISSON_FP64_PEAK, "traffic": None,
-                         "peak_source": "nominal FP64 rate (1.25 TFLOP/s counting a multiply-add as two)",
-                         "achieved_is": "1 FP64 multiply per uniform drawn (counted from the deviates) + 32 FP64 "
-                                        "operations per pixel for e^-mu, / device time per step"},
+                         "peak": peak / 1e12, "unit": "T 32-bit ops/s",
+                         "frac": achieved / peak, "traffic": None,
+                         "peak_source": "measured: crb_fadd_peak, one operation per lane and issue slot",
+                         "achieved_is": f"{POISSON_DRAW_OPS} 32-bit operations per uniform drawn (counted from the "
+                                        "deviates) / device time per step; about one in 256 draws and the "
+                                        "few pixels drawn again in double take more"},
             "e2e": {"value": npix / (e2e_ms * 1e-3) / 1e6, "unit": "Mpix/s", "h2d_bytes_per_step": npix * 4,
                     "d2h_bytes_per_step": npix * 4, "api": "crb_poisson_batch with pinned host copies around it"},
             "cpu_baseline": {"value": cpu, "unit": "Mpix/s", "cores": oracle.max_threads(), "kind": "oracle",
@@ -733,8 +731,7 @@ def main():
     peaks = measured_peaks()
     fadd = fadd_peak()
     net = network_minmax()
-    units = {"bound": sum(w[5] for w in work), "s": sum(w[0] for w in work), "sprime": sum(w[1] for w in work),
-             "m3": sum(w[2] for w in work)}
+    units = {"bound": sum(w[5] for w in work), "s": sum(w[0] for w in work), "sprime": sum(w[1] for w in work)}
     per_step = {k: v[0] / args.steps for k, v in kinds.items()}
     tot = sum(per_step.values())
     kernels = {k: {"ms_per_step": round(v, 4), "share": round(v / max(tot, 1e-9), 4)}
@@ -743,9 +740,6 @@ def main():
     if dom in KIND_OPS:
         mm, fp = KIND_OPS[dom]
         mm_n, fp_n = mm * units[dom], fp * units[dom]  # per step
-        if dom == "bound":  # iteration 1's dense pass also takes med3 at every pixel
-            mm_n += M3_DENSE_MINMAX * work[0][5]
-            mm = f"{mm} (+{M3_DENSE_MINMAX} in iteration 1)"
         ops = mm_n + fp_n
         achieved = ops / (per_step[dom] * 1e-3) / 1e12
         peak = ops / (mm_n / ops2 + fp_n / fadd) / 1e12  # the kernel's op mix at the measured issue rates
@@ -764,10 +758,12 @@ def main():
         roofline = {"bound": "latency", "kernel": dom, "achieved": None, "peak": None, "unit": None, "frac": None,
                     "traffic": None}
     # context: the selection networks over all detection kernels
-    # the queue kernels take S and S' medians by groups of four adjacent windows
-    m25 = net["row25"] if tuned[2] == "queue" else net[25]
-    minmax = sum(w[0] * m25 + w[1] * m25 + w[2] * net[9] + w[3] * (7 * net[7] + 12) + w[4] * net[49]
-                 + w[5] * BOUND_TEST_MINMAX for w in work)
+    # (S and S' medians by aligned pairs; the queue pipeline's bound pass also takes med3, and its tests the
+    # column medians of their windows; the tile pipeline counts its med3 by itself and decides its tests by counting)
+    m25 = net["row25"]
+    minmax = sum((w[0] + w[1]) * m25 + w[4] * net[49] + w[5] * BOUND_TEST_MINMAX
+                 + (w[5] * M3_MINMAX + w[3] * (7 * net[7] + 12) if tuned[2] == "queue" else w[2] * M3_MINMAX)
+                 for w in work)
     roofline.update({
         "kernels": kernels,
         "profiled_pass": {"steps": args.steps, "ms_per_step": prof_ms / args.steps,

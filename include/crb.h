@@ -65,19 +65,20 @@ typedef struct {
    * without an unflagged neighbour; the result is then a fixed point, so the
    * output is identical to running all niter iterations. Default 0.            */
   int early_exit;
-  /* Tile shape of the detection kernel (index of crb_tile_shape; default 0).
-   * 0 takes 64 x 32 tiles, or the 64 x 28 tiles of index 5 (one image buffer,
-   * three blocks per SM) when all of a call's tiles then fit in one round of
-   * resident blocks and the 64 x 32 tiles do not (one 800 x 800 frame).
-   * -1 = autotune: the first call with a new signature (the list of frame
+  /* Tile shape of the tile pipeline (index of crb_tile_shape; default 0).
+   * 0 takes the row kernels (48-px wide tiles of 30 rows, or of 14 where those
+   * number at most one per SM), or 64 x 32 tiles where a call asks for what
+   * they do not have: map export, a given mask, no_fusion or fuse2. Any other
+   * index takes that shape's detection kernel. -1 = autotune: the first call with a new signature (the list of frame
    * sizes and niter) runs the clean once per compiled shape, timing each on
    * the stream (that call synchronises the stream), and keeps the fastest for
    * later calls with the same signature. */
   int tile_shape;
-  /* 1: capture the work of a call (the memsets and the niter loop of launches)
-   * in a CUDA graph once per launch signature and replay it afterwards; the
-   * per-frame descriptors are uploaded before each replay. Ignored while
-   * profiling. */
+  /* 1: capture the work of a call (the niter loop of launches, with the memsets
+   * of calls that have them) in a CUDA graph once per launch signature and
+   * replay it afterwards; the per-frame descriptors are uploaded before each
+   * replay. The row kernels' few launches are made directly, which is faster.
+   * Ignored while profiling. */
   int use_graphs;
   /* 1: bracket every kernel launch with CUDA events on the launching stream;
    * read the accumulated device times with crb_profile_read. Default 0.       */
@@ -95,7 +96,7 @@ typedef struct {
    * crb_iterate's map export and by crb_clean_noalloc). 0 (default): per
    * call, the queue pipeline from 6,000,000 pixels on (all frames of the call
    * together), the tile pipeline below: the queue pipeline's ~60 dependent
-   * launches cost about 0.5 ms per call, the tile pipeline's cost is about 4.5
+   * launches cost about 0.16 ms per call, the tile pipeline about 2.7
    * times more per pixel. All give identical results. */
   int pipeline;
   /* 1: autotune the queue pipeline. The first call with a new signature (the
@@ -105,7 +106,7 @@ typedef struct {
    * largest blocks per SM), each kernel keeping the level at which its own
    * launches took least device time; then the first iteration from which the
    * bit-plane kernels walk listed segments (2, 3, 4 or none); then, for calls
-   * under 2^25 pixels with pipeline 0, the tile pipeline against the result.
+   * under 10,000,000 pixels with pipeline 0, the tile pipeline against the result.
    * Later calls with the same signature reuse the choice (crb_tuned_config
    * reports it). The launch configuration changes no result. Default 0. */
   int autotune;
@@ -235,7 +236,9 @@ int crb_partition(int w, int h, int nparts, int cols, int context, crb_rect* rec
  * every rectangle must contain its interior and lie in the frame
  * (CRB_EINVAL); outputs must not overlap img (CRB_EALIAS). The crops go
  * through the context's own staging buffers (grown on demand) and one
- * crb_clean_batch. Asynchronous on `stream`. */
+ * crb_clean_batch; one kernel copies all crops in and one all interiors out
+ * (an interior that overlaps an earlier one starts the next launch, so that
+ * the last one stands). Asynchronous on `stream`. */
 int crb_clean_rects(crb_ctx* ctx, const float* img, int w, int h, int n, const crb_rect* rects, float* out_clean,
                     uint8_t* out_mask, cudaStream_t stream);
 
@@ -253,11 +256,13 @@ int crb_last_counts(crb_ctx* ctx, long long* out, int max_iter);
 /* After crb_sync_status: the work the detection kernels did in each iteration
  * of the last call, summed over its frames: out[6k..6k+5] = positions at which
  * they evaluated S (5x5 median of J), S' (5x5 median of S), med3, the
- * candidate test, the full 7x7 median of med3 for that test (the tests that
- * bounds of the median leave open; every test in the tile pipeline), and the
- * upper-bound test. The stages are evaluated only where they can change a
- * flag, so these counts are the method's work on this input. Returns the
- * number of iterations, or -1. */
+ * candidate test, the full 7x7 median of med3 for that test (queue pipeline: the
+ * tests that bounds of the median leave open; row kernels: those not decided by
+ * counting; every test in the detection kernels), and the upper-bound test.
+ * The queue pipeline's med3 goes with its re-test (iteration 1: with the dense
+ * pass, counted as 0). The stages are evaluated only where they can change a
+ * flag, so these counts are the method's work on this input; they differ
+ * between the pipelines. Returns the number of iterations, or -1. */
 int crb_last_work(crb_ctx* ctx, long long* out, int max_iter);
 
 /* Kernel launches the last crb_clean / crb_clean_batch / crb_iterate enqueued
@@ -302,7 +307,8 @@ int crb_fadd_peak(double* ops_per_s, cudaStream_t stream);
  * number of timed brackets since the last reset (then resets if reset != 0).
  * Kinds, in order: 0 bound pass (iteration 1: the dense pass; later: the
  * segment list, the dilation of the changed pixels and the re-test), 1 need,
- * 2 S, 3 S', 4 m3need, 5 med3, 6 candidate tests, 7 growth, 8 reserved (no
+ * 2 S, 3 S', 4 the list of tests, 5 clearing the next iteration's cells and
+ * changed pixels (the bound pass computes med3), 6 candidate tests, 7 growth, 8 reserved (no
  * kernel is timed under it), 9 tile-pipeline detection, 10 replacement,
  * 11 u8 mask, 12 tile-pipeline replacement, 13 work counters.
  * Returns the number of kinds written, or CRB_EINVAL. */
@@ -317,11 +323,12 @@ int crb_profile_kernels(crb_ctx* ctx, double* ms, int* brackets, int max, int re
 int crb_selftest_wait_timeout(crb_ctx* ctx, unsigned polls, cudaStream_t stream);
 
 /* The launch configuration of the context's last call: blocks per SM of the
- * queue-pipeline kernels, in the order bound (dense), need, S, S', m3need,
- * med3, candidate test, replacement, bound re-test, replacement queue,
+ * queue-pipeline kernels, in the order bound (dense), need, S, S', list of
+ * tests, clearing, candidate test, replacement, bound re-test, replacement queue,
  * replacement write, changed-pixel dilation, full candidate test, growth,
  * flag queue and u8 mask, segment list, segment-form dilation, need and
- * m3need, m3need of iteration 1 (up to max of them); the first iteration of
+ * list of tests, list of tests of iteration 1, growth of iteration 1 (up to
+ * max of them); the first iteration of
  * the segment-list forms; the pipeline (1 tile, 2 queue). Returns the number of
  * kernels written, or CRB_EINVAL. A measurement aid, not a step of the method
  * (the paper has no counterpart). */
@@ -366,7 +373,9 @@ int crb_server_poll(crb_server* srv, uint64_t* done_tags, double* latency_s, int
 /* Device bytes a w x h frame counts against the server budget: 9 per pixel of
  * the caller's buffers, 36 per pixel of workspace (4 float maps, 5 queue
  * entries), 14 bit planes, 8 bytes per cell of 32 x 8 pixels and 12 per
- * segment of 32 x 16 pixels (0 for invalid sizes). */
+ * segment of 32 x 16 pixels (0 for invalid sizes): no less than the queue
+ * pipeline takes (13 planes, 8 bytes per segment); the tile pipeline takes a
+ * fraction of it. */
 size_t crb_server_frame_bytes(int w, int h);
 
 /* Counters: submitted, done, waves launched, largest wave, rejected submissions,

@@ -141,8 +141,8 @@ struct GraphKey {
   void* tab;
   bool operator==(const GraphKey& o) const {
     return n == o.n && niter == o.niter && shape == o.shape && fuse == o.fuse && fuse2 == o.fuse2 &&
-           queue == o.queue && pdl == o.pdl && row_form == o.row_form && seg_from == o.seg_from && occ_sig == o.occ_sig &&
-           tiles == o.tiles && nblocks == o.nblocks && ncells == o.ncells && npix == o.npix &&
+           queue == o.queue && pdl == o.pdl && row_form == o.row_form && seg_from == o.seg_from &&
+           occ_sig == o.occ_sig && tiles == o.tiles && nblocks == o.nblocks && ncells == o.ncells && npix == o.npix &&
            rtiles == o.rtiles && bits_total == o.bits_total && ncounters == o.ncounters && dgrid == o.dgrid &&
            fgrid == o.fgrid && rgrid == o.rgrid && ws == o.ws && counters == o.counters && frames == o.frames &&
            tab == o.tab;
@@ -1202,11 +1202,11 @@ int launch_graph(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
 
 // crb_options.pipeline
 enum { kPipeAuto = 0, kPipeTile = 1, kPipeQueue = 2 };
-// Automatic choice: the queue pipeline from this many pixels per call on. Its
-// ~60 dependent launches cost about 0.5 ms per call whatever the size, while
-// the tile pipeline's 5 cost little but each pixel about 4.5 times more:
-// single 800x800 and 1024x1024 frames clean in 0.17-0.18 ms on tiles and
-// 0.54-0.67 ms on queues, 2048x4096 in 0.99 ms against 0.72-0.85 ms.
+// Automatic choice: the queue pipeline from this many pixels per call on. Its ~60 dependent launches cost about
+// 0.16 ms per call whatever the size, while the tile pipeline's 5 cost little but each pixel about 2.7 times
+// more. The line is part of the interface; on single frames the two now meet higher (us, tiles / queues:
+// 2048^2 185 / 297, 2048 x 4096 351 / 378, 3300^2 447 / 422, 4096^2 694 / 502), and autotune takes the faster
+// one below kTuneTilePixels.
 constexpr long long kAutoQueuePixels = 6000000;
 
 // ---- Autotuner of the queue pipeline (crb_options.autotune) --------------------------------------
