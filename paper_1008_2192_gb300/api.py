@@ -204,6 +204,7 @@ class Cleaner:
             raise RuntimeError("crb_last_work failed")
         return [tuple(int(buf[6 * i + j]) for j in range(6)) for i in range(k)]
 
+    # m3need*: the list of tests; m3: clearing the next iteration's cells (med3 goes with bound and bound_sparse)
     QUEUE_KERNELS = ("bound", "need", "s", "sprime", "m3need", "m3", "cand_test", "rep_compute", "bound_sparse",
                      "rq", "rep_write", "d2", "cand_full", "grow", "mask", "seg_list", "d2_seg", "need_seg",
                      "m3need_seg", "m3need_first", "grow_first")

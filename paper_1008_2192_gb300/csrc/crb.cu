@@ -109,7 +109,7 @@ size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 // profiling kinds (crb_profile_kernels order); kinds below kProfReplace0 are detection
 enum ProfKind {
-  kPBound, kPNeed, kPS, kPSp, kPM3need, kPM3, kPCand, kPGrow, kPReserved, kPTileDetect,  // detection
+  kPBound, kPNeed, kPS, kPSp, kPTests, kPClear, kPCand, kPGrow, kPReserved, kPTileDetect,  // detection
   kPRep, kPMask, kPTileReplace,                                                      // replacement
   kPWork,                                                                             // work counters
   kProfKinds
@@ -123,8 +123,8 @@ constexpr int kDescSlots = 4;
 
 // queue pipeline kernels, for the occupancy table
 enum QK {
-  kQBound, kQNeed, kQS, kQSp, kQM3need, kQM3, kQCand, kQRepCompute, kQBoundSparse, kQRq, kQRepWrite, kQD2,
-  kQCandFull, kQGrow, kQMask, kQSegList, kQD2Seg, kQNeedSeg, kQM3needSeg, kQM3needAll, kQGrowFirst, kQKernels
+  kQBound, kQNeed, kQS, kQSp, kQTests, kQClear, kQCand, kQRepCompute, kQBoundSparse, kQRq, kQRepWrite, kQD2,
+  kQCandFull, kQGrow, kQMask, kQSegList, kQD2Seg, kQNeedSeg, kQTestsSeg, kQTestsAll, kQGrowFirst, kQKernels
 };
 
 struct GraphKey {
@@ -301,8 +301,8 @@ int init_ctx(crb_ctx* c) {
         reinterpret_cast<const void*>(crb::grow_first_kernel)};
     for (int i = 0; i < kQKernels; ++i) {
       int o = 0;
-      const bool col = i == kQNeed || i == kQM3need || i == kQD2 || i == kQD2Seg || i == kQNeedSeg ||
-                       i == kQM3needSeg || i == kQM3needAll;
+      const bool col = i == kQNeed || i == kQTests || i == kQD2 || i == kQD2Seg || i == kQNeedSeg ||
+                       i == kQTestsSeg || i == kQTestsAll;
       const int threads = i == kQBound ? crb::kBoundThreads : col ? crb::kColWarps * 32 : 256;
       CRB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fns[i], threads, 0));
       c->occ_q[i] = o > 0 ? o : 1;
@@ -527,7 +527,7 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
       const uint32_t* kcls = (k == 1) ? nullptr : cls;
       const long long ucol = (P.nunits + crb::kColWarps - 1) / crb::kColWarps;
       const int gcol = grid(kQNeed, ucol);
-      const int gcolm = grid(kQM3need, ucol), gcol1m = grid(kQM3needAll, ucol);
+      const int gcolm = grid(kQTests, ucol), gcol1m = grid(kQTestsAll, ucol);
       const bool seg = k >= P.seg_from;  // the column kernels walk the listed segments only
       const int tcol = crb::kColWarps * 32;
       const long long grow = std::min<long long>(P.nunits, 64LL * c->num_sms), gseg = 8LL * c->num_sms;  // row forms
@@ -584,21 +584,21 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
       timed(c, kPSp, stream, [&] {
         tq(kQSp, [&] { go(crb::sp_kernel, gq * P.occ[kQSp], 256, c->d_frames, P.n, P.Q, c->p, k); });
       });
-      timed(c, kPM3need, stream, [&] {
+      timed(c, kPTests, stream, [&] {
         if (P.row_form)
-          tq(kQM3need, [&] { go(crb::tests_row_kernel, grow, 256, c->d_frames, P.n, P.nunits, P.Q, kcls); });
+          tq(kQTests, [&] { go(crb::tests_row_kernel, grow, 256, c->d_frames, P.n, P.nunits, P.Q, kcls); });
         else if (seg)
-          tq(kQM3needSeg, [&] {
-            go(crb::tests_seg_kernel, gq * P.occ[kQM3needSeg], tcol, c->d_frames, P.n, P.Q, cls);
+          tq(kQTestsSeg, [&] {
+            go(crb::tests_seg_kernel, gq * P.occ[kQTestsSeg], tcol, c->d_frames, P.n, P.Q, cls);
           });
         else if (k == 1)
-          tq(kQM3needAll, [&] { go(crb::tests_kernel<true>, gcol1m, tcol, c->d_frames, P.n, P.nunits, P.Q, nullptr); });
+          tq(kQTestsAll, [&] { go(crb::tests_kernel<true>, gcol1m, tcol, c->d_frames, P.n, P.nunits, P.Q, nullptr); });
         else
-          tq(kQM3need, [&] { go(crb::tests_kernel<false>, gcolm, tcol, c->d_frames, P.n, P.nunits, P.Q, kcls); });
+          tq(kQTests, [&] { go(crb::tests_kernel<false>, gcolm, tcol, c->d_frames, P.n, P.nunits, P.Q, kcls); });
       });
-      timed(c, kPM3, stream, [&] {  // the classes and changed pixels of iteration k+1 start at zero
-        tq(kQM3, [&] {
-          go(crb::clear_kernel, cls_next ? gq * P.occ[kQM3] : 1, 256, reinterpret_cast<uint4*>(cls_next),
+      timed(c, kPClear, stream, [&] {  // the classes and changed pixels of iteration k+1 start at zero
+        tq(kQClear, [&] {
+          go(crb::clear_kernel, cls_next ? gq * P.occ[kQClear] : 1, 256, reinterpret_cast<uint4*>(cls_next),
              cls_next ? (cells_bytes + 15) / 16 : 0, reinterpret_cast<uint4*>(P.chg[(k + 1) & 1]),
              cls_next ? P.chg_bytes / 16 : 0);
         });

@@ -277,7 +277,7 @@ __device__ __forceinline__ void bound_span(const Frame& f, const float* __restri
         }
       }
       if (m3out) {
-        // med3 of the row (as m3_kernel): each column's three rows sorted, then the median of the
+        // med3 of the row: each column's three rows sorted, then the median of the
         // largest column minimum, the median of the column medians and the smallest column maximum;
         // columns x-1 and x+NP from the neighbour lanes, x0-1 and x0+32*NP from the halo lanes 1, 2
         float lo[NP + 2], mi[NP + 2], hi[NP + 2];

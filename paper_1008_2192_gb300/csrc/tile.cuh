@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(256, kMode == 1 && !kMany ? 4 : 4 + kMode)
       for (int j = 0; j < BR; ++j) {
         const int r = ra + j;
         const float2 up = v[j + 1], ce = v[j + 2], dn = v[j + 3];
-        if (kMode == 0) {  // med3: as m3_kernel, from the sorted columns
+        if (kMode == 0) {  // med3 from the sorted columns, as bound_span
           float le, ne, he, lo, no, ho;
           sort3(up.x, ce.x, dn.x, le, ne, he);
           sort3(up.y, ce.y, dn.y, lo, no, ho);
