@@ -7,6 +7,7 @@
 // so descriptors and workspace can be reused.
 
 #include <algorithm>
+#include <array>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -127,28 +128,6 @@ enum QK {
   kQCandFull, kQGrow, kQMask, kQSegList, kQD2Seg, kQNeedSeg, kQTestsSeg, kQTestsAll, kQGrowFirst, kQKernels
 };
 
-struct GraphKey {
-  int n, niter, shape;
-  bool fuse, fuse2, queue, pdl, row_form;
-  int seg_from;
-  long long occ_sig;  // the queue kernels' blocks per SM, packed
-  long long tiles, rtiles, nblocks, ncells, npix;
-  size_t bits_total;
-  int ncounters, dgrid, fgrid, rgrid;
-  void* ws;
-  void* counters;
-  void* frames;
-  void* tab;
-  bool operator==(const GraphKey& o) const {
-    return n == o.n && niter == o.niter && shape == o.shape && fuse == o.fuse && fuse2 == o.fuse2 &&
-           queue == o.queue && pdl == o.pdl && row_form == o.row_form && seg_from == o.seg_from &&
-           occ_sig == o.occ_sig && tiles == o.tiles && nblocks == o.nblocks && ncells == o.ncells && npix == o.npix &&
-           rtiles == o.rtiles && bits_total == o.bits_total && ncounters == o.ncounters && dgrid == o.dgrid &&
-           fgrid == o.fgrid && rgrid == o.rgrid && ws == o.ws && counters == o.counters && frames == o.frames &&
-           tab == o.tab;
-  }
-};
-
 struct FrameSpec {
   const float* img;
   float* out_clean;
@@ -157,6 +136,36 @@ struct FrameSpec {
   const uint8_t* mprev;  // crb_iterate only
   int w, h;
   float gain, rn;
+};
+
+// What a call's launches are laid out by: niter and the sizes of its frames in order.
+std::vector<long long> call_signature(const std::vector<FrameSpec>& specs, int niter) {
+  std::vector<long long> sig{niter};
+  for (const auto& s : specs) {
+    sig.push_back(s.w);
+    sig.push_back(s.h);
+  }
+  return sig;
+}
+
+// A captured graph holds the launches' grids and arguments by value: offsets into the workspace and counts of
+// strips, cells and tiles, all functions of the signature and the choice of kernels, and the addresses of the
+// context's buffers. Sums over the frames do not tell calls apart: 4096 x 2560 and 2560 x 4096 agree in pixels,
+// words, cells and tiles but have 640 and 768 strips.
+struct GraphKey {
+  std::vector<long long> sig;
+  int shape, seg_from;
+  bool fuse, fuse2, queue, pdl, row_form;
+  std::array<int, kQKernels> occ;
+  void* ws;
+  void* counters;
+  void* frames;
+  void* tab;
+  bool operator==(const GraphKey& o) const {
+    return sig == o.sig && shape == o.shape && seg_from == o.seg_from && fuse == o.fuse && fuse2 == o.fuse2 &&
+           queue == o.queue && pdl == o.pdl && row_form == o.row_form && occ == o.occ && ws == o.ws &&
+           counters == o.counters && frames == o.frames && tab == o.tab;
+  }
 };
 
 }  // namespace
@@ -1166,12 +1175,9 @@ int upload(crb_ctx* c, const Plan& P, cudaStream_t stream) {
 
 // Replays (or captures once) the work of plan P as a CUDA graph on `stream`.
 int launch_graph(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs, cudaStream_t stream) {
-  long long occ_sig = 0;
-  for (int i = 0; i < kQKernels; ++i) occ_sig = occ_sig * 31 + P.occ[i];
-  GraphKey key{P.n,       P.niter,  P.shape,   P.fuse,  P.fuse2,  P.queue,      P.pdl,
-               P.row_form, P.seg_from, occ_sig, P.tiles, P.rtiles, P.nblocks,   P.ncells,
-               P.npix,    P.bits_total, P.ncounters, P.dgrid, P.fgrid, P.rgrid, c->ws,
-               c->d_counters, c->d_frames, P.queue ? c->d_tab : nullptr};
+  GraphKey key{call_signature(specs, P.niter), P.shape, P.seg_from, P.fuse, P.fuse2, P.queue, P.pdl, P.row_form, {},
+               c->ws, c->d_counters, c->d_frames, P.queue ? c->d_tab : nullptr};
+  std::copy(P.occ, P.occ + kQKernels, key.occ.begin());
   for (auto& g : c->graphs)
     if (g.first == key) {
       CRB_CUDA(cudaGraphLaunch(g.second, stream));
@@ -1359,11 +1365,7 @@ int run(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool maps, c
                             (c->opt.pipeline == kPipeAuto && npix >= kAutoQueuePixels));
   const crb_ctx::QTune* tuned = nullptr;
   if (c->opt.autotune && queue_ok && c->opt.pipeline != kPipeTile) {
-    std::vector<long long> sig{niter};
-    for (const auto& s : specs) {
-      sig.push_back(s.w);
-      sig.push_back(s.h);
-    }
+    const std::vector<long long> sig = call_signature(specs, niter);
     for (const auto& t : c->qtuned)
       if (t.sig == sig) tuned = &t;
     if (!tuned) {
@@ -1381,11 +1383,7 @@ int run(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool maps, c
   if (c->opt.fuse2) shape = kFuse2Shape;
   if (shape < 0 && !maps && !queue) {
     // autotuning: the first call of a signature (frame sizes, niter) times every tile shape
-    std::vector<long long> sig{niter};
-    for (const auto& s : specs) {
-      sig.push_back(s.w);
-      sig.push_back(s.h);
-    }
+    const std::vector<long long> sig = call_signature(specs, niter);
     shape = -1;
     for (const auto& t : c->tuned)
       if (t.first == sig) shape = t.second;
