@@ -67,9 +67,12 @@ typedef struct {
   int early_exit;
   /* Tile shape of the tile pipeline (index of crb_tile_shape; default 0).
    * 0 takes the row kernels (48-px wide tiles of 30 rows, or of 14 where those
-   * number at most one per SM), or 64 x 32 tiles where a call asks for what
-   * they do not have: map export, a given mask, no_fusion or fuse2. Any other
-   * index takes that shape's detection kernel. -1 = autotune: the first call with a new signature (the list of frame
+   * number at most one per SM). Where a call asks for what they do not have it
+   * takes detection kernels: 64 x 32 tiles with map export; with a given mask or
+   * no_fusion those, or the 64 x 28 tiles of index 5 (three blocks per SM) when
+   * all of a call's tiles then fit in one round of resident blocks and the 64 x
+   * 32 tiles do not (one 800 x 800 frame); those of index 2 with fuse2. Any
+   * other index takes that shape's detection kernel. -1 = autotune: the first call with a new signature (the list of frame
    * sizes and niter) runs the clean once per compiled shape, timing each on
    * the stream (that call synchronises the stream), and keeps the fastest for
    * later calls with the same signature. */

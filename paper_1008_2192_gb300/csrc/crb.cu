@@ -73,7 +73,12 @@ const std::vector<DetectShape>& detect_shapes() {
   return v;
 }
 
-// Three blocks of this shape per SM need the largest shared-memory carveout.
+// The detection kernels that tile_shape 0 takes where a call asks for what the row kernels do not have
+// (default_shape): 64 x 32 tiles, or the single-buffered 64 x 28 tiles when all of those fit in one round of
+// resident blocks (three per SM, which need the largest shared-memory carveout) and the 64 x 32 tiles do not. A
+// tile's detection is a chain of block-wide phases whose latency bounds the launch, so a second round of a few
+// tiles costs nearly a whole tile latency: on 800 x 800, 325 tiles of 64 x 32 on 152 SMs x 2 blocks against 377 of
+// 64 x 28 on 152 x 3, a clean without fusion takes 177 / 146 us, an iteration with a given mask 65 / 55 us.
 constexpr int kOneRoundShape = 5;
 
 // The row kernels (tile.cuh) by tile height.
@@ -1273,11 +1278,24 @@ bool takes_rows(const crb_ctx* c, const std::vector<FrameSpec>& specs, bool maps
   return tiles < (1LL << 31);
 }
 
+// The detection kernels' shape that tile_shape 0 takes for a call without the row kernels (see kOneRoundShape).
+int default_shape(const crb_ctx* c, const std::vector<FrameSpec>& specs) {
+  const auto& v = detect_shapes();
+  auto one_round = [&](int i) {
+    const DetectShape& d = v[size_t(i)];
+    long long tiles = 0;
+    for (const auto& s : specs) tiles += (long long)((s.w + d.tw - 1) / d.tw) * ((s.h + d.th - 1) / d.th);
+    return tiles <= (long long)c->num_sms * std::min(c->occ_detect[size_t(i)], c->occ_fused[size_t(i)]);
+  };
+  return one_round(kOneRoundShape) && !one_round(0) ? kOneRoundShape : 0;
+}
+
 // Times one tile-pipeline clean (with the kernels tile_shape 0 takes when that
 // is the option, else 64 x 32 tiles), synchronising `stream`.
 int trial_tile(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, cudaStream_t stream, float* ms) {
   Plan P;
-  int rc = takes_rows(c, specs, false) ? prepare_tile(c, specs, niter, P) : prepare(c, specs, niter, false, 0, P);
+  int rc = takes_rows(c, specs, false) ? prepare_tile(c, specs, niter, P)
+                                        : prepare(c, specs, niter, false, c->opt.tile_shape == 0 ? default_shape(c, specs) : 0, P);
   if (rc == CRB_OK) rc = upload(c, P, stream);
   if (rc) return rc;
   cudaEvent_t a = take_event(c), b = take_event(c);
@@ -1421,6 +1439,7 @@ int run(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool maps, c
     }
   }
   if (shape < 0) shape = 0;
+  if (shape == 0 && c->opt.tile_shape == 0 && !maps && !queue) shape = default_shape(c, specs);
   Plan P;
   int rc = queue ? prepare_queue(c, specs, niter, P)
                  : takes_rows(c, specs, maps) ? prepare_tile(c, specs, niter, P)

@@ -62,3 +62,13 @@ def test_server_of_transposed_frames():
             assert torch.equal(m, want[i][1]) and torch.equal(o, want[i][0]), i
     finally:
         srv.close()
+
+
+@pytest.mark.parametrize("w,h", [(800, 800), (768, 616), (1216, 670), (1217, 700)])
+def test_separate_launches_by_rounds_of_tiles(w, h):
+    """Without fusion, tile_shape 0 takes 64x32 tiles or, where only those of 64x28 fit one round of resident blocks
+    (the first and third), these: sizes either side of both lines equal the FP32 oracle."""
+    img = synth.frame(w, h, seed=85)
+    out, mask = gpu_clean(Cleaner(niter=3, pipeline="tile", fusion=False), img)
+    r32 = oracle.clean(img, params_of({}), 3, precision="f32")
+    assert np.array_equal(mask, r32.mask) and np.array_equal(out, r32.clean)
