@@ -72,10 +72,12 @@ typedef struct {
    * no_fusion those, or the 64 x 28 tiles of index 5 (three blocks per SM) when
    * all of a call's tiles then fit in one round of resident blocks and the 64 x
    * 32 tiles do not (one 800 x 800 frame); those of index 2 with fuse2. Any
-   * other index takes that shape's detection kernel. -1 = autotune: the first call with a new signature (the list of frame
-   * sizes and niter) runs the clean once per compiled shape, timing each on
-   * the stream (that call synchronises the stream), and keeps the fastest for
-   * later calls with the same signature. */
+   * other index takes that shape's detection kernel (one past the last: 64 x 32).
+   * -1 = autotune: the first call with a new signature (the list of frame sizes
+   * and niter) runs the clean twice with the row kernels, where it can take them,
+   * and twice with each compiled shape, timing each on the stream (that call
+   * synchronises the stream), and keeps the fastest for itself and later calls
+   * with the same signature. */
   int tile_shape;
   /* 1: capture the work of a call (the niter loop of launches, with the memsets
    * of calls that have them) in a CUDA graph once per launch signature and

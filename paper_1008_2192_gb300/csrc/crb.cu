@@ -1228,9 +1228,29 @@ constexpr long long kAutoQueuePixels = 6000000;
 // therefore times trial cleans of the call's own frames and keeps the fastest
 // configuration for the call signature (frame sizes and niter).
 
+// Times one clean by plan P from its upload on (the row kernels' first iteration runs beside it),
+// synchronising `stream`.
+int trial(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs, cudaStream_t stream, float* ms) {
+  cudaEvent_t a = take_event(c), b = take_event(c);
+  auto timed_clean = [&]() -> int {
+    CRB_CUDA(cudaEventRecord(a, stream));
+    int rc = upload(c, P, stream);
+    if (rc == CRB_OK) rc = enqueue_work(c, P, specs, stream);
+    if (rc) return rc;
+    CRB_CUDA(cudaEventRecord(b, stream));
+    CRB_CUDA(cudaEventSynchronize(b));
+    CRB_CUDA(cudaEventElapsedTime(ms, a, b));
+    return CRB_OK;
+  };
+  const int rc = timed_clean();
+  c->ev_pool.push_back(a);
+  c->ev_pool.push_back(b);
+  return rc;
+}
+
 // Times one queue-pipeline clean of specs with blocks per SM occ[] and segment
-// lists from iteration seg_from, synchronising `stream`; per_kernel (if not
-// NULL) receives the device time of each kernel summed over its launches.
+// lists from iteration seg_from; per_kernel (if not NULL) receives the device
+// time of each kernel summed over its launches.
 int trial_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, const int* occ, int seg_from,
                 cudaStream_t stream, float* ms, double* per_kernel) {
   Plan P;
@@ -1238,19 +1258,10 @@ int trial_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, cons
   if (rc) return rc;
   std::copy(occ, occ + kQKernels, P.occ);
   P.seg_from = seg_from;
-  rc = upload(c, P, stream);
-  if (rc) return rc;
-  cudaEvent_t a = take_event(c), b = take_event(c);
-  CRB_CUDA(cudaEventRecord(a, stream));
   c->tuning = per_kernel != nullptr;
-  rc = enqueue_work(c, P, specs, stream);
+  rc = trial(c, P, specs, stream, ms);
   c->tuning = false;
   if (rc) return rc;
-  CRB_CUDA(cudaEventRecord(b, stream));
-  CRB_CUDA(cudaEventSynchronize(b));
-  CRB_CUDA(cudaEventElapsedTime(ms, a, b));
-  c->ev_pool.push_back(a);
-  c->ev_pool.push_back(b);
   if (per_kernel) {
     std::fill(per_kernel, per_kernel + kQKernels, 0.0);
     for (auto& e : c->tune_ev) {
@@ -1265,11 +1276,10 @@ int trial_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, cons
   return CRB_OK;
 }
 
-// Whether a tile-pipeline call takes the row kernels (tile.cuh): tile_shape 0
-// without map export, a given mask or the options that ask for other launches.
-// The tile count must fit a grid.
-bool takes_rows(const crb_ctx* c, const std::vector<FrameSpec>& specs, bool maps) {
-  if (maps || c->opt.no_fusion || c->opt.fuse2 || c->opt.tile_shape != 0) return false;
+// Whether the row kernels (tile.cuh) can take a call: no map export, given mask
+// or options that ask for other launches. The tile count must fit a grid.
+bool rows_possible(const crb_ctx* c, const std::vector<FrameSpec>& specs, bool maps) {
+  if (maps || c->opt.no_fusion || c->opt.fuse2) return false;
   long long tiles = 0;
   for (const auto& s : specs) {
     if (s.mprev) return false;
@@ -1290,24 +1300,61 @@ int default_shape(const crb_ctx* c, const std::vector<FrameSpec>& specs) {
   return one_round(kOneRoundShape) && !one_round(0) ? kOneRoundShape : 0;
 }
 
-// Times one tile-pipeline clean (with the kernels tile_shape 0 takes when that
-// is the option, else 64 x 32 tiles), synchronising `stream`.
+// The tile pipeline's kernels for a call: an index of detect_shapes, or the row kernels.
+constexpr int kTileRows = -1;
+
+int prepare_choice(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool maps, int choice, Plan& P) {
+  return choice == kTileRows ? prepare_tile(c, specs, niter, P) : prepare(c, specs, niter, maps, choice, P);
+}
+
+// The choice crb_options.tile_shape makes for a call. -1: the fastest of the row
+// kernels and every detection shape, timed (best of two cleans each,
+// synchronising `stream`) at the first call of its signature; with map export, 0.
+int tile_choice(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool maps, cudaStream_t stream,
+                int* choice) {
+  const int nshapes = int(detect_shapes().size()), opt = c->opt.tile_shape;
+  const bool rows = rows_possible(c, specs, maps);
+  if (c->opt.fuse2) {
+    *choice = kFuse2Shape;
+  } else if (opt >= 0 || maps) {
+    *choice = opt > 0 && opt < nshapes ? opt : opt != 0 || maps ? 0 : rows ? kTileRows : default_shape(c, specs);
+  } else {
+    std::vector<long long> sig = call_signature(specs, niter);
+    sig.push_back(rows);
+    for (const auto& t : c->tuned)
+      if (t.first == sig) {
+        *choice = t.second;
+        return CRB_OK;
+      }
+    const int saved_profile = c->opt.profile;
+    c->opt.profile = 0;  // trials are not profiled
+    float best = 1e30f;
+    int rc = CRB_OK;
+    for (int sh = rows ? kTileRows : 0; sh < nshapes && rc == CRB_OK; ++sh)
+      for (int rep = 0; rep < 2 && rc == CRB_OK; ++rep) {
+        Plan P;
+        float ms = 0.f;
+        rc = prepare_choice(c, specs, niter, maps, sh, P);
+        if (rc == CRB_OK) rc = trial(c, P, specs, stream, &ms);
+        if (rc == CRB_OK && ms < best) {
+          best = ms;
+          *choice = sh;
+        }
+      }
+    c->opt.profile = saved_profile;
+    if (rc) return rc;
+    c->tuned.emplace_back(sig, *choice);
+  }
+  return CRB_OK;
+}
+
+// Times one tile-pipeline clean with the kernels the call would take, synchronising `stream`.
 int trial_tile(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, cudaStream_t stream, float* ms) {
   Plan P;
-  int rc = takes_rows(c, specs, false) ? prepare_tile(c, specs, niter, P)
-                                        : prepare(c, specs, niter, false, c->opt.tile_shape == 0 ? default_shape(c, specs) : 0, P);
-  if (rc == CRB_OK) rc = upload(c, P, stream);
-  if (rc) return rc;
-  cudaEvent_t a = take_event(c), b = take_event(c);
-  CRB_CUDA(cudaEventRecord(a, stream));
-  rc = enqueue_work(c, P, specs, stream);
-  if (rc) return rc;
-  CRB_CUDA(cudaEventRecord(b, stream));
-  CRB_CUDA(cudaEventSynchronize(b));
-  CRB_CUDA(cudaEventElapsedTime(ms, a, b));
-  c->ev_pool.push_back(a);
-  c->ev_pool.push_back(b);
-  return CRB_OK;
+  int choice = 0;
+  int rc = tile_choice(c, specs, niter, false, stream, &choice);
+  if (rc == CRB_OK) rc = prepare_choice(c, specs, niter, false, choice, P);
+  return rc ? rc : trial(c, P, specs, stream, ms);
 }
 
 // Calls below this many pixels also try the tile pipeline.
@@ -1373,7 +1420,6 @@ int tune_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, long 
 
 // Enqueues the whole clean of `specs` (niter iterations) on `stream`.
 int run(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool maps, cudaStream_t stream) {
-  const int nshapes = int(detect_shapes().size());
   if (c->any_call) CRB_CUDA(cudaStreamWaitEvent(stream, c->done_ev, 0));
   long long npix = 0;
   for (const auto& s : specs) npix += (long long)s.w * s.h;
@@ -1396,54 +1442,11 @@ int run(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool maps, c
     }
     queue = !tuned->tile;
   }
-  int shape = c->opt.tile_shape;
-  if (shape >= nshapes) shape = 0;
-  if (c->opt.fuse2) shape = kFuse2Shape;
-  if (shape < 0 && !maps && !queue) {
-    // autotuning: the first call of a signature (frame sizes, niter) times every tile shape
-    const std::vector<long long> sig = call_signature(specs, niter);
-    shape = -1;
-    for (const auto& t : c->tuned)
-      if (t.first == sig) shape = t.second;
-    if (shape < 0) {
-      float best = 0.f;
-      int best_shape = 0;
-      cudaEvent_t a = nullptr, b = nullptr;
-      CRB_CUDA(cudaEventCreate(&a));
-      CRB_CUDA(cudaEventCreate(&b));
-      for (int sh = 0; sh < nshapes; ++sh) {
-        Plan P;
-        int rc = prepare(c, specs, niter, maps, sh, P);
-        if (rc == CRB_OK) rc = upload(c, P, stream);
-        if (rc == CRB_OK && cudaEventRecord(a, stream) != cudaSuccess) rc = CRB_ECUDA;
-        if (rc == CRB_OK) rc = enqueue_work(c, P, specs, stream);
-        float ms = 0.f;
-        if (rc == CRB_OK && (cudaEventRecord(b, stream) != cudaSuccess || cudaEventSynchronize(b) != cudaSuccess ||
-                             cudaEventElapsedTime(&ms, a, b) != cudaSuccess))
-          rc = CRB_ECUDA;
-        if (rc != CRB_OK) {
-          cudaEventDestroy(a);
-          cudaEventDestroy(b);
-          return rc;
-        }
-        if (sh == 0 || ms < best) {
-          best = ms;
-          best_shape = sh;
-        }
-      }
-      cudaEventDestroy(a);
-      cudaEventDestroy(b);
-      c->tuned.emplace_back(sig, best_shape);
-      // every trial produced the same outputs; the last one stays
-      return finish(c, stream);
-    }
-  }
-  if (shape < 0) shape = 0;
-  if (shape == 0 && c->opt.tile_shape == 0 && !maps && !queue) shape = default_shape(c, specs);
   Plan P;
-  int rc = queue ? prepare_queue(c, specs, niter, P)
-                 : takes_rows(c, specs, maps) ? prepare_tile(c, specs, niter, P)
-                                              : prepare(c, specs, niter, maps, shape, P);
+  int choice = 0;
+  int rc = queue ? CRB_OK : tile_choice(c, specs, niter, maps, stream, &choice);
+  if (rc == CRB_OK)
+    rc = queue ? prepare_queue(c, specs, niter, P) : prepare_choice(c, specs, niter, maps, choice, P);
   if (rc) return rc;
   if (queue && tuned) {
     std::copy(tuned->occ, tuned->occ + kQKernels, P.occ);

@@ -72,3 +72,68 @@ def test_separate_launches_by_rounds_of_tiles(w, h):
     out, mask = gpu_clean(Cleaner(niter=3, pipeline="tile", fusion=False), img)
     r32 = oracle.clean(img, params_of({}), 3, precision="f32")
     assert np.array_equal(mask, r32.mask) and np.array_equal(out, r32.clean)
+
+
+@pytest.mark.parametrize("autotune", [False, True], ids=["shapes", "pipelines-too"])
+def test_autotuned_shape_is_the_fastest(autotune):
+    """tile_shape -1 tries the row kernels beside the detection shapes, none of which is within a factor of two of
+    them here, and the trial of the tile pipeline against the queue pipeline runs what the call then takes. The work
+    counters tell the kernels apart: the row kernels decide the objlim tests by counting, the others by a 7x7 median each."""
+    for w, h in ((800, 800), (2048, 1100)):
+        img = synth.frame(w, h, seed=87)
+        want = Cleaner(niter=4, pipeline="tile")
+        o, m = gpu_clean(want, img)
+        c = Cleaner(niter=4, tile_shape=-1, pipeline="auto" if autotune else "tile", autotune=autotune)
+        for _ in range(2):
+            out, mask = gpu_clean(c, img)
+            assert np.array_equal(mask, m) and np.array_equal(out, o)
+            assert c.last_work() == want.last_work() and c.tuned_config()[2] == "tile"
+            assert c.last_launches() == want.last_launches()
+
+
+@pytest.mark.parametrize("kw", [dict(fusion=False), dict(fuse2=True), dict(tile_shape=1), dict(tile_shape=99), dict(tile_shape=-1)],
+                         ids=["two-launch", "two-iterations", "shape-1", "past-the-last", "tuned-shape"])
+def test_autotune_with_tile_options(kw):
+    """The tile pipeline that the autotuner tries is the one the options ask for: results of the first (tuning) and
+    later calls equal the FP32 oracle."""
+    img = synth.frame(500, 331, seed=88)
+    r32 = oracle.clean(img, params_of({}), 4, precision="f32")
+    c = Cleaner(niter=4, autotune=True, **kw)
+    for _ in range(2):
+        out, mask = gpu_clean(c, img)
+        assert np.array_equal(mask, r32.mask) and np.array_equal(out, r32.clean)
+
+
+@pytest.mark.parametrize("given", [False, True])
+def test_given_mask_does_not_take_the_tuned_row_kernels(given):
+    """A handle tuned to the row kernels by a call without a previous mask keeps to the detection kernels where one is
+    given, and the other way round."""
+    img = synth.frame(300, 200, seed=89)
+    M = np.zeros(img.shape, np.uint8)
+    M[::7, ::5] = 1
+    c = Cleaner(niter=1, tile_shape=-1, pipeline="tile")
+    for k in (0, 1, 0, 1):
+        mp = M if bool(k) != given else None
+        r = oracle.iterate(img, M if mp is not None else np.zeros_like(M), params_of({}), precision="f32")
+        gJ, gM, _ = c.iterate(dev(img), dev(mp) if mp is not None else None)
+        c.sync()
+        assert np.array_equal(host(gM), r.Mk) and np.array_equal(host(gJ), r.Ik), k
+
+
+@pytest.mark.parametrize("niter", [2, 4])
+def test_fused_64x32_tiles_and_graphs_of_shapes(niter):
+    """The fused 64x32 detection kernel (an index past the last) and the capture of detection kernels in a graph,
+    both launched and replayed, on a frame of several tiles with remainders and on a batch."""
+    img = synth.frame(333, 251, seed=90)
+    r32 = oracle.clean(img, params_of({}), niter, precision="f32")
+    for shape in (99, 1, 5):
+        for graphs in (False, True):
+            c = Cleaner(niter=niter, tile_shape=shape, use_graphs=graphs, pipeline="tile")
+            for _ in range(2):
+                out, mask = gpu_clean(c, img)
+                assert np.array_equal(mask, r32.mask) and np.array_equal(out, r32.clean), (shape, graphs)
+            outs, masks = c.clean_batch([dev(img), dev(img[:97].copy())])
+            c.sync()
+            r2 = oracle.clean(img[:97].copy(), params_of({}), niter, precision="f32")
+            assert np.array_equal(host(masks[0]), r32.mask) and np.array_equal(host(outs[0]), r32.clean)
+            assert np.array_equal(host(masks[1]), r2.mask) and np.array_equal(host(outs[1]), r2.clean)
