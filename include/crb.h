@@ -111,7 +111,7 @@ typedef struct {
    * largest blocks per SM), each kernel keeping the level at which its own
    * launches took least device time; then the first iteration from which the
    * bit-plane kernels walk listed segments (2, 3, 4 or none); then, for calls
-   * under 10,000,000 pixels with pipeline 0, the tile pipeline against the result.
+   * under 2^25 pixels with pipeline 0, the tile pipeline against the result.
    * Later calls with the same signature reuse the choice (crb_tuned_config
    * reports it). The launch configuration changes no result. Default 0. */
   int autotune;

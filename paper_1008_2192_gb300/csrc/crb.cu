@@ -1258,6 +1258,7 @@ int trial_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, cons
   if (rc) return rc;
   std::copy(occ, occ + kQKernels, P.occ);
   P.seg_from = seg_from;
+  P.pdl = true;  // a graph's replay takes what launches ahead of time take, not plain ones (4096^2: 509, 506, 639 us)
   c->tuning = per_kernel != nullptr;
   rc = trial(c, P, specs, stream, ms);
   c->tuning = false;
@@ -1357,8 +1358,11 @@ int trial_tile(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, cudaS
   return rc ? rc : trial(c, P, specs, stream, ms);
 }
 
-// Calls below this many pixels also try the tile pipeline.
-constexpr long long kTuneTilePixels = 10000000;
+// Calls below this many pixels also try the tile pipeline. On frames of the usual content the queue pipeline is the
+// faster one from about 10 Mpix on (486 us against 458 on five frames of 11.3 Mpix, 664 / 651 on 170 of 256 x 256,
+// 1019 / 690 on 36 of 800 x 800), but with many flags the tiles keep ahead far above that (3300 x 3300, tiles /
+// queues: pure noise at sigclip 2.5 2722 / 4842 us, 50 times the cosmic rays 1578 / 2212, niter 8 605 / 645).
+constexpr long long kTuneTilePixels = 1LL << 25;
 
 // Tunes the queue pipeline for specs: (1) four occupancy levels (all, 3/4, 1/2,
 // 1/4 of each kernel's largest blocks per SM), each kernel keeping the level at
@@ -1367,7 +1371,7 @@ constexpr long long kTuneTilePixels = 10000000;
 // by 2 %; (2) the first iteration of the segment-list forms (2, 3, 4 or none),
 // by the time of the whole clean (best of two), another than the default only
 // if it wins by 1 %; (3) below kTuneTilePixels, the tile pipeline against the
-// result. The margins keep timing noise from deciding.
+// result, taken if it wins by 1 %. The margins keep timing noise from deciding.
 int tune_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, long long npix, bool may_tile,
                cudaStream_t stream, crb_ctx::QTune& t) {
   const int saved_profile = c->opt.profile;
@@ -1412,7 +1416,7 @@ int tune_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, long 
       rc = trial_tile(c, specs, niter, stream, &ms);
       m = std::min(m, ms);
     }
-    t.tile = m < best_ms;
+    t.tile = m < 0.99f * best_ms;
   }
   c->opt.profile = saved_profile;
   return rc;

@@ -137,3 +137,20 @@ def test_fused_64x32_tiles_and_graphs_of_shapes(niter):
             r2 = oracle.clean(img[:97].copy(), params_of({}), niter, precision="f32")
             assert np.array_equal(host(masks[0]), r32.mask) and np.array_equal(host(outs[0]), r32.clean)
             assert np.array_equal(host(masks[1]), r2.mask) and np.array_equal(host(outs[1]), r2.clean)
+
+
+@pytest.mark.parametrize("graphs", [False, True])
+def test_autotune_finds_the_tile_pipeline_above_10_mpix(graphs):
+    """On a frame of noise with flags everywhere the tile pipeline takes little more than half the queue pipeline's
+    time; the tuner tries it up to 2^25 pixels, and the result is the same."""
+    rng = np.random.default_rng(91)
+    x = dev((rng.standard_normal((3300, 3300)) * 50 + 200).astype(np.float32))
+    q = Cleaner(niter=2, sigclip=2.5, pipeline="queue")
+    wo, wm = q.clean(x)
+    q.sync()
+    c = Cleaner(niter=2, sigclip=2.5, autotune=True, use_graphs=graphs)
+    for _ in range(2):
+        o, m = c.clean(x)
+        c.sync()
+        assert torch.equal(m, wm) and torch.equal(o, wo)
+    assert c.tuned_config()[2] == "tile"
