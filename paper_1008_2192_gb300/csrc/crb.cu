@@ -82,16 +82,21 @@ const std::vector<DetectShape>& detect_shapes() {
 constexpr int kOneRoundShape = 5;
 
 // The row kernels (tile.cuh) by tile height.
+using TileFn = void (*)(const crb::Frame*, int, crb::Params, int, int, int, const crb::Frame);
 struct TileKernels {
   int th;
-  void (*fn[3])(const crb::Frame*, int, crb::Params, int, int, const crb::Frame);  // iteration 1, later ones, the last replacement
-  int smem[3];
+  TileFn fn[2][3];  // a batch, one frame: iteration 1, later ones, the last replacement
+  int smem[3], blocks[3];
 };
 template <int TH, bool kMany>
 constexpr TileKernels make_tile() {
   return TileKernels{TH,
-                     {crb::tile_kernel<TH, 0, false>, crb::tile_kernel<TH, 1, kMany>, crb::tile_kernel<TH, 2, false>},
-                     {crb::TileLayout<TH, 0>::bytes, crb::TileLayout<TH, 1>::bytes, crb::TileLayout<TH, 2>::bytes}};
+                     {{crb::tile_kernel<TH, 0, false, false>, crb::tile_kernel<TH, 1, kMany, false>,
+                       crb::tile_kernel<TH, 2, false, false>},
+                      {crb::tile_kernel<TH, 0, false, true>, crb::tile_kernel<TH, 1, kMany, true>,
+                       crb::tile_kernel<TH, 2, false, true>}},
+                     {crb::TileLayout<TH, 0>::bytes, crb::TileLayout<TH, 1>::bytes, crb::TileLayout<TH, 2>::bytes},
+                     {crb::tile_blocks(0, false), crb::tile_blocks(1, kMany), crb::tile_blocks(2, false)}};
 }
 // Tiles of 30 rows: the time of a call by height, 14 / 22 / 30 / 38 rows: 70 / 61 / 60 / 61 us on 800 x 800,
 // 299 / 238 / 213 / 219 us on 2048 x 2048 (fewer rows: more of them recomputed around the tile; 38: three
@@ -188,6 +193,7 @@ struct crb_ctx {
   int occ_q[kQKernels] = {};  // queue pipeline kernels (QK order)
   int occ_replace = 0;
   int occ_detect2 = 0;
+  int occ_tile = 0;  // row kernels of one round: the fewest blocks per SM of the first and later iterations
 
   void* ws = nullptr;
   size_t ws_bytes = 0;
@@ -295,11 +301,21 @@ int init_ctx(crb_ctx* c) {
     c->occ_fused.push_back(occf > 0 ? occf : 1);
   }
   for (const auto& t : kTileKernels)
-    for (int m = 0; m < 3; ++m) {  // the blocks per SM need the largest shared-memory carveout
-      CRB_CUDA(cudaFuncSetAttribute(t.fn[m], cudaFuncAttributeMaxDynamicSharedMemorySize, t.smem[m]));
-      CRB_CUDA(cudaFuncSetAttribute(t.fn[m], cudaFuncAttributePreferredSharedMemoryCarveout,
-                                    int(cudaSharedmemCarveoutMaxShared)));
-    }
+    for (int m = 0; m < 3; ++m)
+      for (TileFn fn : {t.fn[0][m], t.fn[1][m]}) {
+        if (&t == &kTileKernels[2] && m != 1) continue;  // those of the first
+        if (t.smem[m] > 48 * 1024)
+          CRB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, t.smem[m]));
+        // the blocks per SM need the largest shared-memory carveout
+        CRB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                      int(cudaSharedmemCarveoutMaxShared)));
+      }
+  for (int m = 0; m < 2; ++m) {
+    int occ = 0;
+    CRB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kTileKernels[0].fn[1][m], 256,
+                                                           size_t(kTileKernels[0].smem[m])));
+    c->occ_tile = m ? std::min(c->occ_tile, occ) : occ;
+  }
   {
     const void* fns[kQKernels] = {
         reinterpret_cast<const void*>(crb::bound_dense_kernel),      reinterpret_cast<const void*>(crb::need_kernel),
@@ -660,9 +676,9 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
     for (int k = 1; k <= P.niter + 1; ++k) {
       const int mode = k == 1 ? 0 : k <= P.niter ? 1 : 2;
       timed(c, mode == 2 ? kPTileReplace : kPTileDetect, stream, [&] {
-        // of one frame, iteration 1 takes the descriptor with its launch, and runs beside the upload
-        launch_pdl(t.fn[mode], unsigned(P.tiles), 256, t.smem[mode], stream, c->d_frames,
-                   k == 1 && P.n == 1 ? 0 : P.n, c->p, k, P.niter, c->h_frames[0]);
+        // of one frame, the launches carry the descriptor, and iteration 1 runs beside the upload
+        launch_pdl(t.fn[P.n == 1][mode], unsigned(P.tiles), 256, t.smem[mode], stream, c->d_frames, P.n, c->p, k,
+                   P.niter, c->num_sms * t.blocks[mode], c->h_frames[0]);
       });
     }
     CRB_CUDA(cudaGetLastError());
@@ -943,7 +959,7 @@ int prepare_tile(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pla
     high += tiles_of(s, kTileKernels[0].th);
     low += tiles_of(s, kTileKernels[1].th);
   }
-  const int v = low <= c->num_sms ? 1 : high > 4LL * c->num_sms ? 2 : 0;
+  const int v = low <= c->num_sms ? 1 : high > (long long)c->num_sms * c->occ_tile ? 2 : 0;
   const int th = kTileKernels[v].th;
   char* pb = static_cast<char*>(c->ws);
   char* pi = pb + bits;

@@ -321,8 +321,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, unsign
 // kernel to start (once every block has called it or ended). Both do nothing in
 // a kernel launched without the attribute. Every kernel of a chain waits before it
 // lets the next one start, so what an earlier kernel of the chain than the
-// previous one wrote is visible before the wait too. Without pdl_launch the next
-// one starts when all blocks have ended, ahead of the completion of their writes.
+// previous one wrote has reached memory before the wait too; but only the wait
+// orders this kernel's loads after it, and a line that an SM's L1 holds from an
+// earlier kernel may be old. Loads ahead of the wait therefore go past L1
+// (ld.global.cg, cp.async.cg). Without pdl_launch the next kernel starts when all
+// blocks have ended, ahead of the completion of their writes.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // Polls of a TMA wait before it gives up (each poll suspends the thread for a

@@ -124,16 +124,21 @@ struct TilePos {
 };
 
 // Bits of region row `gy` (clamped by the caller) of a flag plane, the columns
-// outside the frame taking the flag of the frame's edge column.
-__device__ __forceinline__ uint2 plane_row(const uint32_t* __restrict__ plane, int wps, int gy, const TilePos& T) {
+// outside the frame taking the flag of the frame's edge column. ahead: read before
+// the wait (pdl_wait), past L1.
+__device__ __forceinline__ uint2 plane_row(const uint32_t* __restrict__ plane, int wps, int gy, const TilePos& T,
+                                           bool ahead) {
   const int b = T.x0 / 2 - 4, wi = b >> 5, sh = b & 31;
-  uint32_t v[2];
+  uint32_t v[2], lo[2], hi[2];
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     const uint32_t* p = plane + (size_t(gy) * 2 + j) * wps;
-    const uint32_t lo = (wi >= 0 && wi < wps) ? p[wi] : 0u, hi = (wi + 1 < wps) ? p[wi + 1] : 0u;
-    v[j] = __funnelshift_r(lo, hi, sh);
+    auto word = [&](int i) { return i < 0 || i >= wps ? 0u : ahead ? __ldcg(p + i) : p[i]; };
+    lo[j] = word(wi);
+    hi[j] = word(wi + 1);
   }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) v[j] = __funnelshift_r(lo[j], hi[j], sh);
   uint2 m = make_uint2(v[0], v[1]);
   if (T.c0 > 0) {  // columns left of the frame
     const uint2 out = cols2(0, T.c0);
@@ -221,17 +226,40 @@ __device__ __forceinline__ bool test_holds(const Params& p, float fval, float nn
   return __fdiv_rn(num, fmaxf(__fdiv_rn(fval, nn), 0.01f)) > p.objlim;
 }
 
+// resident blocks per SM the kernels are compiled for
+constexpr int tile_blocks(int mode, bool many) { return mode == 1 && !many ? 4 : 4 + mode; }
+
+// The frame of tile t (frame_of) by a whole warp, read past L1: each step of the search looks at 32 frames at once
+// (a binary search's steps wait for memory one after another).
+__device__ __forceinline__ int frame_of_ahead(const Frame* frames, int nframes, long long t) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0;
+  for (int n = nframes, step; n > 1; n = min(step, nframes - lo)) {  // the frame is one of lo .. lo + n - 1
+    step = (n + 31) / 32;
+    const int i = lo + lane * step;
+    const bool at = lane * step < n && __ldcg(&frames[i].tile0) <= t;
+    lo += (__popc(__ballot_sync(0xffffffffu, at)) - 1) * step;
+  }
+  return lo;
+}
+
 // What a launch does before pdl_wait depends on nothing the launch ahead of it
-// writes: iteration 1 of a call of one frame (nframes 0: its descriptor `one`
-// comes with the launch) needs only the input until it writes its flags, so it
-// runs beside the upload; later launches load M_{k-2}, and iteration 2 the
-// input, while the launch ahead ends (letting the next launch start so early: 40.6
-// -> 38.9 us on 137 x 137, 54.0 -> 52.8 on 800 x 800).
+// writes: iteration 1 of a call of one frame (kSolo: the descriptor `one` comes
+// with the launch) needs only the input until it writes its flags, so it runs
+// beside the upload; later launches load M_{k-2}, iteration 2 the input, and those
+// of a batch the descriptor, while the launch ahead ends (letting the next launch
+// start so early: 40.6 -> 38.9 us on 137 x 137, 54.0 -> 52.8 on 800 x 800). These
+// loads go past L1 (pdl_wait's comment). Only the blocks of the first round of
+// resident ones (first_round of them) can start so early; the others wait first,
+// which costs them nothing, and load through L1, where the descriptor is (every
+// block ahead: 189 us on 2048 x 2048, and 191 on six frames of 801 x 799).
+// One frame's descriptor is read as launch parameters: 185 -> 174 us on 2048 x
+// 2048, 52.0 -> 51.0 on 800 x 800 against a copy in shared memory.
 // kMode 0: iteration 1. 1: the replacement of iteration k-1, then iteration k.
 // 2: the replacement of iteration niter (k = niter + 1) and the u8 mask.
-template <int TH, int kMode, bool kMany>
-__global__ void __launch_bounds__(256, kMode == 1 && !kMany ? 4 : 4 + kMode)
-    tile_kernel(const Frame* __restrict__ frames, int nframes, Params p, int k, int niter,
+template <int TH, int kMode, bool kMany, bool kSolo>
+__global__ void __launch_bounds__(256, tile_blocks(kMode, kMany))
+    tile_kernel(const Frame* __restrict__ frames, int nframes, Params p, int k, int niter, int first_round,
                 const __grid_constant__ Frame one) {
   using L = TileLayout<TH, kMode>;
   constexpr int R = L::R;
@@ -254,22 +282,26 @@ __global__ void __launch_bounds__(256, kMode == 1 && !kMany ? 4 : 4 + kMode)
   int* cnt = reinterpret_cast<int*>(smem + L::oCnt);  // 0 replacement, 1 S and S', 3 tests, 4 full windows, 5.. work
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-  // the bit maps and counters; then the frame's descriptor, which in the later iterations does not depend
-  // on the kernel before this one (pdl_wait)
+  // the bit maps and counters, and the frame's descriptor
   for (int i = tid; i < (kMode == 2 ? 0 : 6 * R); i += 256) mC[i] = make_uint2(0u, 0u);
   if (tid < 16) cnt[tid] = 0;
-  if (kMode == 0 && nframes) {
-    pdl_wait();
-    pdl_launch();
-  }
   __shared__ Frame sf;
-  {
-    const uint32_t* d = reinterpret_cast<const uint32_t*>(
-        (kMode == 0 && !nframes) ? &one : frames + frame_of<false>(frames, nframes, blockIdx.x));
-    for (int i = tid; i < int(sizeof(Frame) / 4); i += 256) reinterpret_cast<uint32_t*>(&sf)[i] = d[i];
+  const Frame& f = [&]() -> const Frame& {
+    if constexpr (kSolo) return one;
+    else return sf;
+  }();
+  const bool ahead = int(blockIdx.x) < first_round && (kMode != 0 || kSolo);
+  if (!ahead) {
+    pdl_wait();
+    if (kMode == 1 || (kMode == 0 && !kSolo)) pdl_launch();
   }
-  __syncthreads();
-  const Frame& f = sf;
+  if constexpr (!kSolo) {
+    const uint32_t* d = reinterpret_cast<const uint32_t*>(
+        frames + (ahead ? frame_of_ahead(frames, nframes, blockIdx.x) : frame_of<false>(frames, nframes, blockIdx.x)));
+    for (int i = tid; i < int(sizeof(Frame) / 4); i += 256)
+      reinterpret_cast<uint32_t*>(&sf)[i] = ahead ? __ldcg(d + i) : d[i];
+    __syncthreads();
+  }
   const int w = f.w, h = f.h, wps = f.wps;
   TilePos T;
   {
@@ -282,9 +314,12 @@ __global__ void __launch_bounds__(256, kMode == 1 && !kMany ? 4 : 4 + kMode)
     T.r1 = min(h - T.y0 + 8, R);
     T.edge = T.c0 > 2 || T.r0 > 2 || T.c1 < 62 || T.r1 < R - 2;
   }
+
   const float* src = kMode == 0 ? f.img : iter_src(f, k - 1, niter);
 
-  // the image region (mode 2: the tile and the 2 rows around it), clamped into the frame
+  // the image region (mode 2: the tile and the 2 rows around it), clamped into the frame; ahead of the wait past
+  // L1, single values too (a 4-byte cp.async exists through L1 only)
+  const bool early = ahead && (kMode == 0 || k == 2);
   auto load_image = [&] {
     constexpr int ra = kMode == 2 ? 6 : kMode == 0 ? 2 : 0, rb = R - ra;
     if ((w & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
@@ -296,16 +331,39 @@ __global__ void __launch_bounds__(256, kMode == 1 && !kMany ? 4 : 4 + kMode)
           cp_async16(d, row + gx);
         } else {
           const float* e = row + (gx < 0 ? 0 : w - 1);
+          if (early) {
+            const float v = __ldcg(e);
+            *reinterpret_cast<float4*>(d) = make_float4(v, v, v, v);
+          } else {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) cp_async4(d + q, e);
+            for (int q = 0; q < 4; ++q) cp_async4(d + q, e);
+          }
         }
       }
-    } else {
+    } else {  // a row per warp
       const int ca = clampi(T.x0 - 8 + lane, 0, w - 1), cb = clampi(T.x0 + 24 + lane, 0, w - 1);
-      for (int r = ra + warp; r < rb; r += 8) {  // a row per warp
-        const float* row = src + size_t(clampi(T.y0 - 8 + r, 0, h - 1)) * w;
-        cp_async4(sJ + r * kT2P + lane, row + ca);
-        cp_async4(sJ + r * kT2P + lane + 32, row + cb);
+      if (early) {
+        constexpr int kRows = (rb - ra + 7) / 8;
+        float va[kRows], vb[kRows];
+#pragma unroll
+        for (int j = 0; j < kRows; ++j) {
+          const float* row = src + size_t(clampi(T.y0 - 8 + min(ra + warp + 8 * j, rb - 1), 0, h - 1)) * w;
+          va[j] = __ldcg(row + ca);
+          vb[j] = __ldcg(row + cb);
+        }
+#pragma unroll
+        for (int j = 0; j < kRows; ++j) {
+          const int r = ra + warp + 8 * j;
+          if (r >= rb) continue;
+          sJ[r * kT2P + lane] = va[j];
+          sJ[r * kT2P + lane + 32] = vb[j];
+        }
+      } else {
+        for (int r = ra + warp; r < rb; r += 8) {
+          const float* row = src + size_t(clampi(T.y0 - 8 + r, 0, h - 1)) * w;
+          cp_async4(sJ + r * kT2P + lane, row + ca);
+          cp_async4(sJ + r * kT2P + lane + 32, row + cb);
+        }
       }
     }
     cp_async_commit();
@@ -318,11 +376,13 @@ __global__ void __launch_bounds__(256, kMode == 1 && !kMany ? 4 : 4 + kMode)
     static_assert(R <= 256, "a thread per row");
     const int gy = clampi(T.y0 - 8 + tid, 0, h - 1);
     uint2 before = make_uint2(0u, 0u);
-    if (tid < R) before = plane_row(f.mp[(kr + 2) % 3], wps, gy, T);
-    pdl_wait();
-    if (kMode == 1) pdl_launch();  // the last kernel's results are the caller's: nothing starts before they are whole
+    if (tid < R) before = plane_row(f.mp[(kr + 2) % 3], wps, gy, T, ahead);
+    if (ahead) {
+      pdl_wait();
+      if (kMode == 1) pdl_launch();  // the last kernel's results are the caller's: nothing starts before they are whole
+    }
     if (tid < R) {
-      const uint2 a = plane_row(f.mp[kr % 3], wps, gy, T);
+      const uint2 a = plane_row(f.mp[kr % 3], wps, gy, T, false);
       mM[tid] = a;
       mF[tid] = make_uint2(a.x & ~before.x, a.y & ~before.y);
     }
@@ -605,7 +665,7 @@ __global__ void __launch_bounds__(256, kMode == 1 && !kMany ? 4 : 4 + kMode)
       const int b = __ffs(v) - 1;
       L1[op++] = uint16_t((r << 7) | (b << 2) | ((mine.x >> b) & 1u) | ((mine.y >> b) & 1u) << 1);
     }
-    if (f.work) {
+    {
       const uint2 hm = make_uint2(half, half);
       const int n = __reduce_add_sync(0xffffffffu, unsigned(popc2(and2(need, hm))) | unsigned(popc2(and2(mine, hm))) << 16);
       if (lane == 0 && n) {
@@ -725,14 +785,14 @@ __global__ void __launch_bounds__(256, kMode == 1 && !kMany ? 4 : 4 + kMode)
                                                      : med3_at(sJ, clampi(r - 3 + i / 7, rl, rh), clampi(c - 3 + i % 7, cl, ch))),
                         nn, num);
       cand = m >= 25;
-      if (f.work) atomicAdd(&cnt[7], 1);
+      atomicAdd(&cnt[7], 1);
     }
     if (cand) set_bit2(&mG[r], c);
   }
   __syncthreads();
 
   // ---- both growths; M_k = M_{k-1} | g2
-  if (kMode == 0 && !nframes) {
+  if (kMode == 0 && kSolo) {
     pdl_wait();
     pdl_launch();
   }
@@ -755,7 +815,7 @@ __global__ void __launch_bounds__(256, kMode == 1 && !kMany ? 4 : 4 + kMode)
     fresh = __reduce_add_sync(0xffffffffu, unsigned(fresh));
     if (lane == 0 && fresh) atomicAdd(f.counters + 2 * (k - 1), (unsigned long long)fresh);
   }
-  if (tid == 255 && f.work) {
+  if (tid == 255) {
     unsigned long long* wk = f.work + kWork * (k - 1);
     auto span = [&](int m) {
       return (long long)(min(8 + kT2W + m, T.c1) - max(8 - m, T.c0)) * (min(8 + TH + m, T.r1) - max(8 - m, T.r0));

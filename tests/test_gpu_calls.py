@@ -16,7 +16,7 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
-from paper_1008_2192_gb300 import Cleaner, Server  # noqa: E402
+from paper_1008_2192_gb300 import Cleaner, Server, poisson_into  # noqa: E402
 
 
 # calls of one pixel count, tile count, number of words, cells and zeroed bytes: single frames that differ in their
@@ -154,3 +154,73 @@ def test_autotune_finds_the_tile_pipeline_above_10_mpix(graphs):
         c.sync()
         assert torch.equal(m, wm) and torch.equal(o, wo)
     assert c.tuned_config()[2] == "tile"
+
+
+CHAIN_SIZES = [(137, 137), (400, 300), (401, 299), (800, 800), (801, 799), (1200, 1000), (1201, 999)]
+
+
+@pytest.mark.parametrize("niter", [1, 2, 4])
+def test_chained_calls_without_a_wait(niter):
+    """One stream and one handle, nothing waited for in between: a clean of the output of the one before, POISSON
+    into the input of the next clean, and an input that a kernel overwrites between two calls, with the frame size, gain
+    and buffers changing from call to call. Each result equals that of calls waited for one by one."""
+    rng = np.random.default_rng(93)
+    calls = []
+    for w, h in CHAIN_SIZES:
+        a, b = (synth.frame(w, h, seed=94, index=i) for i in range(2))
+        mean = np.full((h, w), 24.3, np.float32)
+        calls.append(dict(a=dev(a), b=dev(b), mean=dev(mean), g=[float(np.float32(rng.uniform(2, 7))) for _ in range(3)]))
+
+    def go(c, wait):
+        outs = []
+        step = c.sync if wait else (lambda: None)
+        for rep in range(3):
+            for k in calls:
+                x = k.setdefault("x", torch.empty_like(k["a"]))
+                bufs = [torch.empty_like(x) for _ in range(5)]
+                masks = [torch.empty(x.shape, dtype=torch.uint8, device="cuda") for _ in range(5)]
+
+                def clean(src, i, g):
+                    c.clean_batch_into([src], [bufs[i]], [masks[i]], [g], [5.0])
+                    step()
+
+                x.copy_(k["a"])
+                clean(x, 0, k["g"][0])
+                x.copy_(k["b"])
+                clean(x, 1, k["g"][1])
+                clean(bufs[1], 2, k["g"][2])
+                poisson_into(k["mean"], x, 95 + rep)
+                step()
+                clean(x, 3, k["g"][0])
+                x.add_(k["a"])
+                clean(x, 4, k["g"][1])
+                outs += bufs + masks
+        c.sync()
+        return outs
+
+    want = go(Cleaner(niter=niter), True)
+    for _ in range(3):
+        got = go(Cleaner(niter=niter), False)
+        assert len(got) == len(want) and all(torch.equal(p, q) for p, q in zip(got, want))
+
+
+def test_chained_batches_without_a_wait():
+    """Batches of changing sizes and numbers of frames, the input of each being the output of the one before."""
+    sizes = [[(137, 137), (200, 100)], [(801, 799)], [(401, 299), (64, 64), (400, 300)], [(1201, 999), (97, 61)]]
+    frames = [[dev(synth.frame(w, h, seed=96, index=i)) for i, (w, h) in enumerate(s)] for s in sizes]
+
+    def go(c, wait):
+        outs = []
+        for f in frames * 3:
+            for _ in range(2):
+                f, masks = c.clean_batch(f, [6.5 - len(f)] * len(f), [4.0 + len(f)] * len(f))
+                if wait:
+                    c.sync()
+                outs += f + masks
+        c.sync()
+        return outs
+
+    want = go(Cleaner(niter=4), True)
+    for _ in range(3):
+        got = go(Cleaner(niter=4), False)
+        assert all(torch.equal(p, q) for p, q in zip(got, want))
