@@ -181,23 +181,18 @@ __device__ __forceinline__ void load_pair_smem(const float* a, int r, int c0, fl
     }
 }
 
-// The value of rank 12 of a clamped 5x5 window, by counting: for the rare exact
-// path only, so that the network is not instantiated once more.
+// The 5x5 median at (r, c), c0 = c & ~1 the pair's column, the window clamped to rows [rlo, rhi] and columns [clo,
+// chi]: the network of the S and S' stages, for the rare exact path only.
 __device__ __noinline__ float median25_at(const float* a, int r, int c, int rlo, int rhi, int clo, int chi) {
-  auto at = [&](int q) {
-    return a[clampi(r - 2 + q / 5, rlo, rhi) * kT2P + clampi(c - 2 + q % 5, clo, chi)];
-  };
-  for (int i = 0; i < 25; ++i) {
-    const float x = at(i);
-    int less = 0, le = 0;
-    for (int j = 0; j < 25; ++j) {
-      const float y = at(j);
-      less += y < x;
-      le += y <= x;
-    }
-    if (less <= 12 && 12 < le) return x;
-  }
-  return a[r * kT2P + c];
+  const int c0 = c & ~1;
+  float v[5][6], m[2];
+#pragma unroll
+  for (int dy = 0; dy < 5; ++dy)
+#pragma unroll
+    for (int dx = 0; dx < 6; ++dx)
+      v[dy][dx] = a[clampi(r - 2 + dy, rlo, rhi) * kT2P + clampi(c0 - 2 + dx, clo, chi)];
+  med25_row2(v, m);
+  return (c & 1) ? m[1] : m[0];
 }
 
 // med3 at (r, c) of the image region.
@@ -213,17 +208,39 @@ __device__ __noinline__ float med3_at(const float* a, int r, int c) {
 // window in the place of the median exactly where S'/max(F/N, 0.01) > objlim
 // with F = m3 - v (article form: 2S for S'), that is where F < X up to
 // rounding, X = N * num / objlim. The four roundings stay within 2^-22, so F
-// outside X (1 -+ 2e-6) decides; num/objlim near 0.01 or below, or an X out of the
-// normal range, is marked -1 (decided step by step), and num/objlim < 0.0099
-// can never pass (0: F/N is floored at 0.01).
+// outside X (1 -+ 2e-6) decides; num/objlim near 0.01 or below, or an X or objlim
+// out of the normal range, is marked -1 (decided step by step), and num/objlim <
+// 0.0099 can never pass (0: F/N is floored at 0.01).
 __device__ __forceinline__ float test_scale(float num, float nn, float objlim) {
   const float q = __fdiv_rn(num, objlim), x = __fmul_rn(q, nn);
   if (q < 0.0099f) return 0.f;
-  return (q > 0.0101f && x > 1e-30f && x < 1e30f) ? x : -1.f;
+  return (q > 0.0101f && x > 1e-30f && x < 1e38f && objlim > 1e-30f) ? x : -1.f;
 }
 
 __device__ __forceinline__ bool test_holds(const Params& p, float fval, float nn, float num) {
   return __fdiv_rn(num, fmaxf(__fdiv_rn(fval, nn), 0.01f)) > p.objlim;
+}
+
+// The objlim test at row rc >> 6, column rc & 63 by the stated steps for each value of the window, by a whole warp: N and S' by the
+// networks again, then a value per lane (800 x 800 with objlim 500: one lane per test 105 us, this 54; 137 x 137 with
+// values up to 1e38: 327, this 78). m3: med3 of the region, or nullptr where it is formed from J.
+__device__ __noinline__ bool test_exact(const float* J, const float* S, const float* m3, int rc, int rlo, int rhi, int clo,
+                                        int chi, float gain, float rn2, Params p) {
+  const int lane = threadIdx.x & 31, r = rc >> 6, c = rc & 63;
+  const float mc = m3 ? m3[r * kT2P + c] : med3_at(J, r, c);
+  const float nn = noise_of(floor_m5(median25_at(J, r, c, 0, r + 2, 0, 63)), gain, rn2);
+  const float s = S[r * kT2P + c];
+  const float num = p.objlim_form == 1 ? __fmul_rn(2.f, s) : __fsub_rn(s, median25_at(S, r, c, rlo, rhi, clo, chi));
+  int m = 0;
+  for (int i = lane; i < 64; i += 32) {
+    bool holds = false;
+    if (i < 49) {
+      const int y = clampi(r - 3 + i / 7, rlo, rhi), x = clampi(c - 3 + i % 7, clo, chi);
+      holds = test_holds(p, __fsub_rn(mc, m3 ? m3[y * kT2P + x] : med3_at(J, y, x)), nn, num);
+    }
+    m += __popc(__ballot_sync(0xffffffffu, holds));
+  }
+  return m >= 25;
 }
 
 // resident blocks per SM the kernels are compiled for
@@ -766,27 +783,22 @@ __global__ void __launch_bounds__(256, tile_blocks(kMode, kMany))
 #pragma unroll
       for (int d = 0; d < 7; ++d) {
         const float fv = __fsub_rn(mc, v[d]);
-        n += (fv < xl ? 1 : 0) + (fv <= xh ? 65536 : 0);
+        n += (fv >= xl ? 0 : 1) + (fv > xh ? 0 : 65536);  // infinity less itself passes, as F/N floored at 0.01 does
       }
     }
     n += __shfl_xor_sync(0xffffffffu, n, 1);
     n += __shfl_xor_sync(0xffffffffu, n, 2);
     n += __shfl_xor_sync(0xffffffffu, n, 4);
-    if (!on || q != 0) continue;
     bool cand = (n & 0xffff) >= 25;
-    if (x < 0.f || (!cand && (n >> 16) >= 25)) {  // the count cannot decide: every value by the stated steps
-      const int rl = T.r0, rh = T.r1 - 1, cl = T.c0, ch = T.c1 - 1;
-      const float nn = noise_of(floor_m5(median25_at(sJ, r, c, 0, R - 1, 0, 63)), gain, rn2);
-      const float s = sS[r * kT2P + c];
-      const float num = p.objlim_form == 1 ? __fmul_rn(2.f, s) : __fsub_rn(s, median25_at(sS, r, c, rl, rh, cl, ch));
-      int m = 0;
-      for (int i = 0; i < 49; ++i)
-        m += test_holds(p, __fsub_rn(mc, kMode == 0 ? sM3[(r - 3 + i / 7) * kT2P + c - 3 + i % 7]
-                                                     : med3_at(sJ, clampi(r - 3 + i / 7, rl, rh), clampi(c - 3 + i % 7, cl, ch))),
-                        nn, num);
-      cand = m >= 25;
-      atomicAdd(&cnt[7], 1);
+    const bool open = on && q == 0 && (x < 0.f || (!cand && (n >> 16) >= 25));  // the count cannot decide
+    for (unsigned m = __ballot_sync(0xffffffffu, open); m; m &= m - 1u) {
+      const int l = __ffs(m) - 1;
+      const bool holds = test_exact(sJ, sS, kMode == 0 ? sM3 : nullptr, L0[t0 + (l >> 3)], T.r0, T.r1 - 1, T.c0,
+                                    T.c1 - 1, gain, rn2, p);
+      if (lane == l) cand = holds;
     }
+    if (!on || q != 0) continue;
+    if (open) atomicAdd(&cnt[7], 1);
     if (cand) set_bit2(&mG[r], c);
   }
   __syncthreads();

@@ -224,3 +224,25 @@ def test_chained_batches_without_a_wait():
     for _ in range(3):
         got = go(Cleaner(niter=4), False)
         assert all(torch.equal(p, q) for p, q in zip(got, want))
+
+
+@pytest.mark.parametrize("w,h", [(137, 90), (150, 331), (1153, 781)])
+@pytest.mark.parametrize("kw", [dict(objlim=1e-29), dict(objlim=1e-35), dict(objlim=450.0), dict(objlim=450.0, objlim_form=1),
+                                dict(sigclip=1e-3, objlim=1e-38), dict(amp=1e33), dict(amp=1e36), dict(amp=1e38)],
+                         ids=lambda k: "-".join(f"{a}{b:g}" for a, b in k.items()))
+def test_objlim_beyond_counting(w, h, kw):
+    """The row kernels' objlim test where a count of the window decides at scales near float's range, and where it
+    cannot decide and the steps are taken value by value (S'/objlim near 0.01; scales out of range): masks, images and
+    counters equal the FP32 oracle's, on tiles of 14 and 30 rows, in one round and in more."""
+    kw = dict(kw)
+    img = synth.frame(w, h, seed=97, ncr=max(1, int(3 * w * h * synth.CR_DENSITY)))
+    amp = kw.pop("amp", None)
+    if amp:
+        rng = np.random.default_rng(98)
+        hit = rng.random(img.shape) < 0.01
+        img[hit] = (rng.uniform(-1.0, 1.0, int(hit.sum())) * amp).astype(np.float32)
+    c = Cleaner(niter=3, pipeline="tile", **kw)
+    out, mask = gpu_clean(c, img)
+    r32 = oracle.clean(img, params_of(kw), 3, precision="f32")
+    assert np.array_equal(mask, r32.mask) and np.array_equal(out, r32.clean)
+    assert c.last_counts() == list(zip(r32.n_new, r32.n_none_left))
