@@ -180,7 +180,9 @@ __global__ void __launch_bounds__(kPThreads) poisson_kernel(const __grid_constan
       for (;;) {
         const bool last = e <= 90;
         thr = last ? mhi * __int_as_float((127 - e) << 23) : 0x1p-64f;
-        if (q < thr) {  // two tiny factors in a row after a scaling
+        // two tiny factors in a row: the product below the threshold already, or before its scaling below 2^-126,
+        // where float loses bits that the error bound does not count
+        if (q < fmaxf(thr, 0x1p-62f)) {
           exact = true;
           break;
         }

@@ -86,3 +86,16 @@ def test_invalid_arguments():
     assert lib.crb_poisson(p, 4, -1, 0, p, None) == L.CRB_EINVAL
     assert lib.crb_poisson_batch(-1, None, None, None, None, None, None) == L.CRB_EINVAL
     assert lib.crb_poisson_batch(0, None, None, None, None, None, None) == L.CRB_OK
+
+
+@pytest.mark.parametrize("mean", [120.0, 250.0, 690.0])
+def test_products_below_the_normal_range(mean):
+    """Seeds (found by inverting the generator) whose first pixel draws two factors with a product near 2^-63 one after
+    the other, so that the running product, before it is scaled up, falls below float's normal range: after 0 to 4
+    scalings. Such pixels are taken again in double."""
+    seeds = [9796533934964748776, 1142700078899050769, 8589809309024554849, 13703604691797313703, 5762708181886060360,
+             1741285944254986629, 3449822246592346243, 4048324880749360500, 15912223027965287662, 3183809587945724739,
+             13688508111628718151, 12934896684533608378]
+    img = np.full((3, 2), mean, np.float32)
+    for seed in seeds:
+        assert np.array_equal(gpu_poisson(img, seed), oracle.poisson(img, seed)), seed
