@@ -85,19 +85,34 @@ __device__ __forceinline__ double exp_neg(double mu, const PLaunch& P) {
 }
 
 // The deviate of pixel p by the defining steps in double: every product and
-// comparison as stated in the header.
+// comparison as stated in the header. After the first draw eight at a time, their
+// uniforms ahead of the chain of products, which fall monotonically: a product
+// above e^-mu has none below it before. One pixel's chain holds up a small image's call
+// (64 x 64 of mean 690, 3 such pixels: 121 us with one draw at a time, so 97).
 __device__ __noinline__ int deviate_exact(float mean, uint64_t key, const PLaunch& P) {
   // q and e^-mu are non-negative doubles, which order as their bit patterns
   const long long L = __double_as_longlong(exp_neg(fmin(double(mean), kMuMax), P));
-  uint64_t ctr = key + kGamma;  // key + (j + 1) * gamma for draw j
-  double q = uniform53(mix13(ctr));
-  int k = 0;
-  while (__double_as_longlong(q) >= L && k < kQMax) {
-    ++k;
-    ctr += kGamma;
-    q = __dmul_rn(q, uniform53(mix13(ctr)));
+  auto draw = [&](int j) { return uniform53(mix13(key + uint64_t(j + 1) * kGamma)); };
+  double q = draw(0);
+  if (__double_as_longlong(q) < L) return 0;
+  for (int k = 1; k < kQMax; k += 8) {
+    double u[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) u[i] = draw(k + i);
+    double q8 = q;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) q8 = __dmul_rn(q8, u[i]);
+    if (__double_as_longlong(q8) >= L) {
+      q = q8;
+      continue;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      q = __dmul_rn(q, u[i]);
+      if (__double_as_longlong(q) < L) return min(k + i, kQMax);
+    }
   }
-  return k;
+  return kQMax;
 }
 
 // hi * 2^-32 in float, rounded once: the top 23 bits and the low 9 as

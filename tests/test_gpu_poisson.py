@@ -99,3 +99,11 @@ def test_products_below_the_normal_range(mean):
     img = np.full((3, 2), mean, np.float32)
     for seed in seeds:
         assert np.array_equal(gpu_poisson(img, seed), oracle.poisson(img, seed)), seed
+
+
+@pytest.mark.parametrize("mean", [33.0, 250.0, 690.0, 1e6])
+def test_pixels_drawn_again(mean):
+    """Chains in double of every length: means with enough pixels that several dozen products land within the float
+    bound of e^-mu, and are drawn again eight at a time."""
+    img = np.full((300, 301), mean, np.float32)
+    assert np.array_equal(gpu_poisson(img, 47), oracle.poisson(img, 47))
