@@ -333,9 +333,11 @@ int crb_selftest_wait_timeout(crb_ctx* ctx, unsigned polls, cudaStream_t stream)
  * replacement write, changed-pixel dilation, full candidate test, growth,
  * flag queue and u8 mask, segment list, segment-form dilation, need and
  * list of tests, list of tests of iteration 1, growth of iteration 1 (up to
- * max of them); the first iteration of
- * the segment-list forms; the pipeline (1 tile, 2 queue). Returns the number of
- * kernels written, or CRB_EINVAL. A measurement aid, not a step of the method
+ * max of them); the growth of iteration 1 and, below 2^26 pixels, the row forms
+ * of the dilation, need and list kernels have grids that follow no occupancy and
+ * are not tuned: for these the most blocks per SM of that grid. Then the first
+ * iteration of the segment-list forms and the pipeline (1 tile, 2 queue).
+ * Returns the number of kernels written, or CRB_EINVAL. A measurement aid, not a step of the method
  * (the paper has no counterpart). */
 int crb_tuned_config(const crb_ctx* ctx, int* blocks_per_sm, int max, int* seg_from, int* pipeline);
 

@@ -328,8 +328,9 @@ int init_ctx(crb_ctx* c) {
         reinterpret_cast<const void*>(crb::mask_kernel),        reinterpret_cast<const void*>(crb::seg_list_kernel),
         reinterpret_cast<const void*>(crb::d2_seg_kernel),      reinterpret_cast<const void*>(crb::need_seg_kernel),
         reinterpret_cast<const void*>(crb::tests_seg_kernel),   reinterpret_cast<const void*>(crb::tests_kernel<true>),
-        reinterpret_cast<const void*>(crb::grow_first_kernel)};
+        nullptr};  // kQGrowFirst: a row form
     for (int i = 0; i < kQKernels; ++i) {
+      if (!fns[i]) continue;
       int o = 0;
       const bool col = i == kQNeed || i == kQTests || i == kQD2 || i == kQD2Seg || i == kQNeedSeg ||
                        i == kQTestsSeg || i == kQTestsAll;
@@ -479,9 +480,21 @@ struct Plan {
   char* chg[2] = {nullptr, nullptr};         // changed-pixel planes (all frames) for even / odd iterations
   size_t chg_bytes = 0;
   crb::Queues Q{};
-  int occ[kQKernels] = {};       // queue pipeline: blocks per SM of each kernel (QK order)
+  int occ[kQKernels] = {};       // queue pipeline: blocks per SM of each kernel (QK order), by set_occ
   int seg_from = crb::kSegFrom;  // queue pipeline: first iteration of the segment-list forms
 };
+
+// Blocks per SM, at most, of the row forms' grids: a strip per block, or a walk over the listed segments.
+constexpr int kRowBlocks = 64, kSegRowBlocks = 8;
+
+// The blocks per SM of a queue plan's kernels: occ[], and the row forms' own where a row form is launched.
+void set_occ(Plan& P, const int* occ) {
+  std::copy(occ, occ + kQKernels, P.occ);
+  P.occ[kQGrowFirst] = kRowBlocks;
+  if (!P.row_form) return;
+  for (int i : {kQNeed, kQTests, kQTestsAll, kQTestsSeg, kQD2}) P.occ[i] = kRowBlocks;
+  for (int i : {kQNeedSeg, kQD2Seg}) P.occ[i] = kSegRowBlocks;
+}
 
 // Launches fn so that it may start before the kernel ahead of it in the stream
 // has ended (it waits for it in crb::pdl_wait).
@@ -560,7 +573,7 @@ int enqueue_work(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
       const int gcolm = grid(kQTests, ucol), gcol1m = grid(kQTestsAll, ucol);
       const bool seg = k >= P.seg_from;  // the column kernels walk the listed segments only
       const int tcol = crb::kColWarps * 32;
-      const long long grow = std::min<long long>(P.nunits, 64LL * c->num_sms), gseg = 8LL * c->num_sms;  // row forms
+      const long long grow = grid(kQGrowFirst, P.nunits), gseg = gq * kSegRowBlocks;  // row forms
       timed(c, kPBound, stream, [&] {
         if (k == 1) {
           tq(kQBound, [&] {
@@ -864,7 +877,7 @@ int prepare_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, Pl
   P.bits_total = zero_bytes;
   P.ncounters = ncounters;
   P.rgrid = int(std::min<long long>(rtiles, (long long)c->num_sms * c->occ_replace));
-  std::copy(c->occ_q, c->occ_q + kQKernels, P.occ);
+  set_occ(P, c->occ_q);
   P.seg_from = crb::kSegFrom;
   P.nblocks = nblocks;
   P.npix = npix;
@@ -1272,7 +1285,7 @@ int trial_queue(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, cons
   Plan P;
   int rc = prepare_queue(c, specs, niter, P);
   if (rc) return rc;
-  std::copy(occ, occ + kQKernels, P.occ);
+  set_occ(P, occ);
   P.seg_from = seg_from;
   P.pdl = true;  // a graph's replay takes what launches ahead of time take, not plain ones (4096^2: 509, 506, 639 us)
   c->tuning = per_kernel != nullptr;
@@ -1469,7 +1482,7 @@ int run(crb_ctx* c, const std::vector<FrameSpec>& specs, int niter, bool maps, c
     rc = queue ? prepare_queue(c, specs, niter, P) : prepare_choice(c, specs, niter, maps, choice, P);
   if (rc) return rc;
   if (queue && tuned) {
-    std::copy(tuned->occ, tuned->occ + kQKernels, P.occ);
+    set_occ(P, tuned->occ);
     P.seg_from = tuned->seg_from;
   }
   std::copy(P.occ, P.occ + kQKernels, c->last_occ);

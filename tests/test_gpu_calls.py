@@ -246,3 +246,17 @@ def test_objlim_beyond_counting(w, h, kw):
     r32 = oracle.clean(img, params_of(kw), 3, precision="f32")
     assert np.array_equal(mask, r32.mask) and np.array_equal(out, r32.clean)
     assert c.last_counts() == list(zip(r32.n_new, r32.n_none_left))
+
+
+def test_tuning_leaves_fixed_grids():
+    """Kernels whose grid follows no occupancy are reported with that grid's blocks per SM, tuned or not: the row forms
+    below 2^26 pixels, and the growth of iteration 1."""
+    img = synth.frame(900, 700, seed=99)
+    plain, tuned = (Cleaner(niter=4, pipeline="queue", autotune=t) for t in (False, True))
+    (o, m), (o2, m2) = gpu_clean(plain, img), gpu_clean(tuned, img)
+    assert np.array_equal(m, m2) and np.array_equal(o, o2)
+    a, b = plain.tuned_config()[0], tuned.tuned_config()[0]
+    names = list(a)
+    rows = [names[i] for i in (1, 4, 11, 18, 19, 20)]  # need, tests (three forms), d2, grow_first
+    segs = [names[i] for i in (16, 17)]
+    assert all(a[k] == b[k] == 64 for k in rows) and all(a[k] == b[k] == 8 for k in segs), (a, b)
