@@ -204,10 +204,10 @@ class Cleaner:
             raise RuntimeError("crb_last_work failed")
         return [tuple(int(buf[6 * i + j]) for j in range(6)) for i in range(k)]
 
-    # m3need*: the list of tests; m3: clearing the next iteration's cells (med3 goes with bound and bound_sparse)
-    QUEUE_KERNELS = ("bound", "need", "s", "sprime", "m3need", "m3", "cand_test", "rep_compute", "bound_sparse",
+    # tests*: the list of tests; clear: the next iteration's cells (med3 goes with bound and bound_sparse)
+    QUEUE_KERNELS = ("bound", "need", "s", "sprime", "tests", "clear", "cand_test", "rep_compute", "bound_sparse",
                      "rq", "rep_write", "d2", "cand_full", "grow", "mask", "seg_list", "d2_seg", "need_seg",
-                     "m3need_seg", "m3need_first", "grow_first")
+                     "tests_seg", "tests_first", "grow_first")
 
     def tuned_config(self):
         """Launch configuration of the last call: ({kernel: blocks per SM}, first segment-list iteration,
@@ -232,7 +232,7 @@ class Cleaner:
                                            ctypes.byref(rn), int(reset)), "crb_profile_read")
         return dm.value, dn.value, rm.value, rn.value
 
-    PROFILE_KINDS = ("bound", "need", "s", "sprime", "m3need", "m3", "cand", "grow", "reserved", "tile_detect",
+    PROFILE_KINDS = ("bound", "need", "s", "sprime", "tests", "clear", "cand", "grow", "reserved", "tile_detect",
                      "replace", "mask", "tile_replace", "work")
 
     def profile_kernels(self, reset=True):
