@@ -78,21 +78,19 @@ enum : int {
   kNSpx = 1,
   kNSP = 2,     // QSP
   kNSPpx = 3,
-  kNFree = 4,   // (not used)
-  kNFree2 = 5,
-  kNT = 6,      // QT
-  kNTpx = 7,
-  kNB = 8,      // pixels to re-test in the bound pass
-  kNBpx = 9,
-  kNRep = 10,   // replacement queue (pixels; its second counter is not used)
-  kNRep2 = 11,
-  kNPass = 12,  // candidates (passed the objlim test)
-  kNAmb = 13,   // tests the column-median bounds leave open
-  kNFresh = 14, // new flags of this iteration
-  kNFb = 15,    // pixels with a fully flagged window (kept over the iterations)
-  kNSegN = 16,  // segments (1 word x kSH rows) listed for need_seg_kernel and tests_seg_kernel,
-  kNSegD = 17,  // for d2_seg_kernel (the two in Queues::seg order)
-  kNCount = 18
+  kNT = 4,      // QT
+  kNTpx = 5,
+  kNB = 6,      // pixels to re-test in the bound pass
+  kNBpx = 7,
+  kNRep = 8,   // replacement queue (pixels; its second counter is not used)
+  kNRep2 = 9,
+  kNPass = 10,  // candidates (passed the objlim test)
+  kNAmb = 11,   // tests the column-median bounds leave open
+  kNFresh = 12, // new flags of this iteration
+  kNFb = 13,    // pixels with a fully flagged window (kept over the iterations)
+  kNSegN = 14,  // segments (1 word x kSH rows) listed for need_seg_kernel and tests_seg_kernel,
+  kNSegD = 15,  // for d2_seg_kernel (the two in Queues::seg order)
+  kNCount = 16
 };
 
 // QS, QSP and QT hold word entries: (global word index, mask of the
