@@ -262,3 +262,24 @@ def test_tuning_leaves_fixed_grids():
     rows = [names[i] for i in (1, 4, 11, 18, 19, 20)]  # need, tests (three forms), d2, grow_first
     segs = [names[i] for i in (16, 17)]
     assert all(a[k] == b[k] == 64 for k in rows) and all(a[k] == b[k] == 8 for k in segs), (a, b)
+
+
+def test_chained_calls_on_two_streams():
+    """One handle, calls alternating between two streams with no wait on the host: each call's upload and kernels, launched
+    ahead of time, start after the call before on the other stream, whose workspace and descriptors they take over."""
+    sizes = [(137, 137), (801, 799), (401, 299), (1201, 999)]
+    imgs = [dev(synth.frame(w, h, seed=100, index=i)) for i, (w, h) in enumerate(sizes)]
+    c = Cleaner(niter=4)
+    want = []
+    for x in imgs:
+        want.append(c.clean(x))
+        c.sync()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    outs = [(torch.empty_like(imgs[i % 4]), torch.empty(imgs[i % 4].shape, dtype=torch.uint8, device="cuda")) for i in range(60)]
+    torch.cuda.synchronize()
+    for i, (o, m) in enumerate(outs):
+        c.clean_into(imgs[i % 4], o, m, stream=streams[(i // 3 + i) % 2])
+    torch.cuda.synchronize()
+    for i, (o, m) in enumerate(outs):
+        assert torch.equal(m, want[i % 4][1]) and torch.equal(o, want[i % 4][0]), i
