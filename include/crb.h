@@ -23,8 +23,9 @@
  * Conventions for every call:
  *   - Images are float32 DN, row-major, contiguous (row pitch = w), DEVICE
  *     pointers. Masks are uint8 (0/1), same layout. The caller owns all buffers.
- *   - Sizes: 1 <= w, h; w*h < 2^31. Input must be finite (a NaN gives undefined
- *     output, never a fault).
+ *   - Sizes: 1 <= w, h; w*h < 2^31. Input must be finite, and so must the
+ *     differences of neighbouring pixels (else, and with a NaN, the output is
+ *     undefined there, never a fault).
  *   - Calls are asynchronous on `stream`: they validate, enqueue and return.
  *     Validation errors are returned synchronously. Device-side errors are
  *     latched in the context and reported by crb_sync_status().
@@ -80,8 +81,8 @@ typedef struct {
    * with the same signature. */
   int tile_shape;
   /* 1: capture the work of a call (the niter loop of launches, with the memsets
-   * of calls that have them) in a CUDA graph once per launch signature and
-   * replay it afterwards; the per-frame descriptors are uploaded before each
+   * of calls that have them) in a CUDA graph once per signature (frame sizes
+   * and niter) and replay it afterwards; the per-frame descriptors are uploaded before each
    * replay. The row kernels' few launches are made directly, which is faster.
    * Ignored while profiling. */
   int use_graphs;
@@ -101,7 +102,7 @@ typedef struct {
    * crb_iterate's map export and by crb_clean_noalloc). 0 (default): per
    * call, the queue pipeline from 6,000,000 pixels on (all frames of the call
    * together), the tile pipeline below: the queue pipeline's ~60 dependent
-   * launches cost about 0.16 ms per call, the tile pipeline about 2.7
+   * launches cost about 0.16 ms per call, the tile pipeline about 2.5
    * times more per pixel. All give identical results. */
   int pipeline;
   /* 1: autotune the queue pipeline. The first call with a new signature (the

@@ -101,9 +101,9 @@ constexpr TileKernels make_tile() {
 // Tiles of 30 rows: the time of a call by height, 14 / 22 / 30 / 38 rows: 70 / 61 / 60 / 61 us on 800 x 800,
 // 299 / 238 / 213 / 219 us on 2048 x 2048 (fewer rows: more of them recomputed around the tile; 38: three
 // blocks per SM). Tiles of 14 rows where they number at most one per SM: a block's latency is all there is,
-// and fewer rows per warp shorten it (137 x 137: 41 / 43 / 47 / 50 us).
-// More tiles than one round of four blocks per SM: iterations 2 on at five blocks (1024 x 1024: 73.1 -> 67.1 us,
-// 2048 x 2048: 199 -> 187; 800 x 800, one round: 52.7 -> 53.6).
+// and fewer rows per warp shorten it (137 x 137: 41 / 43 / 47 / 50 us; both rows of figures of the first builds).
+// More tiles than one round of four blocks per SM (as the runtime reports them): iterations 2 on at five blocks
+// (1024 x 1024: 73.1 -> 67.1 us, 2048 x 2048: 199 -> 187; 800 x 800, one round: 52.7 -> 53.6).
 const TileKernels kTileKernels[] = {make_tile<30, false>(), make_tile<14, false>(), make_tile<30, true>()};
 
 constexpr int kRW = 64, kRH = 16;  // replacement tile
@@ -1243,9 +1243,9 @@ int launch_graph(crb_ctx* c, const Plan& P, const std::vector<FrameSpec>& specs,
 // crb_options.pipeline
 enum { kPipeAuto = 0, kPipeTile = 1, kPipeQueue = 2 };
 // Automatic choice: the queue pipeline from this many pixels per call on. Its ~60 dependent launches cost about
-// 0.16 ms per call whatever the size, while the tile pipeline's 5 cost little but each pixel about 2.7 times
+// 0.16 ms per call whatever the size, while the tile pipeline's 5 cost little but each pixel about 2.5 times
 // more. The line is part of the interface; on single frames the two now meet higher (us, tiles / queues:
-// 2048^2 185 / 297, 2048 x 4096 351 / 378, 3300^2 447 / 422, 4096^2 694 / 502), and autotune takes the faster
+// 2048^2 174 / 292, 2048 x 4096 323 / 367, 3300^2 419 / 412, 4096^2 639 / 504), and autotune takes the faster
 // one below kTuneTilePixels.
 constexpr long long kAutoQueuePixels = 6000000;
 
